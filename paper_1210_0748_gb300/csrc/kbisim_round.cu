@@ -1331,11 +1331,18 @@ __global__ void __launch_bounds__(kVerNodeThreads) k_group_verify(GroupArgs g, V
       }
 #pragma unroll
       for (int t = 0; t < kVerItems; ++t) {
-        if (act[t] && eq[t] && U[t] > kShortSig) {  // long signature: compared by a CTA later
-          const unsigned long long q = atomicAdd(v.n_long, 1ull);
-          v.long_list[2 * q] = p[t];
-          v.long_list[2 * q + 1] = r[t];
-          act[t] = false;
+        // long signatures: compared by a CTA later (a warp takes its places in the list together)
+        const bool lng = act[t] && eq[t] && U[t] > kShortSig;
+        const unsigned lm = __ballot_sync(kFull, lng);
+        if (lm) {
+          unsigned long long q = 0;
+          if ((threadIdx.x & 31) == 0) q = atomicAdd(v.n_long, (unsigned long long)__popc(lm));
+          q = __shfl_sync(kFull, q, 0) + __popc(lm & lanes_below(threadIdx.x & 31));
+          if (lng) {
+            v.long_list[2 * q] = p[t];
+            v.long_list[2 * q + 1] = r[t];
+            act[t] = false;
+          }
         }
       }
 #pragma unroll
@@ -1420,17 +1427,86 @@ struct RankArgs {
   const uint32_t* rep;
   const uint32_t* p2o;
   const uint32_t* ucnt;    // may be null (level 0)
-  uint32_t* hbits;         // [words] head bitmap, original order
-  uint64_t* hword;         // [words] head count per word, then heads before the word
+  const uint2* hrank;      // [words] head bitmap word and the heads before it in its tile
+  const uint32_t* tbase;   // [tiles] heads before each tile of kRankTile words
   uint8_t* member;         // [n] internal order: the head has other members
   uint8_t* alone;          // [n] internal order: output, node alone in its block
   uint32_t* pid;           // output level, internal order
-  unsigned long long* stats;  // [2] key total, [3] max signature, [8] nodes alone in their block
+  const uint32_t* err;     // error flags, copied to stats[7]
+  unsigned long long* stats;  // [2] key total, [3] max signature, [7] error flags, [8] nodes alone in their block
 };
 
-__global__ void k_word_counts(const uint32_t* hbits, uint64_t words, uint64_t* hword) {
-  for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w < words; w += (uint64_t)gridDim.x * blockDim.x)
-    hword[w] = __popc(hbits[w]);
+// Heads before every bitmap word, in one pass: a CTA takes a tile of kRankTile
+// words and writes each word beside the heads before it in the tile; the CTA
+// that finishes last (a ticket, so nothing waits) turns the tile totals into
+// heads before each tile and the level's block count.  Word and rank sit in
+// one 8-byte entry, so k_pid_fill fetches both with one random access.  One
+// launch instead of a word count, two tile passes and a scan of the tiles:
+// bound by launch latency (31K words at 1M nodes; 9.5 us for the four before).
+constexpr int kRankThreads = 256, kRankItems = 4, kRankTile = kRankThreads * kRankItems;
+constexpr int kRankTileShift = 10 + 5;  // original ids of a tile: 2^15
+static_assert(kRankTile * 32 == 1 << kRankTileShift, "tile of original ids");
+
+// Exclusive sum of v over the CTA; *total gets the CTA's sum.  red: NT / 32 words.
+template <int NT>
+__device__ __forceinline__ uint32_t cta_exclusive_sum(uint32_t v, uint32_t* red, uint32_t* total) {
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  uint32_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(kFull, x, o);
+    if (lane >= (uint32_t)o) x += y;
+  }
+  if (lane == 31) red[w] = x;
+  __syncthreads();
+  uint32_t before = 0, all = 0;
+#pragma unroll
+  for (uint32_t i = 0; i < NT / 32; ++i) {
+    const uint32_t r = red[i];
+    before += i < w ? r : 0u;
+    all += r;
+  }
+  __syncthreads();
+  *total = all;
+  return before + x - v;
+}
+
+__global__ void __launch_bounds__(kRankThreads) k_head_ranks(const uint32_t* hbits, uint64_t words, uint2* hrank,
+                                                             uint32_t* tbase, unsigned long long* ticket,
+                                                             unsigned long long* total) {
+  __shared__ uint32_t red[kRankThreads / 32];
+  __shared__ uint32_t last;
+  const uint64_t w0 = (uint64_t)blockIdx.x * kRankTile + (uint64_t)threadIdx.x * kRankItems;
+  uint32_t b[kRankItems], c = 0;
+#pragma unroll
+  for (int t = 0; t < kRankItems; ++t) {
+    b[t] = w0 + t < words ? hbits[w0 + t] : 0u;
+    c += __popc(b[t]);
+  }
+  uint32_t all;
+  uint32_t run = cta_exclusive_sum<kRankThreads>(c, red, &all);
+#pragma unroll
+  for (int t = 0; t < kRankItems; ++t) {
+    if (w0 + t < words) hrank[w0 + t] = make_uint2(b[t], run);
+    run += __popc(b[t]);
+  }
+  if (threadIdx.x == 0) {
+    tbase[blockIdx.x] = all;
+    __threadfence();
+    last = atomicAdd(ticket, 1ull) == gridDim.x - 1 ? 1u : 0u;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  uint32_t carry = 0;
+  for (uint32_t t0 = 0; t0 < gridDim.x; t0 += kRankThreads) {
+    const uint32_t i = t0 + threadIdx.x;
+    const uint32_t v = i < gridDim.x ? __ldcg(tbase + i) : 0u;
+    const uint32_t before = cta_exclusive_sum<kRankThreads>(v, red, &all);
+    if (i < gridDim.x) tbase[i] = carry + before;
+    carry += all;
+  }
+  if (threadIdx.x == 0) *total = carry;
 }
 
 // Exclusive scan of bsum[0..nb) in one CTA; total into *total.
@@ -1476,15 +1552,25 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(uint64_t* bsum, uin
 // thread takes kFillItems nodes at a time and issues each step's loads for
 // all of them together (representatives; their original ids; the bitmap
 // words), so the three dependent gathers of a node overlap with the others'.
-constexpr int kFillItems = 4;
+// The grid is one resident wave and a CTA adds its counts with one atomic per
+// statistic: with one per warp the same-address atomics took most of the time
+// (1M nodes: 39 us a call, 16M: 106 us).
+constexpr int kFillThreads = 256, kFillItems = 4;
 
-__global__ void k_pid_fill(RankArgs r) {
+__global__ void __launch_bounds__(kFillThreads) k_pid_fill(RankArgs r) {
+  __shared__ unsigned int s_alone, s_mx;
+  __shared__ unsigned long long s_keys;
+  if (threadIdx.x == 0) {
+    s_alone = s_mx = 0;
+    s_keys = 0;
+  }
+  __syncthreads();
   unsigned int n_alone = 0, mx = 0;
   unsigned long long keys = 0;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t p0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p0 < r.n; p0 += stride * kFillItems) {
-    uint32_t h[kFillItems], o[kFillItems], hb[kFillItems];
-    uint64_t hw[kFillItems];
+    uint32_t h[kFillItems], o[kFillItems];
+    uint2 hr[kFillItems];
     bool live[kFillItems];
 #pragma unroll
     for (int t = 0; t < kFillItems; ++t) {
@@ -1496,12 +1582,8 @@ __global__ void k_pid_fill(RankArgs r) {
     for (int t = 0; t < kFillItems; ++t)
       if (live[t]) o[t] = r.p2o[h[t]];
 #pragma unroll
-    for (int t = 0; t < kFillItems; ++t) {
-      if (live[t]) {
-        hw[t] = r.hword[o[t] >> 5];
-        hb[t] = r.hbits[o[t] >> 5];
-      }
-    }
+    for (int t = 0; t < kFillItems; ++t)
+      if (live[t]) hr[t] = r.hrank[o[t] >> 5];
 #pragma unroll
     for (int t = 0; t < kFillItems; ++t) {
       const uint64_t p = p0 + (uint64_t)t * stride;
@@ -1512,7 +1594,7 @@ __global__ void k_pid_fill(RankArgs r) {
           keys += q;
           mx = max(mx, q);
         }
-        r.pid[p] = (uint32_t)hw[t] + (uint32_t)__popc(hb[t] & ((1u << (o[t] & 31)) - 1u));
+        r.pid[p] = r.tbase[o[t] >> kRankTileShift] + hr[t].y + (uint32_t)__popc(hr[t].x & ((1u << (o[t] & 31)) - 1u));
         const bool al = h[t] == (uint32_t)p && !r.member[p];
         r.alone[p] = al ? 1 : 0;
         n_alone += al ? 1u : 0u;
@@ -1522,17 +1604,22 @@ __global__ void k_pid_fill(RankArgs r) {
     }
   }
   n_alone = __reduce_add_sync(kFull, n_alone);
-  if ((threadIdx.x & 31) == 0 && n_alone) atomicAdd(&r.stats[8], (unsigned long long)n_alone);
-  if (r.ucnt) {
+  mx = __reduce_max_sync(kFull, mx);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      keys += __shfl_xor_sync(kFull, keys, o);
-      mx = max(mx, __shfl_xor_sync(kFull, mx, o));
+  for (int o = 16; o > 0; o >>= 1) keys += __shfl_xor_sync(kFull, keys, o);
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&s_alone, n_alone);
+    atomicMax(&s_mx, mx);
+    atomicAdd(&s_keys, keys);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (s_alone) atomicAdd(&r.stats[8], (unsigned long long)s_alone);
+    if (r.ucnt) {
+      atomicAdd(&r.stats[2], s_keys);
+      atomicMax(&r.stats[3], (unsigned long long)s_mx);
     }
-    if ((threadIdx.x & 31) == 0) {
-      atomicAdd(&r.stats[2], keys);
-      atomicMax(&r.stats[3], (unsigned long long)mx);
-    }
+    if (blockIdx.x == 0) r.stats[7] = *r.err;
   }
 }
 
@@ -2052,8 +2139,8 @@ Status settle_unresolved(Store& s, const GroupArgs& g, const VerifyArgs& v, bool
 // Scalars used per round (uint64 words of Store::d_scalars):
 //  [1] unresolved after the first pass, [2] key total, [3] largest signature,
 //  [4] collided nodes, [5] unresolved after a repair pass, [6] long-signature
-//  pairs, [7] error flags copy, [8] nodes alone in their block, [15] scan
-//  total (after renumbering: the number of blocks).
+//  pairs, [7] error flags copy, [8] nodes alone in their block, [9] ticket of
+//  k_head_ranks, [15] the number of blocks.
 Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint32_t* pid, uint64_t* blocks,
                       uint64_t* collided, bool with_stats, uint64_t* keys, uint64_t* maxsig, bool use_alone) {
   const uint64_t n = s.n, na = s.n_alive;
@@ -2128,23 +2215,24 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
   r.rep = g.rep;
   r.p2o = g.p2o;
   r.ucnt = with_stats ? ptr<uint32_t>(s.ucnt) : nullptr;
-  r.hbits = ptr<uint32_t>(s.hbits);
-  r.hword = ptr<uint64_t>(s.hword);
+  r.hrank = ptr<uint2>(s.hword);
+  r.tbase = ptr<uint32_t>(s.bsum);
+  r.err = ptr<uint32_t>(s.d_err);
   r.member = ptr<uint8_t>(s.member);
   r.alone = ptr<uint8_t>(s.alone);
   r.pid = pid;
   r.stats = sc;
   {
-    TimedScope ts(s, KBISIM_KERNEL_RENUMBER, n ? 5 : 0);  // 2 kernels + the 3 of scan64
+    TimedScope ts(s, KBISIM_KERNEL_RENUMBER, n ? 2 : 0);
     if (n) {
-      k_word_counts<<<(unsigned)std::min<uint64_t>(grid_for(words, 256), (uint64_t)sms * 16), 256, 0, s.stream>>>(
-          r.hbits, words, r.hword);
-      if (!(st = scan64(s, r.hword, words, nullptr)).ok()) return st;
-      k_pid_fill<<<(unsigned)std::min<uint64_t>(grid_for(n, 256), (uint64_t)sms * 16), 256, 0, s.stream>>>(r);
+      k_head_ranks<<<(unsigned)((words + kRankTile - 1) / kRankTile), kRankThreads, 0, s.stream>>>(
+          ptr<uint32_t>(s.hbits), words, ptr<uint2>(s.hword), ptr<uint32_t>(s.bsum), sc + 9, sc + 15);
+      k_pid_fill<<<(unsigned)std::min<uint64_t>(grid_for(n, kFillThreads * kFillItems),
+                                                resident_blocks(k_pid_fill, kFillThreads, 0, sms)),
+                   kFillThreads, 0, s.stream>>>(r);
     }
   }
   if (!(st = launch_check("renumber")).ok()) return st;
-  cudaMemcpyAsync(sc + 7, s.d_err.p, 4, cudaMemcpyDeviceToDevice, s.stream);
   if (!(st = read_scalars(s, h)).ok()) return st;
   *blocks = n ? h[15] : 0;  // scan total: heads
   if (s.checked && !(st = check_below(s, pid, na, *blocks, "identifiers")).ok()) return st;
