@@ -134,6 +134,16 @@ int sm_count(int device) {
   return cached[device];
 }
 
+// resident_blocks of one kernel, asked of the runtime once per device (the
+// answer depends on the compiled kernel and the device only).
+template <typename F>
+unsigned resident_grid(F kernel, int threads, size_t dyn_smem, int device, int* cached) {
+  const int sms = sm_count(device);
+  if (device < 0 || device >= 64) return resident_blocks(kernel, threads, dyn_smem, sms);
+  if (!cached[device]) cached[device] = (int)resident_blocks(kernel, threads, dyn_smem, 1);
+  return (unsigned)cached[device] * (unsigned)sms;
+}
+
 // --------------------------------------------------------------------------
 // Small device helpers
 // --------------------------------------------------------------------------
@@ -1232,13 +1242,18 @@ struct VerifyArgs {
   uint32_t* out_list;       // unresolved nodes
   unsigned long long* n_out;
   unsigned long long* n_collided;
-  uint32_t* long_list;      // (node, candidate) pairs with long signatures
+  // (node, candidate) pairs left to k_verify_long, in one array of pair_cap
+  // pairs: up to kMidSig elements from the front, longer ones from the back
+  uint32_t* long_list;
+  uint64_t pair_cap;
+  unsigned long long* n_mid;
   unsigned long long* n_long;
   uint32_t* hbits;          // head bitmap over original ids (canonical numbering)
   uint8_t* member;          // per internal id: this head has other members
 };
 
-constexpr uint32_t kShortSig = 8;
+constexpr uint32_t kShortSig = 8;   // compared by one thread
+constexpr uint32_t kMidSig = 64;    // compared by one warp, two elements per lane
 
 // Set equality of two duplicate-free key lists of the same length n <= kShortSig.
 template <typename K>
@@ -1331,18 +1346,21 @@ __global__ void __launch_bounds__(kVerNodeThreads) k_group_verify(GroupArgs g, V
       }
 #pragma unroll
       for (int t = 0; t < kVerItems; ++t) {
-        // long signatures: compared by a CTA later (a warp takes its places in the list together)
+        // longer signatures go to k_verify_long (a warp takes its places in a list together)
         const bool lng = act[t] && eq[t] && U[t] > kShortSig;
-        const unsigned lm = __ballot_sync(kFull, lng);
-        if (lm) {
-          unsigned long long q = 0;
-          if ((threadIdx.x & 31) == 0) q = atomicAdd(v.n_long, (unsigned long long)__popc(lm));
-          q = __shfl_sync(kFull, q, 0) + __popc(lm & lanes_below(threadIdx.x & 31));
-          if (lng) {
-            v.long_list[2 * q] = p[t];
-            v.long_list[2 * q + 1] = r[t];
-            act[t] = false;
-          }
+        if (!__any_sync(kFull, lng)) continue;
+        const uint32_t lane = threadIdx.x & 31;
+        const unsigned mm = __ballot_sync(kFull, lng && U[t] <= kMidSig), lm = __ballot_sync(kFull, lng && U[t] > kMidSig);
+        unsigned long long q = 0;
+        if (lane == 0 && mm) q = atomicAdd(v.n_mid, (unsigned long long)__popc(mm));
+        if (lane == 1 && lm) q = atomicAdd(v.n_long, (unsigned long long)__popc(lm));
+        const unsigned long long qm = __shfl_sync(kFull, q, 0), ql = __shfl_sync(kFull, q, 1);
+        if (lng) {
+          q = U[t] <= kMidSig ? qm + __popc(mm & lanes_below(lane))
+                              : v.pair_cap - 1 - (ql + __popc(lm & lanes_below(lane)));
+          v.long_list[2 * q] = p[t];
+          v.long_list[2 * q + 1] = r[t];
+          act[t] = false;
         }
       }
 #pragma unroll
@@ -1368,25 +1386,63 @@ __global__ void __launch_bounds__(kVerNodeThreads) k_group_verify(GroupArgs g, V
   }
 }
 
-// One CTA per (node, candidate) pair with a long signature: the candidate's
-// keys go into a shared-memory set, chunk by chunk, and the node's keys are
-// looked up; the sets are equal iff every one of the node's keys is found
-// (both lists are duplicate-free and of equal length).
+// The pairs k_group_verify left, their numbers read from the device, so that
+// the host need not wait for them before the next launches.  Lists are
+// duplicate-free and of equal length, so the sets are equal iff every one of
+// the node's keys is found among the candidate's.
+// Up to kMidSig elements (most pairs: the few blocks of level 0 bound the sets
+// of level 1): a warp per pair, two keys of each list per lane, the
+// candidate's keys handed round by shuffles.  Longer ones: a CTA per pair, the
+// candidate's keys in a shared-memory set, chunk by chunk.
 constexpr int kVerThreads = 256, kVerChunk = 4096;
 
 template <typename K>
 __host__ __device__ constexpr size_t verify_ws_bytes() { return team_set_bytes<K>(2 * kVerChunk, 0, kVerThreads); }
 
+__device__ __forceinline__ void settle_pair(const GroupArgs& g, const VerifyArgs& v, uint32_t p, uint32_t r, bool same) {
+  if (same) {
+    g.rep[p] = r;
+    mark_member(v, r);
+  } else {
+    mark_unresolved(v, g.rep, p);
+  }
+}
+
 template <typename K>
-__global__ void __launch_bounds__(kVerThreads) k_verify_long(GroupArgs g, VerifyArgs v, uint64_t count) {
+__global__ void __launch_bounds__(kVerThreads) k_verify_long(GroupArgs g, VerifyArgs v) {
   extern __shared__ __align__(16) char smem[];
-  TeamSet<K> ts = carve_set<K>(smem, 2 * kVerChunk, 0);
   const K* keys = static_cast<const K*>(v.sigkey);
-  for (uint64_t q = blockIdx.x; q < count; q += gridDim.x) {
-    const uint32_t p = v.long_list[2 * q], r = v.long_list[2 * q + 1];
-    const uint32_t U = v.ucnt[p];
-    const K* ka = keys + v.off[p];
-    const K* kb = keys + v.off[r];
+  const uint64_t n_mid = *v.n_mid, n_long = *v.n_long;
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t warps = ((uint64_t)gridDim.x * kVerThreads) >> 5;
+  for (uint64_t q = ((uint64_t)blockIdx.x * kVerThreads + threadIdx.x) >> 5; q < n_mid; q += warps) {
+    const uint2 pr = reinterpret_cast<const uint2*>(v.long_list)[q];
+    const uint32_t U = v.ucnt[pr.x];
+    const K* ka = keys + v.off[pr.x];
+    const K* kb = keys + v.off[pr.y];
+    const bool h0 = lane < U, h1 = lane + 32 < U;
+    const K a0 = h0 ? ka[lane] : (K)0, a1 = h1 ? ka[lane + 32] : (K)0;
+    const K b0 = h0 ? kb[lane] : (K)0, b1 = h1 ? kb[lane + 32] : (K)0;
+    bool f0 = !h0, f1 = !h1;
+    for (uint32_t j = 0; j < min(U, 32u); ++j) {
+      const K x = __shfl_sync(kFull, b0, j);
+      f0 |= a0 == x;
+      f1 |= a1 == x;
+    }
+    for (uint32_t j = 32; j < U; ++j) {
+      const K x = __shfl_sync(kFull, b1, j - 32);
+      f0 |= a0 == x;
+      f1 |= a1 == x;
+    }
+    const bool same = __all_sync(kFull, f0 && f1);
+    if (lane == 0) settle_pair(g, v, pr.x, pr.y, same);
+  }
+  TeamSet<K> ts = carve_set<K>(smem, 2 * kVerChunk, 0);
+  for (uint64_t q = blockIdx.x; q < n_long; q += gridDim.x) {
+    const uint2 pr = reinterpret_cast<const uint2*>(v.long_list)[v.pair_cap - 1 - q];
+    const uint32_t U = v.ucnt[pr.x];
+    const K* ka = keys + v.off[pr.x];
+    const K* kb = keys + v.off[pr.y];
     uint32_t found = 0;
     for (uint32_t c0 = 0; c0 < U; c0 += kVerChunk) {
       const uint32_t cn = min((uint32_t)kVerChunk, U - c0);
@@ -1399,14 +1455,7 @@ __global__ void __launch_bounds__(kVerThreads) k_verify_long(GroupArgs g, Verify
       __syncthreads();
     }
     found = team_sum<kVerThreads>(found, ts.red, threadIdx.x);
-    if (threadIdx.x == 0) {
-      if (found == U) {
-        g.rep[p] = r;
-        mark_member(v, r);
-      } else {
-        mark_unresolved(v, g.rep, p);
-      }
-    }
+    if (threadIdx.x == 0) settle_pair(g, v, pr.x, pr.y, found == U);
     __syncthreads();
   }
 }
@@ -1578,9 +1627,11 @@ __global__ void __launch_bounds__(kFillThreads) k_pid_fill(RankArgs r) {
       live[t] = p < r.n_alive;
       if (live[t]) h[t] = r.rep[p];
     }
+    // a hash collision leaves nodes without a head: the fill runs again once
+    // they are settled
 #pragma unroll
     for (int t = 0; t < kFillItems; ++t)
-      if (live[t]) o[t] = r.p2o[h[t]];
+      if (live[t]) o[t] = h[t] < r.n_alive ? r.p2o[h[t]] : 0u;
 #pragma unroll
     for (int t = 0; t < kFillItems; ++t)
       if (live[t]) hr[t] = r.hrank[o[t] >> 5];
@@ -1620,6 +1671,31 @@ __global__ void __launch_bounds__(kFillThreads) k_pid_fill(RankArgs r) {
       atomicMax(&r.stats[3], (unsigned long long)s_mx);
     }
     if (blockIdx.x == 0) r.stats[7] = *r.err;
+  }
+}
+
+// What a round starts from, cleared by one launch: up to kClearMax arrays of
+// 16-byte units, each filled with one word.  Seven cudaMemsetAsync of mostly a
+// few KB cost their launches: 1.5 us of device time and 2.5 us of host each.
+constexpr int kClearMax = 8, kClearThreads = 256;
+struct ClearArgs {
+  uint4* p[kClearMax];
+  uint64_t units[kClearMax];
+  uint32_t word[kClearMax];
+  int n = 0;
+  void add(void* a, uint64_t bytes, uint32_t w) {  // bytes rounded up: the arrays are allocated so
+    if (!bytes) return;
+    p[n] = static_cast<uint4*>(a);
+    units[n] = (bytes + 15) / 16;
+    word[n++] = w;
+  }
+};
+
+__global__ void __launch_bounds__(kClearThreads) k_clear(ClearArgs c) {
+  const uint64_t t0 = blockIdx.x * (uint64_t)kClearThreads + threadIdx.x, stride = (uint64_t)gridDim.x * kClearThreads;
+  for (int i = 0; i < c.n; ++i) {
+    const uint4 v = make_uint4(c.word[i], c.word[i], c.word[i], c.word[i]);
+    for (uint64_t u = t0; u < c.units[i]; u += stride) c.p[i][u] = v;
   }
 }
 
@@ -2081,25 +2157,42 @@ uint64_t table_capacity(uint64_t n) {
   return c;
 }
 
-// After a first insert + verify pass (scalars in h): compare the long
-// signatures, then regroup the nodes a hash collision left unresolved until
-// none is left.  The unresolved nodes hold whole classes; the smallest
-// unresolved node of each hash group heads its class, so every pass settles
-// at least one class per group (a pass that settles nothing is an error).
-Status settle_unresolved(Store& s, const GroupArgs& g, const VerifyArgs& v, bool key64, uint64_t* h, int long_cls) {
+void launch_insert(Store& s, const GroupArgs& g, const uint32_t* list, uint64_t count) {
+  static int cached[64];
+  const unsigned res = resident_grid(k_group_insert, kInsThreads, 0, s.device, cached);
+  k_group_insert<<<(unsigned)std::min<uint64_t>((count + kInsChunk - 1) / kInsChunk, res), kInsThreads, 0, s.stream>>>(
+      g, list, count);
+}
+
+template <typename K>
+void launch_verify_long(Store& s, const GroupArgs& g, const VerifyArgs& v, uint64_t count) {
+  static int cached[64];
+  const unsigned res = resident_grid(k_verify_long<K>, kVerThreads, verify_ws_bytes<K>(), s.device, cached);
+  k_verify_long<K><<<(unsigned)std::min<uint64_t>((count + 31) / 32, res), kVerThreads, verify_ws_bytes<K>(), s.stream>>>(g, v);
+}
+
+// Exact comparison of `count` nodes (of `list`, or all) with the head of their
+// hash: the short signatures, then the pairs left to k_verify_long.
+Status launch_verify(Store& s, const GroupArgs& g, const VerifyArgs& v, const uint32_t* list, uint64_t count) {
+  static int cached[64];
+  const unsigned res = resident_grid(k_group_verify, kVerNodeThreads, 0, s.device, cached);
+  k_group_verify<<<(unsigned)std::min<uint64_t>(grid_for(count, kVerTile), res), kVerNodeThreads, 0, s.stream>>>(
+      g, v, list, count);
+  if (v.mode != 0) {
+    if (v.key64) launch_verify_long<uint64_t>(s, g, v, count);
+    else launch_verify_long<uint32_t>(s, g, v, count);
+  }
+  return launch_check("exact comparison");
+}
+
+// After a first insert + verify pass (scalars in h): regroup the nodes a hash
+// collision left unresolved until none is left.  The unresolved nodes hold
+// whole classes; the smallest unresolved node of each hash group heads its
+// class, so every pass settles at least one class per group (a pass that
+// settles nothing is an error).
+Status settle_unresolved(Store& s, const GroupArgs& g, const VerifyArgs& v, uint64_t* h) {
   Status st;
   unsigned long long* sc = ptr<unsigned long long>(s.d_scalars);
-  const int sms = sm_count(s.device);
-  const unsigned ver_grid = resident_blocks(k_group_verify, kVerNodeThreads, 0, sms);
-  const unsigned ins_grid = resident_blocks(k_group_insert, kInsThreads, 0, sms);
-  if (h[6]) {
-    TimedScope ts(s, long_cls, 1);
-    const unsigned b = (unsigned)std::min<uint64_t>(h[6], (uint64_t)sms * 8);
-    if (key64) k_verify_long<uint64_t><<<b, kVerThreads, verify_ws_bytes<uint64_t>(), s.stream>>>(g, v, h[6]);
-    else k_verify_long<uint32_t><<<b, kVerThreads, verify_ws_bytes<uint32_t>(), s.stream>>>(g, v, h[6]);
-    if (!(st = launch_check("k_verify_long")).ok()) return st;
-    if (!(st = read_scalars(s, h)).ok()) return st;
-  }
   uint64_t unresolved_n = h[1];
   int cur = 0;
   while (unresolved_n > 0) {
@@ -2109,25 +2202,16 @@ Status settle_unresolved(Store& s, const GroupArgs& g, const VerifyArgs& v, bool
     VerifyArgs v2 = v;
     v2.out_list = ptr<uint32_t>(s.ulist[cur ^ 1]);
     v2.n_out = sc + 5;
-    const unsigned b2 = (unsigned)std::min<uint64_t>(grid_for(unresolved_n, kVerTile), ver_grid);
     {
-      TimedScope ts(s, KBISIM_KERNEL_OTHER, 2);
+      TimedScope ts(s, KBISIM_KERNEL_OTHER, v.mode ? 3 : 2);
       cudaMemsetAsync(s.table.p, 0xFF, cap * 8, s.stream);
-      cudaMemsetAsync(sc + 5, 0, 16, s.stream);  // [5] and [6]
-      k_group_insert<<<(unsigned)std::min<uint64_t>((unresolved_n + kInsChunk - 1) / kInsChunk, ins_grid),
-                       kInsThreads, 0, s.stream>>>(g2, ptr<uint32_t>(s.ulist[cur]), unresolved_n);
-      k_group_verify<<<b2, kVerNodeThreads, 0, s.stream>>>(g2, v2, ptr<uint32_t>(s.ulist[cur]), unresolved_n);
+      cudaMemsetAsync(sc + 5, 0, 16, s.stream);   // [5] and [6]
+      cudaMemsetAsync(sc + 10, 0, 8, s.stream);
+      launch_insert(s, g2, ptr<uint32_t>(s.ulist[cur]), unresolved_n);
+      st = launch_verify(s, g2, v2, ptr<uint32_t>(s.ulist[cur]), unresolved_n);
     }
-    if (!(st = launch_check("collision repair")).ok()) return st;
+    if (!st.ok()) return st;
     if (!(st = read_scalars(s, h)).ok()) return st;
-    if (h[6]) {
-      TimedScope ts(s, KBISIM_KERNEL_OTHER, 1);
-      const unsigned b = (unsigned)std::min<uint64_t>(h[6], (uint64_t)sms * 8);
-      if (key64) k_verify_long<uint64_t><<<b, kVerThreads, verify_ws_bytes<uint64_t>(), s.stream>>>(g2, v2, h[6]);
-      else k_verify_long<uint32_t><<<b, kVerThreads, verify_ws_bytes<uint32_t>(), s.stream>>>(g2, v2, h[6]);
-      if (!(st = launch_check("k_verify_long")).ok()) return st;
-      if (!(st = read_scalars(s, h)).ok()) return st;
-    }
     if (h[5] >= unresolved_n)
       return Status::Err(KBISIM_ERR_TIMEOUT, "collision repair made no progress");
     unresolved_n = h[5];
@@ -2136,27 +2220,27 @@ Status settle_unresolved(Store& s, const GroupArgs& g, const VerifyArgs& v, bool
   return Status::Ok();
 }
 
-// Scalars used per round (uint64 words of Store::d_scalars):
-//  [1] unresolved after the first pass, [2] key total, [3] largest signature,
-//  [4] collided nodes, [5] unresolved after a repair pass, [6] long-signature
-//  pairs, [7] error flags copy, [8] nodes alone in their block, [9] ticket of
-//  k_head_ranks, [15] the number of blocks.
-Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint32_t* pid, uint64_t* blocks,
-                      uint64_t* collided, bool with_stats, uint64_t* keys, uint64_t* maxsig, bool use_alone) {
-  const uint64_t n = s.n, na = s.n_alive;
-  Status st;
-  unsigned long long* sc = ptr<unsigned long long>(s.d_scalars);
+// Table slots of a grouping that inserts `ins` nodes.
+uint64_t group_slots(const Store& s, uint64_t ins) { return std::min<uint64_t>(s.tcap, table_capacity(ins)); }
+
+// Arguments of a grouping over the stored graph.
+GroupArgs group_args(Store& s, uint64_t slots) {
   GroupArgs g;
   g.hash = ptr<uint64_t>(s.hash);
   g.p2o = ptr<uint32_t>(s.p2o);
   g.o2p = ptr<uint32_t>(s.o2p);
   g.table = ptr<unsigned long long>(s.table);
-  g.tmask = s.tcap - 1;
+  g.tmask = slots - 1;
   g.slot = ptr<uint32_t>(s.slot);
   g.rep = ptr<uint32_t>(s.rep);
   g.err = ptr<uint32_t>(s.d_err);
-  g.alone = use_alone ? ptr<uint8_t>(s.alone) : nullptr;
-  g.read_first = mode == 0 ? 1 : 0;
+  g.alone = nullptr;
+  g.read_first = 0;
+  return g;
+}
+
+VerifyArgs verify_args(Store& s, int mode, const uint32_t* prev, bool key64) {
+  unsigned long long* sc = ptr<unsigned long long>(s.d_scalars);
   VerifyArgs v;
   v.mode = mode;
   v.key64 = key64 ? 1 : 0;
@@ -2165,49 +2249,72 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
   v.ucnt = ptr<uint32_t>(s.ucnt);
   v.off = ptr<uint64_t>(s.offsets);
   v.sigkey = s.sigkey.p;
+  v.out_list = ptr<uint32_t>(s.ulist[0]);
+  v.n_out = sc + 1;
   v.n_collided = sc + 4;
   v.long_list = ptr<uint32_t>(s.long_pairs);
+  v.pair_cap = std::max<uint64_t>(s.n, 1);
+  v.n_mid = sc + 10;
   v.n_long = sc + 6;
   v.hbits = ptr<uint32_t>(s.hbits);
   v.member = ptr<uint8_t>(s.member);
+  return v;
+}
+
+// Clear what a level's signatures and grouping start from: error flags,
+// scalars, the marks of the canonical numbering, the hash table for `ins`
+// inserted nodes, and, with hubs, their buckets' cursors and totals.
+Status clear_round(Store& s, uint64_t ins, bool hubs) {
+  ClearArgs c;
+  c.add(s.d_err.p, 16, 0u);
+  c.add(s.d_scalars.p, 16 * 8, 0u);
+  c.add(s.hbits.p, (s.n + 31) / 32 * 4, 0u);
+  c.add(s.member.p, s.n, 0u);
+  c.add(s.table.p, group_slots(s, ins) * 8, ~0u);
+  if (hubs) {
+    c.add(s.hub_cursor.p, s.n_hub_buckets * 4, 0u);
+    c.add(s.hub_acc.p, s.n_hub * 24, 0u);
+    c.add(s.hub_err.p, s.n_hub * 4, 0u);
+  }
+  uint64_t units = 0;
+  for (int i = 0; i < c.n; ++i) units += c.units[i];
+  TimedScope ts(s, KBISIM_KERNEL_OTHER, 1);
+  k_clear<<<(unsigned)std::min<uint64_t>(grid_for(units, kClearThreads), (uint64_t)sm_count(s.device) * 8),
+            kClearThreads, 0, s.stream>>>(c);
+  return launch_check("k_clear");
+}
+
+// Nodes a level's grouping inserts: all, or those not alone in their block at
+// the level before.
+uint64_t insert_count(const Store& s, bool use_alone) {
+  return use_alone ? s.n_alive - std::min(s.n_alive, s.n_alone) : s.n_alive;
+}
+
+// Group the nodes by exact signature (by label in mode 0) and number the
+// blocks, into pid.  clear_round has run.  The host waits once, at the end:
+// the comparison of long signatures takes its pairs' number from the device,
+// and the numbering is launched before the host knows whether a hash collision
+// left nodes unresolved; if one did they are settled and it runs again.
+// *hub_flags (mode 1): overflow flags of the hub passes before; when set, the
+// signatures were incomplete and nothing else is returned.
+//
+// Scalars used per round (uint64 words of Store::d_scalars):
+//  [1] unresolved after the first pass, [2] key total, [3] largest signature,
+//  [4] collided nodes, [5] unresolved after a repair pass, [6] and [10] pairs
+//  with long and with middle signatures, [7] error flags copy, [8] nodes alone
+//  in their block, [9] ticket of k_head_ranks, [15] the number of blocks.
+Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint32_t* pid, uint64_t* blocks,
+                      uint64_t* collided, bool with_stats, uint64_t* keys, uint64_t* maxsig, bool use_alone,
+                      uint32_t* hub_flags) {
+  const uint64_t n = s.n, na = s.n_alive;
+  Status st;
+  unsigned long long* sc = ptr<unsigned long long>(s.d_scalars);
+  GroupArgs g = group_args(s, group_slots(s, insert_count(s, use_alone)));
+  g.alone = use_alone ? ptr<uint8_t>(s.alone) : nullptr;
+  g.read_first = mode == 0 ? 1 : 0;
+  const VerifyArgs v = verify_args(s, mode, prev, key64);
   const uint64_t words = (n + 31) / 32;
-  const int sms = sm_count(s.device);
-  const unsigned ver_grid = resident_blocks(k_group_verify, kVerNodeThreads, 0, sms);
-  const unsigned gblocks = (unsigned)std::min<uint64_t>(grid_for(na, kVerTile), ver_grid);
-  {
-    TimedScope ts(s, KBISIM_KERNEL_OTHER, 0);
-    cudaMemsetAsync(s.d_scalars.p, 0, 15 * 8, s.stream);
-    // marks of the canonical numbering, set as representatives are settled
-    cudaMemsetAsync(s.hbits.p, 0, words * 4, s.stream);
-    cudaMemsetAsync(s.member.p, 0, n, s.stream);
-  }
-  v.out_list = ptr<uint32_t>(s.ulist[0]);
-  v.n_out = sc + 1;
-  // only nodes not alone in their previous block are inserted
-  const uint64_t ins = use_alone ? na - std::min(na, s.n_alone) : na;
-  const unsigned ins_grid = resident_blocks(k_group_insert, kInsThreads, 0, sms);
-  const uint64_t tcap = std::min<uint64_t>(s.tcap, table_capacity(ins));
-  g.tmask = tcap - 1;
-  {
-    TimedScope ts(s, KBISIM_KERNEL_OTHER, 0);
-    cudaMemsetAsync(s.table.p, 0xFF, tcap * 8, s.stream);
-  }
-  const unsigned iblocks = (unsigned)std::min<uint64_t>((na + kInsChunk - 1) / kInsChunk, ins_grid);
-  {
-    TimedScope ts(s, KBISIM_KERNEL_GROUP, na ? 1 : 0);
-    if (na) k_group_insert<<<iblocks, kInsThreads, 0, s.stream>>>(g, nullptr, na);
-  }
-  if (!(st = launch_check("k_group_insert")).ok()) return st;
-  {
-    TimedScope ts(s, KBISIM_KERNEL_VERIFY, 1);
-    k_group_verify<<<gblocks, kVerNodeThreads, 0, s.stream>>>(g, v, nullptr, na);
-  }
-  if (!(st = launch_check("k_group_verify")).ok()) return st;
-  uint64_t h[16];
-  if (!(st = read_scalars(s, h)).ok()) return st;
-  if (!(st = settle_unresolved(s, g, v, key64, h, KBISIM_KERNEL_VERIFY)).ok()) return st;
-  *collided = h[4];
-  if (s.checked && !(st = check_below(s, g.rep, na, n, "block heads")).ok()) return st;
+  uint64_t h[16] = {0};
   // canonical renumbering
   RankArgs r;
   r.n = n;
@@ -2222,19 +2329,43 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
   r.alone = ptr<uint8_t>(s.alone);
   r.pid = pid;
   r.stats = sc;
-  {
+  auto renumber = [&]() -> Status {
+    static int cached[64];
     TimedScope ts(s, KBISIM_KERNEL_RENUMBER, n ? 2 : 0);
-    if (n) {
-      k_head_ranks<<<(unsigned)((words + kRankTile - 1) / kRankTile), kRankThreads, 0, s.stream>>>(
-          ptr<uint32_t>(s.hbits), words, ptr<uint2>(s.hword), ptr<uint32_t>(s.bsum), sc + 9, sc + 15);
-      k_pid_fill<<<(unsigned)std::min<uint64_t>(grid_for(n, kFillThreads * kFillItems),
-                                                resident_blocks(k_pid_fill, kFillThreads, 0, sms)),
-                   kFillThreads, 0, s.stream>>>(r);
+    if (!n) return Status::Ok();
+    k_head_ranks<<<(unsigned)((words + kRankTile - 1) / kRankTile), kRankThreads, 0, s.stream>>>(
+        ptr<uint32_t>(s.hbits), words, ptr<uint2>(s.hword), ptr<uint32_t>(s.bsum), sc + 9, sc + 15);
+    k_pid_fill<<<(unsigned)std::min<uint64_t>(grid_for(n, kFillThreads * kFillItems),
+                                              resident_grid(k_pid_fill, kFillThreads, 0, s.device, cached)),
+                 kFillThreads, 0, s.stream>>>(r);
+    return launch_check("renumber");
+  };
+  if (na) {
+    {
+      TimedScope ts(s, KBISIM_KERNEL_GROUP, 1);
+      launch_insert(s, g, nullptr, na);
     }
+    if (!(st = launch_check("k_group_insert")).ok()) return st;
+    TimedScope ts(s, KBISIM_KERNEL_VERIFY, mode ? 2 : 1);
+    if (!(st = launch_verify(s, g, v, nullptr, na)).ok()) return st;
   }
-  if (!(st = launch_check("renumber")).ok()) return st;
+  if (s.checked) {  // representatives are checked before the numbering uses them
+    if (!(st = read_scalars(s, h)).ok()) return st;
+    if (!(st = settle_unresolved(s, g, v, h)).ok()) return st;
+    if (!(st = check_below(s, g.rep, na, n, "block heads")).ok()) return st;
+  }
+  if (!(st = renumber()).ok()) return st;
   if (!(st = read_scalars(s, h)).ok()) return st;
-  *blocks = n ? h[15] : 0;  // scan total: heads
+  if (hub_flags && (*hub_flags = (uint32_t)h[7] & (kErrHubOverflow | kErrHubSet))) return Status::Ok();
+  if (h[1] && !s.checked) {
+    if (!(st = settle_unresolved(s, g, v, h)).ok()) return st;
+    cudaMemsetAsync(sc + 2, 0, 16, s.stream);  // [2] and [3]
+    cudaMemsetAsync(sc + 8, 0, 16, s.stream);  // [8] and [9]
+    if (!(st = renumber()).ok()) return st;
+    if (!(st = read_scalars(s, h)).ok()) return st;
+  }
+  *collided = h[4];
+  *blocks = n ? h[15] : 0;  // heads
   if (s.checked && !(st = check_below(s, pid, na, *blocks, "identifiers")).ok()) return st;
   s.n_alone = h[8];
   if (keys) *keys = h[2];
@@ -2277,12 +2408,13 @@ Status hub_layout(Store& s) {
   if (!(st = ensure(s, s.hub_bbase, (s.n_hub + 1) * 8)).ok()) return st;
   if (!(st = ensure(s, s.hub_tbase, s.n_hub * 8)).ok()) return st;
   if (!(st = ensure(s, s.bucket_hub, s.n_hub_buckets * 4)).ok()) return st;
-  if (!(st = ensure(s, s.hub_cursor, s.n_hub_buckets * 4)).ok()) return st;
-  if (!(st = ensure(s, s.hub_acc, s.n_hub * 24)).ok()) return st;
+  if (!(st = ensure(s, s.hub_cursor, (s.n_hub_buckets * 4 + 15) & ~15ull)).ok()) return st;
+  if (!(st = ensure(s, s.hub_acc, (s.n_hub * 24 + 15) & ~15ull)).ok()) return st;
   if (!(st = ensure(s, s.hub_mode, s.n_hub)).ok()) return st;
   if (!(st = ensure(s, s.hub_force, s.n_hub)).ok()) return st;
-  if (!(st = ensure(s, s.hub_err, s.n_hub * 4)).ok()) return st;
-  cudaMemcpyAsync(s.hub_force.p, s.h_hub_force.data(), s.n_hub, cudaMemcpyHostToDevice, s.stream);  cudaMemcpyAsync(s.hub_bits.p, bits.data(), s.n_hub * 4, cudaMemcpyHostToDevice, s.stream);
+  if (!(st = ensure(s, s.hub_err, (s.n_hub * 4 + 15) & ~15ull)).ok()) return st;
+  cudaMemcpyAsync(s.hub_force.p, s.h_hub_force.data(), s.n_hub, cudaMemcpyHostToDevice, s.stream);
+  cudaMemcpyAsync(s.hub_bits.p, bits.data(), s.n_hub * 4, cudaMemcpyHostToDevice, s.stream);
   cudaMemcpyAsync(s.hub_cap.p, cap.data(), s.n_hub * 4, cudaMemcpyHostToDevice, s.stream);
   cudaMemcpyAsync(s.hub_bbase.p, bbase.data(), (s.n_hub + 1) * 8, cudaMemcpyHostToDevice, s.stream);
   cudaMemcpyAsync(s.hub_tbase.p, tbase.data(), s.n_hub * 8, cudaMemcpyHostToDevice, s.stream);
@@ -2292,16 +2424,119 @@ Status hub_layout(Store& s) {
 
 // The bucket pass with buckets of at most U key words: one resident wave of CTAs.
 template <typename K, int U>
-void launch_hub_bucket(Store& s, const SigArgs& a, const HubArgs& h, int sms) {
+void launch_hub_bucket(Store& s, const SigArgs& a, const HubArgs& h) {
+  static int cached[64];
   const unsigned g = (unsigned)std::min<uint64_t>(
-      s.n_hub_buckets, resident_blocks(k_hub_bucket<K, U>, kBucketThreads, sizeof(BucketSmem<K, U>), sms));
+      s.n_hub_buckets, resident_grid(k_hub_bucket<K, U>, kBucketThreads, sizeof(BucketSmem<K, U>), s.device, cached));
   k_hub_bucket<K, U><<<g, kBucketThreads, sizeof(BucketSmem<K, U>), s.stream>>>(a, h, s.n_hub_buckets);
 }
 
+// One pass over the hubs of a.fmask (NULL = all).  `cleared`: clear_round has
+// cleared the buckets' cursors, totals and flags.
 template <typename LabelT, typename K>
-Status run_signatures(Store& s, const SigArgs& a) {
+Status launch_hubs(Store& s, const SigArgs& a, bool cleared) {
+  Status st = ensure(s, s.hub_tmp, s.hub_tmp_words * sizeof(K));
+  if (!st.ok()) return st;
+  HubArgs h;
+  h.first = s.class_start[kClassHub];
+  h.hub_bits = ptr<uint32_t>(s.hub_bits);
+  h.hub_bbase = ptr<uint64_t>(s.hub_bbase);
+  h.hub_cap = ptr<uint32_t>(s.hub_cap);
+  h.hub_tbase = ptr<uint64_t>(s.hub_tbase);
+  h.bucket_hub = ptr<uint32_t>(s.bucket_hub);
+  h.chunks = ptr<uint4>(s.hub_chunks);
+  h.cursor = ptr<uint32_t>(s.hub_cursor);
+  h.hub_cur = ptr<unsigned long long>(s.hub_acc);
+  h.hub_term = reinterpret_cast<uint32_t*>(h.hub_cur + s.n_hub);
+  h.tmp = s.hub_tmp.p;
+  h.mode = ptr<uint8_t>(s.hub_mode);
+  h.force = ptr<uint8_t>(s.hub_force);
+  h.hub_err = ptr<uint32_t>(s.hub_err);
+  // each hub's chunks run either the deduplicating pass or the plain
+  // scatter, as its key sample says; both kernels cover all chunks and
+  // skip those of the other kind
+  TimedScope ts(s, KBISIM_KERNEL_SIG_HUB, 5);
+  if (!cleared) {
+    cudaMemsetAsync(h.cursor, 0, s.n_hub_buckets * 4, s.stream);
+    cudaMemsetAsync(s.hub_acc.p, 0, s.n_hub * 24, s.stream);
+    cudaMemsetAsync(s.hub_err.p, 0, s.n_hub * 4, s.stream);
+  }
+  k_hub_sample<LabelT, K><<<(unsigned)((s.n_hub + 7) / 8), 256, 0, s.stream>>>(a, h, s.n_hub);
+  k_hub_chunk<LabelT, K><<<(unsigned)s.n_hub_chunks, kChunkThreads, hub_chunk_smem<K>(), s.stream>>>(a, h);
+  k_hub_scatter<LabelT, K><<<(unsigned)s.n_hub_chunks, kChunkThreads, 0, s.stream>>>(a, h);
+  if (s.hub_ucap == (uint32_t)kHubUcaps[1]) launch_hub_bucket<K, kHubUcaps[1]>(s, a, h);
+  else if (s.hub_ucap == (uint32_t)kHubUcaps[2]) launch_hub_bucket<K, kHubUcaps[2]>(s, a, h);
+  else launch_hub_bucket<K, kHubUcaps[0]>(s, a, h);
+  k_hub_finish<<<(unsigned)((s.n_hub + 255) / 256), 256, 0, s.stream>>>(a, h, s.n_hub);
+  return launch_check("hub kernels");
+}
+
+// After a hub pass with overflow flags: grow the buckets of the hubs it
+// raised them for, and make a->fmask the mask of those hubs (the others'
+// signatures are written).
+Status grow_hubs(Store& s, SigArgs* a) {
+  std::vector<uint32_t> herr(s.n_hub);
+  std::vector<uint8_t> hmode(s.n_hub);
+  Status st = cuda_check(cudaMemcpyAsync(herr.data(), s.hub_err.p, s.n_hub * 4, cudaMemcpyDeviceToHost, s.stream),
+                         "hub flags");
+  if (st.ok())
+    st = cuda_check(cudaMemcpyAsync(hmode.data(), s.hub_mode.p, s.n_hub, cudaMemcpyDeviceToHost, s.stream),
+                    "hub modes");
+  if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "sync");
+  if (!st.ok()) return st;
+  for (uint64_t i = 0; i < s.n_hub; ++i) {
+    // a bucket overflowed (a key repeated many times): larger buckets for
+    // the hub, up to its degree, or, once the scatter has overflowed
+    // buckets kHubScatterShiftMax times larger than the first, the
+    // deduplicating pass; too many distinct keys in a bucket: more buckets
+    if (herr[i] & kErrHubOverflow) {
+      if (hmode[i] && s.h_hub_shift[i] >= kHubScatterShiftMax) s.h_hub_force[i] = 1;
+      else s.h_hub_shift[i] += 1;
+    }
+    if (herr[i] & kErrHubSet) s.h_hub_xbits[i] += 1;
+  }
+  if (!(st = hub_layout(s)).ok()) return st;
+  // the repeat's mask: the words of the hub id range, bits of the failed hubs
+  const uint64_t first = s.class_start[kClassHub], w0 = first >> 5, w1 = (first + s.n_hub + 31) >> 5;
+  std::vector<uint32_t> bits(w1 - w0, 0u);
+  for (uint64_t i = 0; i < s.n_hub; ++i)
+    if (herr[i]) bits[((first + i) >> 5) - w0] |= 1u << ((first + i) & 31);
+  if (!(st = ensure(s, s.hub_retry, (w1 + 1) * 4)).ok()) return st;
+  st = cuda_check(cudaMemcpyAsync(ptr<uint32_t>(s.hub_retry) + w0, bits.data(), bits.size() * 4,
+                                  cudaMemcpyHostToDevice, s.stream), "hub repeat mask");
+  if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "hub repeat mask");  // the host vector goes away
+  if (!st.ok()) return st;
+  a->fmask = ptr<uint32_t>(s.hub_retry);
+  return Status::Ok();
+}
+
+constexpr int kHubAttempts = 40;
+
+// Hub passes until no bucket overflows, the host waiting for each.
+template <typename LabelT, typename K>
+Status run_hubs(Store& s, const SigArgs& a) {
+  SigArgs ah = a;
+  for (int attempt = 0;; ++attempt) {
+    Status st = launch_hubs<LabelT, K>(s, ah, false);
+    if (!st.ok()) return st;
+    uint32_t e = 0;
+    st = cuda_check(cudaMemcpyAsync(&e, s.d_err.p, 4, cudaMemcpyDeviceToHost, s.stream), "read err");
+    if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "sync");
+    if (!st.ok()) return st;
+    if (!(e & (kErrHubOverflow | kErrHubSet))) return Status::Ok();
+    if (attempt >= kHubAttempts) return Status::Err(KBISIM_ERR_TIMEOUT, "hub bucket overflow persists");
+    if (!(st = grow_hubs(s, &ah)).ok()) return st;
+    cudaMemsetAsync(s.d_err.p, 0, 4, s.stream);
+  }
+}
+
+// Signatures of every node class.  With `defer`, the hubs run one pass over
+// what clear_round has cleared, and the caller looks at the overflow flags
+// once the round's other kernels have run (group_and_rank, grow_hubs);
+// otherwise they are complete on return.
+template <typename LabelT, typename K>
+Status run_signatures(Store& s, const SigArgs& a, bool defer) {
   Status st;
-  const int sms = sm_count(s.device);
   // thread-per-node classes: 0..4 (out-degree <= 8) in one launch, 5 and 6
   // (9..16, 17..32) in one launch each, so that each kernel carries only its
   // own unrolled code; class 7 (33..64) runs as 128-thread chunks
@@ -2344,86 +2579,7 @@ Status run_signatures(Store& s, const SigArgs& a) {
   }
   if (!(st = launch_check("k_sig_chunk")).ok()) return st;
   if (s.n_hub) {
-    auto run_hubs = [&]() -> Status {
-      Status st;
-      // a repeat after an overflow runs only the hubs that overflowed (the
-      // others' signatures are written): a mask over their internal ids
-      SigArgs ah = a;
-      for (int attempt = 0;; ++attempt) {
-        if (!(st = ensure(s, s.hub_tmp, s.hub_tmp_words * sizeof(K))).ok()) return st;
-        HubArgs h;
-        h.first = s.class_start[kClassHub];
-        h.hub_bits = ptr<uint32_t>(s.hub_bits);
-        h.hub_bbase = ptr<uint64_t>(s.hub_bbase);
-        h.hub_cap = ptr<uint32_t>(s.hub_cap);
-        h.hub_tbase = ptr<uint64_t>(s.hub_tbase);
-        h.bucket_hub = ptr<uint32_t>(s.bucket_hub);
-        h.chunks = ptr<uint4>(s.hub_chunks);
-        h.cursor = ptr<uint32_t>(s.hub_cursor);
-        h.hub_cur = ptr<unsigned long long>(s.hub_acc);
-        h.hub_term = reinterpret_cast<uint32_t*>(h.hub_cur + s.n_hub);
-        h.tmp = s.hub_tmp.p;
-        h.mode = ptr<uint8_t>(s.hub_mode);
-        h.force = ptr<uint8_t>(s.hub_force);
-        h.hub_err = ptr<uint32_t>(s.hub_err);
-        {
-          // each hub's chunks run either the deduplicating pass or the plain
-          // scatter, as its key sample says; both kernels cover all chunks and
-          // skip those of the other kind
-          TimedScope ts(s, KBISIM_KERNEL_SIG_HUB, 5);
-          cudaMemsetAsync(h.cursor, 0, s.n_hub_buckets * 4, s.stream);
-          cudaMemsetAsync(s.hub_acc.p, 0, s.n_hub * 24, s.stream);
-          cudaMemsetAsync(s.hub_err.p, 0, s.n_hub * 4, s.stream);
-          k_hub_sample<LabelT, K><<<(unsigned)((s.n_hub + 7) / 8), 256, 0, s.stream>>>(ah, h, s.n_hub);
-          k_hub_chunk<LabelT, K><<<(unsigned)s.n_hub_chunks, kChunkThreads, hub_chunk_smem<K>(), s.stream>>>(ah, h);
-          k_hub_scatter<LabelT, K><<<(unsigned)s.n_hub_chunks, kChunkThreads, 0, s.stream>>>(ah, h);
-          if (s.hub_ucap == (uint32_t)kHubUcaps[1]) launch_hub_bucket<K, kHubUcaps[1]>(s, ah, h, sms);
-          else if (s.hub_ucap == (uint32_t)kHubUcaps[2]) launch_hub_bucket<K, kHubUcaps[2]>(s, ah, h, sms);
-          else launch_hub_bucket<K, kHubUcaps[0]>(s, ah, h, sms);
-          k_hub_finish<<<(unsigned)((s.n_hub + 255) / 256), 256, 0, s.stream>>>(ah, h, s.n_hub);
-        }
-        if (!(st = launch_check("hub kernels")).ok()) return st;
-        uint32_t e = 0;
-        st = cuda_check(cudaMemcpyAsync(&e, s.d_err.p, 4, cudaMemcpyDeviceToHost, s.stream), "read err");
-        if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "sync");
-        if (!st.ok()) return st;
-        if (!(e & (kErrHubOverflow | kErrHubSet))) return Status::Ok();
-        if (attempt >= 40) return Status::Err(KBISIM_ERR_TIMEOUT, "hub bucket overflow persists");
-        std::vector<uint32_t> herr(s.n_hub);
-        std::vector<uint8_t> hmode(s.n_hub);
-        st = cuda_check(cudaMemcpyAsync(herr.data(), s.hub_err.p, s.n_hub * 4, cudaMemcpyDeviceToHost, s.stream),
-                        "hub flags");
-        if (st.ok())
-          st = cuda_check(cudaMemcpyAsync(hmode.data(), s.hub_mode.p, s.n_hub, cudaMemcpyDeviceToHost, s.stream),
-                          "hub modes");
-        if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "sync");
-        if (!st.ok()) return st;
-        for (uint64_t i = 0; i < s.n_hub; ++i) {
-          // a bucket overflowed (a key repeated many times): larger buckets for
-          // the hub, up to its degree, or, once the scatter has overflowed
-          // buckets kHubScatterShiftMax times larger than the first, the
-          // deduplicating pass; too many distinct keys in a bucket: more buckets
-          if (herr[i] & kErrHubOverflow) {
-            if (hmode[i] && s.h_hub_shift[i] >= kHubScatterShiftMax) s.h_hub_force[i] = 1;
-            else s.h_hub_shift[i] += 1;
-          }
-          if (herr[i] & kErrHubSet) s.h_hub_xbits[i] += 1;
-        }
-        if (!(st = hub_layout(s)).ok()) return st;
-        // the repeat's mask: the words of the hub id range, bits of the failed hubs
-        const uint64_t first = s.class_start[kClassHub], w0 = first >> 5, w1 = (first + s.n_hub + 31) >> 5;
-        std::vector<uint32_t> bits(w1 - w0, 0u);
-        for (uint64_t i = 0; i < s.n_hub; ++i)
-          if (herr[i]) bits[((first + i) >> 5) - w0] |= 1u << ((first + i) & 31);
-        if (!(st = ensure(s, s.hub_retry, (w1 + 1) * 4)).ok()) return st;
-        st = cuda_check(cudaMemcpyAsync(ptr<uint32_t>(s.hub_retry) + w0, bits.data(), bits.size() * 4,
-                                        cudaMemcpyHostToDevice, s.stream), "hub repeat mask");
-        if (!st.ok()) return st;
-        ah.fmask = ptr<uint32_t>(s.hub_retry);
-        cudaMemsetAsync(s.d_err.p, 0, 4, s.stream);
-      }
-    };
-    if (!s.tune_now) return run_hubs();
+    if (!s.tune_now) return defer ? launch_hubs<LabelT, K>(s, a, true) : run_hubs<LabelT, K>(s, a);
     // tuning (once per handle, on a full round from level 2 on): each bucket
     // size runs the hub pass twice, the sizes alternating, each pass timed
     // with the repeats its overflows need (a repeat runs only the hubs that
@@ -2455,7 +2611,7 @@ Status run_signatures(Store& s, const SigArgs& a) {
         s.hub_ucap = (uint32_t)kHubUcaps[c];
         if (!(st = hub_layout(s)).ok()) break;
         cudaEventRecord(ev[0], s.stream);
-        if (!(st = run_hubs()).ok()) break;
+        if (!(st = run_hubs<LabelT, K>(s, a)).ok()) break;
         cudaEventRecord(ev[1], s.stream);
         if (!(st = cuda_check(cudaEventSynchronize(ev[1]), "event")).ok()) break;
         cudaEventElapsedTime(&s.hub_tune_ms[c], ev[0], ev[1]);
@@ -2935,7 +3091,7 @@ Status compute_level0(Store& s) {
   if (done) return Status::Ok();
   const int sms = sm_count(s.device);
   const unsigned blocks = (unsigned)std::min<uint64_t>(grid_for(s.n_alive, 256), (uint64_t)sms * 16);
-  cudaMemsetAsync(s.d_err.p, 0, 4, s.stream);
+  if (!(st = clear_round(s, s.n_alive, false)).ok()) return st;
   {
     TimedScope ts(s, KBISIM_KERNEL_LABEL_GROUP, s.n_alive ? 1 : 0);
     if (s.n_alive)
@@ -2945,7 +3101,7 @@ Status compute_level0(Store& s) {
   if (!(st = launch_check("k_label_hash")).ok()) return st;
   uint64_t blocks_out = 0, coll = 0;
   st = group_and_rank(s, 0, nullptr, false, ptr<uint32_t>(s.level[0]), &blocks_out, &coll, false, nullptr,
-                      nullptr, false);
+                      nullptr, false, nullptr);
   if (!st.ok()) return st;
   s.counts[0] = blocks_out;
   return Status::Ok();
@@ -2988,7 +3144,7 @@ Status compute_round(Store& s, uint32_t i) {
     return Status::Err(KBISIM_ERR_TIMEOUT, "injected timeout (KBISIM_FAULT_TIMEOUT_ROUND)");
   Status st = ensure_round_scratch(s);
   if (!st.ok()) return st;
-  cudaMemsetAsync(s.d_err.p, 0, 4, s.stream);
+  if (!(st = clear_round(s, insert_count(s, true), s.n_hub != 0)).ok()) return st;
   if (s.checked && !(st = check_round_inputs(s, i)).ok()) return st;
   SigArgs a;
   a.off = ptr<uint64_t>(s.offsets);
@@ -3007,10 +3163,19 @@ Status compute_round(Store& s, uint32_t i) {
   const bool key64 = pbits + s.label_bits > 32;
   a.pbits = (int)pbits;
   s.tune_now = s.hub_tune == 1 && i >= 2 && !s.round_mask && s.n_hub;
-  if (s.label8)
-    st = key64 ? run_signatures<uint8_t, uint64_t>(s, a) : run_signatures<uint8_t, uint32_t>(s, a);
-  else
-    st = key64 ? run_signatures<uint32_t, uint64_t>(s, a) : run_signatures<uint32_t, uint32_t>(s, a);
+  // the hubs' overflow flags are read with the round's result; a round whose
+  // hubs overflowed signs those again and groups again (seldom: the growth is
+  // kept).  Checked mode and the tuning wait for complete signatures first.
+  const bool defer = !s.checked && !s.tune_now;
+  auto signatures = [&](auto label, auto key) {
+    return run_signatures<decltype(label), decltype(key)>(s, a, defer);
+  };
+  auto hubs_again = [&](auto label, auto key) { return launch_hubs<decltype(label), decltype(key)>(s, a, true); };
+  auto typed = [&](auto&& f) {
+    if (s.label8) return key64 ? f(uint8_t(), uint64_t()) : f(uint8_t(), uint32_t());
+    return key64 ? f(uint32_t(), uint64_t()) : f(uint32_t(), uint32_t());
+  };
+  st = typed(signatures);
   s.tune_now = false;
   if (!st.ok()) return st;
   if (s.round_mask && s.n_alive) {
@@ -3022,8 +3187,17 @@ Status compute_round(Store& s, uint32_t i) {
   uint64_t blocks = 0, coll = 0, keys = 0, maxsig = 0;
   // nodes alone in their block at level i-1 stay alone (Proposition 1): they
   // are heads of level i without a table lookup
-  st = group_and_rank(s, 1, a.prev, key64, ptr<uint32_t>(s.level[i]), &blocks, &coll, true, &keys, &maxsig, true);
-  if (!st.ok()) return st;
+  for (int attempt = 0;; ++attempt) {
+    uint32_t hub_flags = 0;
+    st = group_and_rank(s, 1, a.prev, key64, ptr<uint32_t>(s.level[i]), &blocks, &coll, true, &keys, &maxsig, true,
+                        &hub_flags);
+    if (!st.ok()) return st;
+    if (!hub_flags) break;
+    if (attempt >= kHubAttempts) return Status::Err(KBISIM_ERR_TIMEOUT, "hub bucket overflow persists");
+    if (!(st = grow_hubs(s, &a)).ok()) return st;
+    if (!(st = clear_round(s, insert_count(s, true), true)).ok()) return st;
+    if (!(st = typed(hubs_again)).ok()) return st;
+  }
   s.counts[i] = blocks;
   kbisim_round_stats rs;
   rs.blocks = blocks;
@@ -3054,59 +3228,30 @@ Status masked_signatures(Store& s, const uint32_t* prev, const uint32_t* fmask) 
   a.fmask = fmask;
   if (s.mt.key32) {  // labels below 2^pbits (the stores' width)
     a.pbits = (int)s.mt.pbits;
-    return s.label8 ? run_signatures<uint8_t, uint32_t>(s, a) : run_signatures<uint32_t, uint32_t>(s, a);
+    return s.label8 ? run_signatures<uint8_t, uint32_t>(s, a, false) : run_signatures<uint32_t, uint32_t>(s, a, false);
   }
   a.pbits = 32;
-  return s.label8 ? run_signatures<uint8_t, uint64_t>(s, a) : run_signatures<uint32_t, uint64_t>(s, a);
+  return s.label8 ? run_signatures<uint8_t, uint64_t>(s, a, false) : run_signatures<uint32_t, uint64_t>(s, a, false);
 }
 
 Status group_list(Store& s, const uint32_t* list, uint64_t count, const uint32_t* prev) {
   Status st = ensure_round_scratch(s);
   if (!st.ok() || !count) return st;
-  unsigned long long* sc = ptr<unsigned long long>(s.d_scalars);
-  GroupArgs g;
-  g.hash = ptr<uint64_t>(s.hash);
-  g.p2o = ptr<uint32_t>(s.p2o);
-  g.o2p = ptr<uint32_t>(s.o2p);
-  g.table = ptr<unsigned long long>(s.table);
-  g.slot = ptr<uint32_t>(s.slot);
-  g.rep = ptr<uint32_t>(s.rep);
-  g.err = ptr<uint32_t>(s.d_err);
-  g.alone = nullptr;
-  g.read_first = 0;
-  VerifyArgs v;
-  v.mode = 1;
-  v.key64 = s.mt.key32 ? 0 : 1;
-  v.nlabel = ptr<uint32_t>(s.nlabel);
-  v.prev = prev;
-  v.ucnt = ptr<uint32_t>(s.ucnt);
-  v.off = ptr<uint64_t>(s.offsets);
-  v.sigkey = s.sigkey.p;
-  v.n_collided = sc + 4;
-  v.long_list = ptr<uint32_t>(s.long_pairs);
-  v.n_long = sc + 6;
-  v.hbits = ptr<uint32_t>(s.hbits);  // marks of the canonical numbering: not used here
-  v.member = ptr<uint8_t>(s.member);
-  v.out_list = ptr<uint32_t>(s.ulist[0]);
-  v.n_out = sc + 1;
-  const uint64_t tcap = std::min<uint64_t>(s.tcap, table_capacity(count));
-  g.tmask = tcap - 1;
-  const int sms = sm_count(s.device);
+  const uint64_t slots = group_slots(s, count);
+  const GroupArgs g = group_args(s, slots);
+  // (the marks of the canonical numbering are not used here)
+  const VerifyArgs v = verify_args(s, 1, prev, !s.mt.key32);
   cudaMemsetAsync(s.d_scalars.p, 0, 15 * 8, s.stream);
-  cudaMemsetAsync(s.table.p, 0xFF, tcap * 8, s.stream);
+  cudaMemsetAsync(s.table.p, 0xFF, slots * 8, s.stream);
   {
-    TimedScope ts(s, KBISIM_KERNEL_GROUP, 2);
-    k_group_insert<<<(unsigned)std::min<uint64_t>((count + kInsChunk - 1) / kInsChunk,
-                                                  resident_blocks(k_group_insert, kInsThreads, 0, sms)),
-                     kInsThreads, 0, s.stream>>>(g, list, count);
-    k_group_verify<<<(unsigned)std::min<uint64_t>(grid_for(count, kVerTile),
-                                                  resident_blocks(k_group_verify, kVerNodeThreads, 0, sms)),
-                     kVerNodeThreads, 0, s.stream>>>(g, v, list, count);
+    TimedScope ts(s, KBISIM_KERNEL_GROUP, 3);
+    launch_insert(s, g, list, count);
+    st = launch_verify(s, g, v, list, count);
   }
-  if (!(st = launch_check("group list")).ok()) return st;
+  if (!st.ok()) return st;
   uint64_t h[16];
   if (!(st = read_scalars(s, h)).ok()) return st;
-  if (!(st = settle_unresolved(s, g, v, true, h, KBISIM_KERNEL_VERIFY)).ok()) return st;
+  if (!(st = settle_unresolved(s, g, v, h)).ok()) return st;
   uint32_t e = 0;
   st = cuda_check(cudaMemcpyAsync(&e, s.d_err.p, 4, cudaMemcpyDeviceToHost, s.stream), "group list");
   if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "group list");

@@ -1,0 +1,73 @@
+"""Kernel edges against the CPU oracle, bit for bit: sizes at which a kernel
+or a dispatch rule changes over."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1210_0748_gb300 import synth
+from paper_1210_0748_gb300.kbisim import KBisim
+from tests.gpu_util import assert_same, oracle_levels
+
+pytestmark = pytest.mark.gpu
+
+
+def _twins(width, wide, seed):
+    """Nodes whose signatures have `width` distinct elements, in groups of three: two equal sets (in another
+    order, with repeats) and one that differs in a single element."""
+    rng = np.random.default_rng(seed)
+    groups, targets = 40, 2 * width + 2
+    src, dst, lab = [], [], []
+    base = 3 * groups
+    labels = np.arange(base + targets, dtype=np.uint32)  # targets: a block each
+    labels[:base] = 0
+    for j in range(groups):
+        el = rng.choice(targets, width + 1, replace=False)
+        for t, els in enumerate((el[:-1], el[:-1][::-1], el[1:])):
+            els = np.concatenate([els, els[:3]])
+            src.append(np.full(els.size, 3 * j + t))
+            dst.append(base + els)
+            lab.append(els % 7 + (100_000 if wide else 0))
+    cat = [np.concatenate(x).astype(np.uint32) for x in (src, dst, lab)]
+    # a million labels push label and identifier past 32 bits
+    if wide:
+        cat[2][0] += 0xFF000000
+    return synth.from_coo(base + targets, *cat, labels)
+
+
+@pytest.mark.parametrize("wide", [False, True])
+@pytest.mark.parametrize("width", [1, 8, 9, 31, 32, 33, 63, 64, 65, 200])
+@pytest.mark.parametrize("hash_bits", [1, 64])
+def test_exact_comparison_at_the_list_lengths_where_it_changes(width, wide, hash_bits):
+    g = _twins(width, wide, seed=width)
+    ref = oracle_levels(g, 3)
+    with KBisim(hash_bits=hash_bits) as kb:
+        res = kb.build(g, 3)
+        assert_same(res, kb.all_pids(3), ref)
+
+
+@pytest.mark.parametrize("nodes", [1, 31, 32, 33, 1024, 32_767, 32_768, 32_769, 70_001])
+def test_numbering_at_tile_edges(nodes):
+    """Head ranks come in tiles of 2^15 original ids."""
+    g = synth.random_small_graph(nodes, 2 * nodes, node_labels=3, edge_labels=3, seed=nodes)
+    with KBisim() as kb:
+        res = kb.build(g, 4)
+        assert_same(res, kb.all_pids(4), oracle_levels(g, 4))
+
+
+@pytest.mark.parametrize("width", [5, 12, 40, 70])
+def test_frontier_groups_equal_new_signatures(width):
+    """Two nodes that get the same new signature in one batch share a block, whatever its length."""
+    g = synth.from_coo(2 + width + 1, [0] * width + [1] * width, list(range(2, 2 + width)) * 2, [0] * (2 * width),
+                       [0, 0] + list(range(1, width + 2)))
+    new = (np.array([0, 1], np.uint32), np.full(2, 2 + width, np.uint32), np.array([1, 1], np.uint32))
+    with KBisim(maintain="always") as kb:
+        kb.build(g, 2)
+        kb.update(2, ins=(np.array([2], np.uint32), np.array([3], np.uint32), np.array([0], np.uint32)))
+        res, _ = kb.update(2, ins=new)
+        assert kb.update_info()["incremental"]
+        src = np.concatenate([g.src(), [2], new[0]])
+        dst = np.concatenate([g.dst, [3], new[1]])
+        lab = np.concatenate([g.edge_label, [0], new[2]])
+        ref = oracle.kbisim(g.num_nodes, g.node_label, src, dst, lab, 2)
+        assert res.counts == ref.counts.tolist()
+        assert np.array_equal(kb.all_pids(2), ref.pids)
