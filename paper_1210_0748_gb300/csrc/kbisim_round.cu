@@ -144,6 +144,45 @@ unsigned resident_grid(F kernel, int threads, size_t dyn_smem, int device, int* 
   return (unsigned)cached[device] * (unsigned)sms;
 }
 
+// Launch overlap within a round (programmatic dependent launch).  Every
+// round kernel lets the next one start as soon as its own blocks are all
+// resident (overlap_next).  A kernel that reads what earlier ones of the round
+// wrote waits for them first (overlap_wait); the signature kernels do not
+// depend on one another, so they run side by side, each waiting only before it
+// ends, so that the end of any kernel still means the end of all before it.
+// At 1M edges a signature kernel has too few blocks to fill the device and its
+// 5 to 10 us are latency; at 256M edges only the tails overlap.
+//
+// The kernels that wait first (launch_chained) overlap only up to kChainEdges:
+// it hides launch latency (1M edges: 0.67 against 0.80 ms a refinement of five
+// rounds, 16M: 1.46 against 1.59), but blocks that already hold their place,
+// and their shared memory, slow the kernel before (200M edges: 20.2 against
+// 16.9 ms, 64M: 4.98 against 4.65; equal at 32M).
+constexpr uint64_t kChainEdges = 32ull << 20;
+__device__ __forceinline__ void overlap_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void overlap_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+void launch_if_overlapped(bool on, Store& s, void (*kernel)(P...), unsigned blocks, int threads, size_t smem,
+                          A&&... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(blocks);
+  c.blockDim = dim3((unsigned)threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s.stream;
+  c.attrs = &at;
+  c.numAttrs = on ? 1 : 0;
+  cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
+template <typename... P, typename... A>
+void launch_chained(Store& s, void (*kernel)(P...), unsigned blocks, int threads, size_t smem, A&&... args) {
+  launch_if_overlapped(s.m <= kChainEdges, s, kernel, blocks, threads, smem, args...);
+}
+
 // --------------------------------------------------------------------------
 // Small device helpers
 // --------------------------------------------------------------------------
@@ -470,7 +509,7 @@ constexpr int kSmallThreads = 256;
 // so the 64-slot class (most registers) does not limit the occupancy of the
 // others.
 template <int FIRST, int LAST, typename LabelT, typename K>
-__global__ void __launch_bounds__(kSmallThreads, small_min_blocks<LAST, K>()) k_sig_small(SigArgs a, SmallLaunch L) {
+__device__ __forceinline__ void sig_small_block(const SigArgs& a, const SmallLaunch& L) {
   // per-warp staging buffer for the largest class of this launch that is staged
   constexpr int kSLast = LAST == 0 ? 1 : (1 << (LAST - 1));
   constexpr int kSBuf = kSLast <= staged_max_s<K>() ? kSLast : 1;
@@ -512,6 +551,13 @@ __global__ void __launch_bounds__(kSmallThreads, small_min_blocks<LAST, K>()) k_
       break;
   }
 #undef KB_SMALL_CLASS
+}
+
+template <int FIRST, int LAST, typename LabelT, typename K>
+__global__ void __launch_bounds__(kSmallThreads, small_min_blocks<LAST, K>()) k_sig_small(SigArgs a, SmallLaunch L) {
+  overlap_next();
+  sig_small_block<FIRST, LAST, LabelT, K>(a, L);
+  overlap_wait();
 }
 
 // ---- out-degree 65..4096: CTA chunks of whole nodes -----------------------
@@ -618,7 +664,7 @@ __device__ __forceinline__ void chunk_keys(const SigArgs& a, uint64_t ebase, uin
 __device__ __forceinline__ unsigned lanes_below(uint32_t lane) { return (1u << lane) - 1u; }
 
 template <int NT, int MIN_DEG, typename LabelT, typename K>
-__global__ void __launch_bounds__(NT) k_sig_chunk(SigArgs a, const uint2* chunks) {
+__device__ __forceinline__ void sig_chunk_block(const SigArgs& a, const uint2* chunks) {
   extern __shared__ __align__(16) char smem_raw[];
   ChunkSmem<K, NT, MIN_DEG>& sm = *reinterpret_cast<ChunkSmem<K, NT, MIN_DEG>*>(smem_raw);
   const uint2 c = chunks[blockIdx.x];
@@ -687,6 +733,13 @@ __global__ void __launch_bounds__(NT) k_sig_chunk(SigArgs a, const uint2* chunks
   }
 }
 
+template <int NT, int MIN_DEG, typename LabelT, typename K>
+__global__ void __launch_bounds__(NT) k_sig_chunk(SigArgs a, const uint2* chunks) {
+  overlap_next();
+  sig_chunk_block<NT, MIN_DEG, LabelT, K>(a, chunks);
+  overlap_wait();
+}
+
 // ---- hubs: out-degree > kBlockMax ----------------------------------------
 // Pass 1 (k_hub_chunk): a CTA takes kHubChunk edges of one hub, deduplicates
 // their keys in shared memory as above (one region), listing each distinct
@@ -747,6 +800,8 @@ __device__ __forceinline__ uint32_t hub_bucket(K k, uint32_t bits) {
 
 template <typename LabelT, typename K>
 __global__ void __launch_bounds__(kChunkThreads) k_hub_chunk(SigArgs a, HubArgs h) {
+  overlap_next();
+  overlap_wait();
   extern __shared__ __align__(16) char smem_raw[];
   ChunkSmem<K, kChunkThreads, kChunkMinHub>& sm = *reinterpret_cast<ChunkSmem<K, kChunkThreads, kChunkMinHub>*>(smem_raw);
   K* list = reinterpret_cast<K*>(smem_raw + sizeof(ChunkSmem<K, kChunkThreads, kChunkMinHub>));
@@ -822,7 +877,7 @@ __global__ void __launch_bounds__(kChunkThreads) k_hub_chunk(SigArgs a, HubArgs 
 // set, which sends each distinct key of a chunk to the buckets once.  Other
 // hubs skip it, unless an earlier overflow forced the set on them.
 template <typename LabelT, typename K>
-__global__ void __launch_bounds__(256) k_hub_sample(SigArgs a, HubArgs h, uint64_t n_hub) {
+__device__ __forceinline__ void hub_sample_block(const SigArgs& a, const HubArgs& h, uint64_t n_hub) {
   constexpr int kPer = kHubSample / 32;
   __shared__ K sk[256 / 32][kHubSample];
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -846,6 +901,14 @@ __global__ void __launch_bounds__(256) k_hub_sample(SigArgs a, HubArgs h, uint64
   pairs = __reduce_add_sync(kFull, pairs);
   if (lane == 0) h.mode[hub] = (!h.force[hub] && pairs < (uint32_t)kHubSamplePairs) ? 1 : 0;
 }
+
+template <typename LabelT, typename K>
+__global__ void __launch_bounds__(256) k_hub_sample(SigArgs a, HubArgs h, uint64_t n_hub) {
+  overlap_next();
+  hub_sample_block<LabelT, K>(a, h, n_hub);
+  overlap_wait();
+}
+
 // Exclusive prefix sums of v[0..n) in place (n <= 2 * NT), by the whole CTA;
 // wsum holds NT / 32 words.  Ends with a barrier.
 template <int NT>
@@ -879,6 +942,8 @@ __device__ __forceinline__ void cta_exclusive_scan(uint32_t* v, uint32_t n, uint
 
 template <typename LabelT, typename K>
 __global__ void __launch_bounds__(kChunkThreads) k_hub_scatter(SigArgs a, HubArgs h) {
+  overlap_next();
+  overlap_wait();
   __shared__ uint32_t bcnt[kHubSmemBuckets];
   __shared__ uint32_t bpos[kHubSmemBuckets];
   __shared__ uint32_t lstart[kHubSmemBuckets];
@@ -980,6 +1045,8 @@ struct BucketSmem {
 // (its counter restarts from zero, so the keys written are written again).
 template <typename K, int UCAP>
 __global__ void __launch_bounds__(kBucketThreads, sizeof(K) == 4 ? 6 : 3) k_hub_bucket(SigArgs a, HubArgs h, uint64_t n_buckets) {
+  overlap_next();
+  overlap_wait();
   extern __shared__ __align__(16) char smem_raw[];
   BucketSmem<K, UCAP>& sm = *reinterpret_cast<BucketSmem<K, UCAP>*>(smem_raw);
   const uint32_t tid = threadIdx.x, lane = tid & 31;
@@ -1096,6 +1163,8 @@ __global__ void __launch_bounds__(kBucketThreads, sizeof(K) == 4 ? 6 : 3) k_hub_
 
 // Count and hash of every hub (of the mask) from its buckets' totals.
 __global__ void k_hub_finish(SigArgs a, HubArgs h, uint64_t n_hub) {
+  overlap_next();
+  overlap_wait();
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n_hub;
        i += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t p = h.first + i;
@@ -1154,6 +1223,8 @@ __device__ __forceinline__ uint32_t table_insert(const GroupArgs& g, uint64_t h,
 constexpr int kInsThreads = 256, kInsItems = 4, kInsChunk = kInsThreads * kInsItems, kInsSlots = 2 * kInsChunk;
 
 __global__ void __launch_bounds__(kInsThreads) k_group_insert(GroupArgs g, const uint32_t* list, uint64_t count) {
+  overlap_next();
+  overlap_wait();
   __shared__ unsigned long long skey[kInsSlots];
   __shared__ unsigned int smin[kInsSlots];
   __shared__ unsigned int sglob[kInsSlots];
@@ -1297,6 +1368,8 @@ constexpr int kVerNodeThreads = 256, kVerItems = 2, kVerTile = kVerNodeThreads *
 
 __global__ void __launch_bounds__(kVerNodeThreads) k_group_verify(GroupArgs g, VerifyArgs v, const uint32_t* list,
                                                                    uint64_t count) {
+  overlap_next();
+  overlap_wait();
   // heads this CTA has marked as having members: a block of millions of
   // nodes (level 0) then costs one global access per CTA, not per member
   __shared__ uint32_t seen[kMarkSeen];
@@ -1410,6 +1483,8 @@ __device__ __forceinline__ void settle_pair(const GroupArgs& g, const VerifyArgs
 
 template <typename K>
 __global__ void __launch_bounds__(kVerThreads) k_verify_long(GroupArgs g, VerifyArgs v) {
+  overlap_next();
+  overlap_wait();
   extern __shared__ __align__(16) char smem[];
   const K* keys = static_cast<const K*>(v.sigkey);
   const uint64_t n_mid = *v.n_mid, n_long = *v.n_long;
@@ -1523,6 +1598,8 @@ __device__ __forceinline__ uint32_t cta_exclusive_sum(uint32_t v, uint32_t* red,
 __global__ void __launch_bounds__(kRankThreads) k_head_ranks(const uint32_t* hbits, uint64_t words, uint2* hrank,
                                                              uint32_t* tbase, unsigned long long* ticket,
                                                              unsigned long long* total) {
+  overlap_next();
+  overlap_wait();
   __shared__ uint32_t red[kRankThreads / 32];
   __shared__ uint32_t last;
   const uint64_t w0 = (uint64_t)blockIdx.x * kRankTile + (uint64_t)threadIdx.x * kRankItems;
@@ -1607,6 +1684,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(uint64_t* bsum, uin
 constexpr int kFillThreads = 256, kFillItems = 4;
 
 __global__ void __launch_bounds__(kFillThreads) k_pid_fill(RankArgs r) {
+  overlap_next();
+  overlap_wait();
   __shared__ unsigned int s_alone, s_mx;
   __shared__ unsigned long long s_keys;
   if (threadIdx.x == 0) {
@@ -1692,6 +1771,7 @@ struct ClearArgs {
 };
 
 __global__ void __launch_bounds__(kClearThreads) k_clear(ClearArgs c) {
+  overlap_next();
   const uint64_t t0 = blockIdx.x * (uint64_t)kClearThreads + threadIdx.x, stride = (uint64_t)gridDim.x * kClearThreads;
   for (int i = 0; i < c.n; ++i) {
     const uint4 v = make_uint4(c.word[i], c.word[i], c.word[i], c.word[i]);
@@ -2160,15 +2240,16 @@ uint64_t table_capacity(uint64_t n) {
 void launch_insert(Store& s, const GroupArgs& g, const uint32_t* list, uint64_t count) {
   static int cached[64];
   const unsigned res = resident_grid(k_group_insert, kInsThreads, 0, s.device, cached);
-  k_group_insert<<<(unsigned)std::min<uint64_t>((count + kInsChunk - 1) / kInsChunk, res), kInsThreads, 0, s.stream>>>(
-      g, list, count);
+  launch_chained(s, k_group_insert, (unsigned)std::min<uint64_t>((count + kInsChunk - 1) / kInsChunk, res),
+                    kInsThreads, 0, g, list, count);
 }
 
 template <typename K>
 void launch_verify_long(Store& s, const GroupArgs& g, const VerifyArgs& v, uint64_t count) {
   static int cached[64];
   const unsigned res = resident_grid(k_verify_long<K>, kVerThreads, verify_ws_bytes<K>(), s.device, cached);
-  k_verify_long<K><<<(unsigned)std::min<uint64_t>((count + 31) / 32, res), kVerThreads, verify_ws_bytes<K>(), s.stream>>>(g, v);
+  launch_chained(s, k_verify_long<K>, (unsigned)std::min<uint64_t>((count + 31) / 32, res), kVerThreads,
+                    verify_ws_bytes<K>(), g, v);
 }
 
 // Exact comparison of `count` nodes (of `list`, or all) with the head of their
@@ -2176,8 +2257,8 @@ void launch_verify_long(Store& s, const GroupArgs& g, const VerifyArgs& v, uint6
 Status launch_verify(Store& s, const GroupArgs& g, const VerifyArgs& v, const uint32_t* list, uint64_t count) {
   static int cached[64];
   const unsigned res = resident_grid(k_group_verify, kVerNodeThreads, 0, s.device, cached);
-  k_group_verify<<<(unsigned)std::min<uint64_t>(grid_for(count, kVerTile), res), kVerNodeThreads, 0, s.stream>>>(
-      g, v, list, count);
+  launch_chained(s, k_group_verify, (unsigned)std::min<uint64_t>(grid_for(count, kVerTile), res), kVerNodeThreads,
+                    0, g, v, list, count);
   if (v.mode != 0) {
     if (v.key64) launch_verify_long<uint64_t>(s, g, v, count);
     else launch_verify_long<uint32_t>(s, g, v, count);
@@ -2333,11 +2414,12 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
     static int cached[64];
     TimedScope ts(s, KBISIM_KERNEL_RENUMBER, n ? 2 : 0);
     if (!n) return Status::Ok();
-    k_head_ranks<<<(unsigned)((words + kRankTile - 1) / kRankTile), kRankThreads, 0, s.stream>>>(
-        ptr<uint32_t>(s.hbits), words, ptr<uint2>(s.hword), ptr<uint32_t>(s.bsum), sc + 9, sc + 15);
-    k_pid_fill<<<(unsigned)std::min<uint64_t>(grid_for(n, kFillThreads * kFillItems),
-                                              resident_grid(k_pid_fill, kFillThreads, 0, s.device, cached)),
-                 kFillThreads, 0, s.stream>>>(r);
+    launch_chained(s, k_head_ranks, (unsigned)((words + kRankTile - 1) / kRankTile), kRankThreads, 0,
+                      ptr<uint32_t>(s.hbits), words, ptr<uint2>(s.hword), ptr<uint32_t>(s.bsum), sc + 9, sc + 15);
+    launch_chained(s, k_pid_fill,
+                      (unsigned)std::min<uint64_t>(grid_for(n, kFillThreads * kFillItems),
+                                                   resident_grid(k_pid_fill, kFillThreads, 0, s.device, cached)),
+                      kFillThreads, 0, r);
     return launch_check("renumber");
   };
   if (na) {
@@ -2428,7 +2510,7 @@ void launch_hub_bucket(Store& s, const SigArgs& a, const HubArgs& h) {
   static int cached[64];
   const unsigned g = (unsigned)std::min<uint64_t>(
       s.n_hub_buckets, resident_grid(k_hub_bucket<K, U>, kBucketThreads, sizeof(BucketSmem<K, U>), s.device, cached));
-  k_hub_bucket<K, U><<<g, kBucketThreads, sizeof(BucketSmem<K, U>), s.stream>>>(a, h, s.n_hub_buckets);
+  launch_chained(s, k_hub_bucket<K, U>, g, kBucketThreads, sizeof(BucketSmem<K, U>), a, h, s.n_hub_buckets);
 }
 
 // One pass over the hubs of a.fmask (NULL = all).  `cleared`: clear_round has
@@ -2461,13 +2543,13 @@ Status launch_hubs(Store& s, const SigArgs& a, bool cleared) {
     cudaMemsetAsync(s.hub_acc.p, 0, s.n_hub * 24, s.stream);
     cudaMemsetAsync(s.hub_err.p, 0, s.n_hub * 4, s.stream);
   }
-  k_hub_sample<LabelT, K><<<(unsigned)((s.n_hub + 7) / 8), 256, 0, s.stream>>>(a, h, s.n_hub);
-  k_hub_chunk<LabelT, K><<<(unsigned)s.n_hub_chunks, kChunkThreads, hub_chunk_smem<K>(), s.stream>>>(a, h);
-  k_hub_scatter<LabelT, K><<<(unsigned)s.n_hub_chunks, kChunkThreads, 0, s.stream>>>(a, h);
+  launch_chained(s, k_hub_sample<LabelT, K>, (unsigned)((s.n_hub + 7) / 8), 256, 0, a, h, s.n_hub);
+  launch_chained(s, k_hub_chunk<LabelT, K>, (unsigned)s.n_hub_chunks, kChunkThreads, hub_chunk_smem<K>(), a, h);
+  launch_chained(s, k_hub_scatter<LabelT, K>, (unsigned)s.n_hub_chunks, kChunkThreads, 0, a, h);
   if (s.hub_ucap == (uint32_t)kHubUcaps[1]) launch_hub_bucket<K, kHubUcaps[1]>(s, a, h);
   else if (s.hub_ucap == (uint32_t)kHubUcaps[2]) launch_hub_bucket<K, kHubUcaps[2]>(s, a, h);
   else launch_hub_bucket<K, kHubUcaps[0]>(s, a, h);
-  k_hub_finish<<<(unsigned)((s.n_hub + 255) / 256), 256, 0, s.stream>>>(a, h, s.n_hub);
+  launch_chained(s, k_hub_finish, (unsigned)((s.n_hub + 255) / 256), 256, 0, a, h, s.n_hub);
   return launch_check("hub kernels");
 }
 
@@ -2554,28 +2636,32 @@ Status run_signatures(Store& s, const SigArgs& a, bool defer) {
   };
   const SmallLaunch L04 = small_launch(0, 4), L5 = small_launch(5, 5), L6 = small_launch(6, 6);
   const uint32_t n04 = L04.bstart[5], n5 = L5.bstart[6] - L5.bstart[5], n6 = L6.bstart[7] - L6.bstart[6];
+  // the first kernel starts when all earlier work has ended, clear_round's
+  // launch (which starts then and writes nothing these kernels read) excepted
+  bool overlapped = defer;
+  auto run = [&](auto kernel, unsigned blocks, int threads, size_t smem, auto... args) {
+    launch_if_overlapped(overlapped, s, kernel, blocks, threads, smem, args...);
+    overlapped = true;
+  };
   {
     TimedScope ts(s, KBISIM_KERNEL_SIG_SMALL, (n04 ? 1 : 0) + (n5 ? 1 : 0) + (n6 ? 1 : 0) + (s.n_mid_chunks[0] ? 1 : 0));
-    if (n04) k_sig_small<0, 4, LabelT, K><<<n04, kSmallThreads, 0, s.stream>>>(a, L04);
-    if (n5) k_sig_small<5, 5, LabelT, K><<<n5, kSmallThreads, 0, s.stream>>>(a, L5);
-    if (n6) k_sig_small<6, 6, LabelT, K><<<n6, kSmallThreads, 0, s.stream>>>(a, L6);
+    if (n04) run(k_sig_small<0, 4, LabelT, K>, n04, kSmallThreads, 0, a, L04);
+    if (n5) run(k_sig_small<5, 5, LabelT, K>, n5, kSmallThreads, 0, a, L5);
+    if (n6) run(k_sig_small<6, 6, LabelT, K>, n6, kSmallThreads, 0, a, L6);
     if (s.n_mid_chunks[0])
-      k_sig_chunk<kSmallChunkThreads, kChunkMin64, LabelT, K>
-          <<<(unsigned)s.n_mid_chunks[0], kSmallChunkThreads,
-             sizeof(ChunkSmem<K, kSmallChunkThreads, kChunkMin64>), s.stream>>>(a, ptr<uint2>(s.mid_chunks));
+      run(k_sig_chunk<kSmallChunkThreads, kChunkMin64, LabelT, K>, (unsigned)s.n_mid_chunks[0], kSmallChunkThreads,
+          sizeof(ChunkSmem<K, kSmallChunkThreads, kChunkMin64>), a, ptr<uint2>(s.mid_chunks));
   }
   if (!(st = launch_check("k_sig_small")).ok()) return st;
   if (s.n_mid_chunks[1] + s.n_mid_chunks[2]) {
     TimedScope ts(s, KBISIM_KERNEL_SIG_MEDIUM, (s.n_mid_chunks[1] ? 1 : 0) + (s.n_mid_chunks[2] ? 1 : 0));
     if (s.n_mid_chunks[1])
-      k_sig_chunk<kSmallChunkThreads, kChunkMin1K, LabelT, K>
-          <<<(unsigned)s.n_mid_chunks[1], kSmallChunkThreads,
-             sizeof(ChunkSmem<K, kSmallChunkThreads, kChunkMin1K>), s.stream>>>(
-              a, ptr<uint2>(s.mid_chunks) + s.n_mid_chunks[0]);
+      run(k_sig_chunk<kSmallChunkThreads, kChunkMin1K, LabelT, K>, (unsigned)s.n_mid_chunks[1], kSmallChunkThreads,
+          sizeof(ChunkSmem<K, kSmallChunkThreads, kChunkMin1K>), a, ptr<uint2>(s.mid_chunks) + s.n_mid_chunks[0]);
     if (s.n_mid_chunks[2])
-      k_sig_chunk<kChunkThreads, kChunkMin4K, LabelT, K>
-          <<<(unsigned)s.n_mid_chunks[2], kChunkThreads, sizeof(ChunkSmem<K, kChunkThreads, kChunkMin4K>),
-             s.stream>>>(a, ptr<uint2>(s.mid_chunks) + s.n_mid_chunks[0] + s.n_mid_chunks[1]);
+      run(k_sig_chunk<kChunkThreads, kChunkMin4K, LabelT, K>, (unsigned)s.n_mid_chunks[2], kChunkThreads,
+          sizeof(ChunkSmem<K, kChunkThreads, kChunkMin4K>), a,
+          ptr<uint2>(s.mid_chunks) + s.n_mid_chunks[0] + s.n_mid_chunks[1]);
   }
   if (!(st = launch_check("k_sig_chunk")).ok()) return st;
   if (s.n_hub) {
