@@ -242,6 +242,7 @@ struct Store {
   std::vector<uint32_t> h_hub_shift;  // per hub: larger buckets, after a bucket's capacity was exceeded
   std::vector<uint8_t> h_hub_force;   // per hub: deduplicating chunk pass, after a scatter overflowed
   std::vector<uint64_t> h_hub_deg;
+  bool hub_grew = false, hub_calm = false;  // buckets grew in this round; not in the last one from level 2 on
 
   // levels (all kept: history for extend / maintenance), internal order
   std::vector<Buf> level;

@@ -2566,6 +2566,7 @@ Status grow_hubs(Store& s, SigArgs* a) {
                     "hub modes");
   if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "sync");
   if (!st.ok()) return st;
+  s.hub_grew = true;
   for (uint64_t i = 0; i < s.n_hub; ++i) {
     // a bucket overflowed (a key repeated many times): larger buckets for
     // the hub, up to its degree, or, once the scatter has overflowed
@@ -2593,6 +2594,7 @@ Status grow_hubs(Store& s, SigArgs* a) {
 }
 
 constexpr int kHubAttempts = 40;
+constexpr uint64_t kHubCalmNodes = 4u << 20;
 
 // Hub passes until no bucket overflows, the host waiting for each.
 template <typename LabelT, typename K>
@@ -2835,6 +2837,7 @@ Status chunk_lists_hubs(Store& s, bool fresh, MidPlan* mp) {
     s.h_hub_xbits.assign(s.n_hub, 0);
     s.h_hub_shift.assign(s.n_hub, 0);
     s.h_hub_force.assign(s.n_hub, 0);
+    s.hub_calm = false;
   }
   s.h_hub_deg.assign(s.n_hub, 0);
   s.hub_edges = 0;
@@ -3251,8 +3254,11 @@ Status compute_round(Store& s, uint32_t i) {
   s.tune_now = s.hub_tune == 1 && i >= 2 && !s.round_mask && s.n_hub;
   // the hubs' overflow flags are read with the round's result; a round whose
   // hubs overflowed signs those again and groups again (seldom: the growth is
-  // kept).  Checked mode and the tuning wait for complete signatures first.
-  const bool defer = !s.checked && !s.tune_now;
+  // kept).  Checked mode and the tuning wait for complete signatures first, and
+  // so does a large graph until a round has passed without growth: a repeated
+  // grouping costs it more than the wait (200M edges: 1 ms of the first pass).
+  const bool defer = !s.checked && !s.tune_now && (s.hub_calm || s.n_alive <= kHubCalmNodes);
+  s.hub_grew = false;
   auto signatures = [&](auto label, auto key) {
     return run_signatures<decltype(label), decltype(key)>(s, a, defer);
   };
@@ -3284,6 +3290,7 @@ Status compute_round(Store& s, uint32_t i) {
     if (!(st = clear_round(s, insert_count(s, true), true)).ok()) return st;
     if (!(st = typed(hubs_again)).ok()) return st;
   }
+  if (i >= 2) s.hub_calm = !s.hub_grew;  // (level 1 has few distinct keys)
   s.counts[i] = blocks;
   kbisim_round_stats rs;
   rs.blocks = blocks;
