@@ -20,23 +20,21 @@ constexpr uint32_t kNone32 = 0xFFFFFFFFu;
 constexpr uint32_t kDead = KBISIM_DELETED;
 
 // Degree classes of the signature kernels.
-constexpr int kSmallMax = 64;      // out-degree <= 64: one thread per node, keys in registers
-constexpr int kWarpMax = 256;      // class bounds above kSmallMax (65..256, 257..1024, 1025..4096):
-constexpr int kWarp2Max = 1024;    //   node ordering only; all three run as CTA chunks of whole
-constexpr int kBlockMax = 4096;    //   nodes (at most kChunkEdges edges per chunk)
-constexpr int kChunkThreads = 512; // threads of the chunk kernels for out-degree > kWarp2Max and hubs
-constexpr int kSmallChunkThreads = 128;  // threads of the chunk kernel for out-degree kSmallMax+1..kWarp2Max
+constexpr int kSmallMax = 64;      // out-degree <= 32: one thread per node, keys in registers; 33..64: a warp per node
+constexpr int kWarpMax = 256;      // 65..256: a warp per node
+constexpr int kWarp2Max = 1024;    // 257..1024 and 1025..4096: a CTA per node
+constexpr int kBlockMax = 4096;
+constexpr int kChunkThreads = 512; // CTA of a node of out-degree 1025..4096, and of a hub chunk
+constexpr int kSmallChunkThreads = 128;  // CTA of a node of out-degree 257..1024
 constexpr int kChunkItems = 8;     // edges per thread
 constexpr int kChunkEdges = kChunkThreads * kChunkItems;  // 4096 = kBlockMax
-constexpr int kChunkMaxNodes = 64; // nodes per medium chunk (each has > kSmallMax edges)
 constexpr int kHubChunk = kChunkEdges;  // hub edges per chunk CTA
 constexpr int kSmallClasses = 8;        // out-degree 0, 1, 2, 3-4, 5-8, 9-16, 17-32, 33-64
 constexpr int kClassWarp = kSmallClasses, kClassWarp2 = kSmallClasses + 1, kClassBlock = kSmallClasses + 2,
               kClassHub = kSmallClasses + 3, kClassDead = kSmallClasses + 4;
 constexpr int kNumClasses = kSmallClasses + 5;  // including deleted nodes (last)
-static_assert(kChunkEdges >= kBlockMax, "a medium node must fit one chunk");
-static_assert(kChunkEdges / (kSmallMax + 1) < kChunkMaxNodes, "chunk node table too small");
-static_assert(kSmallChunkThreads * kChunkItems >= kWarp2Max, "a node of out-degree <= kWarp2Max must fit one small chunk");
+static_assert(kChunkEdges >= kBlockMax, "a node of out-degree <= kBlockMax must fit one CTA");
+static_assert(kSmallChunkThreads * kChunkItems >= kWarp2Max, "a node of out-degree <= kWarp2Max must fit a small CTA");
 
 // Degree class of a node of out-degree d: 0, 1, 2, 3-4, 5-8, 9-16, 17-32,
 // 33-64, then 65..kWarpMax, ..kWarp2Max, ..kBlockMax, hubs.
@@ -226,8 +224,6 @@ struct Store {
   // degree classes (internal id ranges)
   uint64_t class_start[kNumClasses + 1] = {0};
   uint64_t n_hub = 0;
-  Buf mid_chunks;              // uint2 (first node, node count): runs of whole nodes, three lists
-  uint64_t n_mid_chunks[3] = {0, 0, 0};  // out-degree 33..64, 65..1024, 1025..4096
   Buf hub_bits;                // uint32 [n_hub]  log2(bucket count)
   Buf hub_bbase;               // uint64 [n_hub+1] first bucket of each hub
   Buf hub_cap;                 // uint32 [n_hub]  key words a bucket of this hub can hold

@@ -348,6 +348,9 @@ struct SigArgs {
   int pbits;          // bits of a child identifier in a 32-bit key
   uint32_t* err;
   const uint32_t* fmask;  // bitmap over internal ids of the nodes to sign (NULL = all)
+  // nodes alone in their previous block (NULL = not known): they stay alone, so
+  // nothing reads their keys or hash, only their number of distinct elements
+  const uint8_t* alone;
 };
 
 // The node is to be signed this pass (every node unless a frontier mask is set).
@@ -560,48 +563,18 @@ __global__ void __launch_bounds__(kSmallThreads, small_min_blocks<LAST, K>()) k_
   overlap_wait();
 }
 
-// ---- out-degree 65..4096: CTA chunks of whole nodes -----------------------
-// A chunk is a run of consecutive medium nodes with at most kChunkEdges edges
-// in all; their edges are contiguous in the relabelled CSR.  One CTA:
-//  1. loads the chunk's edges coalesced, kChunkItems per thread, and makes
-//     their keys (every load is in flight before the first key is used);
-//  2. inserts each key into its node's region of a shared-memory hash set
-//     (node j owns slots [2 o_j, 2 o_{j+1}), o_j its first edge in the chunk,
-//     so a region is at most half full).  The lane whose insert puts a key
-//     into the set writes it out at once: the 32 consecutive edges of a warp
-//     belong to at most two nodes, so each node's output position is claimed
-//     once per warp step;
-//  3. adds the hash terms of the keys a warp step inserted to their node's
-//     sums as it claims their output positions, and at the end writes each
-//     node's distinct-key count and hash.
-// The key equal to the empty-slot marker is kept as a per-node flag.
+// ---- chunk-level sets of the hubs ------------------------------------------
+// A region of a shared-memory hash set takes a chunk's keys: the lane whose
+// insert puts a key into the set lists it.  The key equal to the empty-slot
+// marker is kept as a flag.
 
-// A chunk CTA of NT threads takes up to NT * kChunkItems edges of nodes with
-// out-degree >= MIN_DEG (> 32, so that 32 consecutive edges meet at most two
-// nodes).
-template <int NT, int MIN_DEG>
-struct ChunkShape {
-  static_assert(MIN_DEG > 32, "a warp step must meet at most two nodes");
-  static constexpr int kEdges = NT * kChunkItems;
-  static constexpr int kSlots = 2 * kEdges;
-  static constexpr int kMaxNodes = kEdges / MIN_DEG + 1;
-};
-
-template <typename K, int NT, int MIN_DEG>
+template <typename K>
 struct ChunkSmem {
-  using Shape = ChunkShape<NT, MIN_DEG>;
-  K slot[Shape::kSlots];
-  uint32_t off[Shape::kMaxNodes + 1];  // node starts relative to the chunk's first edge
-  uint32_t cnt[Shape::kMaxNodes];      // distinct keys written per node
-  uint32_t empty[Shape::kMaxNodes];    // the node's key equal to KeyOps<K>::kEmpty was seen
-  uint32_t lo[Shape::kMaxNodes];       // term sum halves of the node's distinct keys
-  uint32_t hi[Shape::kMaxNodes];
+  K slot[2 * kHubChunk];
+  uint32_t cnt;    // distinct keys listed
+  uint32_t empty;  // the key equal to KeyOps<K>::kEmpty was seen
+  uint32_t pad[2];
 };
-
-// Chunk kernel shapes: out-degree 33..64 and 65..1024 in 128-thread CTAs,
-// 1025..4096 and hub pieces in 512-thread CTAs.
-constexpr int kChunkMin64 = kSmallMax / 2 + 1, kChunkMin1K = kSmallMax + 1, kChunkMin4K = kWarp2Max + 1;
-constexpr int kChunkMinHub = kBlockMax + 1;
 
 __device__ __forceinline__ uint32_t key_h32(uint32_t k) { return k; }
 __device__ __forceinline__ uint32_t key_h32(uint64_t k) { return (uint32_t)(k >> 32) ^ (uint32_t)k; }
@@ -641,17 +614,13 @@ __device__ __forceinline__ bool region_insert(uint32_t base, uint32_t rb, uint32
   return false;
 }
 
-template <typename K, int NT, int MIN_DEG>
-__device__ __forceinline__ void chunk_clear(ChunkSmem<K, NT, MIN_DEG>& sm, uint32_t slots) {
-  uint4* s4 = reinterpret_cast<uint4*>(sm.slot);
+// All ones into the first `slots` words of a 16-byte aligned array (slots a
+// multiple of 16 / sizeof(K)), by NT threads.
+template <int NT, typename K>
+__device__ __forceinline__ void fill_empty(K* slot, uint32_t slots, uint32_t rank) {
+  uint4* s4 = reinterpret_cast<uint4*>(slot);
   const uint4 ones = make_uint4(~0u, ~0u, ~0u, ~0u);
-  for (uint32_t i = threadIdx.x; i < slots * sizeof(K) / 16; i += NT) s4[i] = ones;
-  for (uint32_t i = threadIdx.x; i < (uint32_t)ChunkShape<NT, MIN_DEG>::kMaxNodes; i += NT) {
-    sm.cnt[i] = 0;
-    sm.empty[i] = 0;
-    sm.lo[i] = 0;
-    sm.hi[i] = 0;
-  }
+  for (uint32_t i = rank; i < slots * (uint32_t)sizeof(K) / 16; i += NT) s4[i] = ones;
 }
 
 template <int NT, typename LabelT, typename K>
@@ -663,80 +632,218 @@ __device__ __forceinline__ void chunk_keys(const SigArgs& a, uint64_t ebase, uin
 // Lanes below `lane`.
 __device__ __forceinline__ unsigned lanes_below(uint32_t lane) { return (1u << lane) - 1u; }
 
-template <int NT, int MIN_DEG, typename LabelT, typename K>
-__device__ __forceinline__ void sig_chunk_block(const SigArgs& a, const uint2* chunks) {
-  extern __shared__ __align__(16) char smem_raw[];
-  ChunkSmem<K, NT, MIN_DEG>& sm = *reinterpret_cast<ChunkSmem<K, NT, MIN_DEG>*>(smem_raw);
-  const uint2 c = chunks[blockIdx.x];
-  const uint64_t first = c.x;
-  const uint32_t nn = c.y;
-  const uint32_t tid = threadIdx.x, lane = tid & 31;
-  if (a.fmask && !__syncthreads_or(tid < nn && in_mask(a, first + tid))) return;
-  const uint64_t ebase = a.off[first];
-  const uint32_t E = (uint32_t)(a.off[first + nn] - ebase);
-  for (uint32_t i = tid; i <= nn; i += NT) sm.off[i] = (uint32_t)(a.off[first + i] - ebase);
-  chunk_clear(sm, (2 * E + 3) & ~3u);
-  __syncthreads();
-  K key[kChunkItems];
-  chunk_keys<NT, LabelT, K>(a, ebase, E, key);
-  K* out = static_cast<K*>(a.sigkey) + ebase;
-  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sm.slot);
-  uint32_t j = 0;
-  // one copy of the loop body: the keys rotate through key[0]
-#pragma unroll 1
-  for (int t = 0; t < kChunkItems; ++t) {
-    const uint32_t e = tid + t * NT;
-    const K kt = key[0];
+
+// Insert k (!= kEmpty) into a power-of-two set of hmask + 1 slots at
+// shared-window address `base`, home slot from the key's low bits (the keys of
+// one hub bucket share their top bits).  The compare-and-swap is the probe
+// itself: one shared access per probed slot, whether the slot is empty, holds
+// k or holds another key.  Returns 1 if this call inserted k, 0 if k was
+// present, -1 if the set is full.
+template <typename K>
+__device__ __forceinline__ int pow2_insert(uint32_t base, uint32_t hmask, K k) {
+  uint32_t s = key_h32(k) & hmask;
+  for (uint32_t t = 0; t <= hmask; ++t) {
+    const K cur = atoms_cas(base + s * (uint32_t)sizeof(K), KeyOps<K>::kEmpty, k);
+    if (cur == KeyOps<K>::kEmpty) return 1;
+    if (cur == k) return 0;
+    s = (s + 1) & hmask;
+  }
+  return -1;
+}
+
+// ---- out-degree 33..256: a warp per node ----------------------------------
+// A warp takes `per` consecutive nodes (at most 32; lane j holds the bounds and
+// results of node j) and signs them one after the other: the node's edges come
+// coalesced, STEPS per lane, their gathers all in flight; every key is inserted
+// into the warp's own power-of-two set in shared memory, and the lane whose
+// insert was the first writes the key out behind those found before.  Count and
+// term sums stay in registers, and the hashes of the warp's nodes are made
+// together at the end, a lane per node.
+// Bound by instruction issue.  Chunks of whole nodes in a CTA-wide set, where a
+// step of 32 edges could meet two nodes, spent most of their 239 warp
+// instructions a step on finding the node, on two-node sums and on shared
+// atomics; a step that belongs to one node needs about 70.  
+constexpr int kNodeWarps = 8;  // per CTA
+
+template <int STEPS, typename LabelT, typename K>
+__device__ __forceinline__ void sig_one_node(const SigArgs& a, uint64_t e0, uint32_t d, bool alone, uint32_t sbase,
+                                             K* set, const Policies& pol, uint32_t& U, uint32_t& lo, uint32_t& hi) {
+  const uint32_t lane = threadIdx.x & 31;
+  K key[STEPS];
+  edge_keys<STEPS, 0, STEPS, LabelT, K>(a, e0 + lane, 32u, e0 + d, pol, key);
+  fill_empty<32>(set, 64u * STEPS, lane);
+  __syncwarp();
+  K* out = static_cast<K*>(a.sigkey) + e0;
+  uint32_t u = 0, l = 0, h = 0;
+  bool seen_empty = false;
 #pragma unroll
-    for (int q = 0; q + 1 < kChunkItems; ++q) key[q] = key[q + 1];
+  for (int t = 0; t < STEPS; ++t) {
+    if (STEPS > 2 && 32u * t >= d) break;
+    const K k = key[t];
     bool fresh = false;
-    if (e < E) {
-      while (sm.off[j + 1] <= e) ++j;
-      fresh = kt == KeyOps<K>::kEmpty
-                  ? atomicExch(&sm.empty[j], 1u) == 0u
-                  : region_insert(sbase, 2 * sm.off[j], 2 * (sm.off[j + 1] - sm.off[j]), kt);
+    const bool valid = lane + 32u * t < d;
+    if (valid && k != KeyOps<K>::kEmpty) fresh = pow2_insert(sbase, 64u * STEPS - 1, k) > 0;
+    const unsigned em = __ballot_sync(kFull, valid && k == KeyOps<K>::kEmpty);
+    if (em) {  // the key that marks empty slots: kept beside the set
+      fresh |= !seen_empty && lane == (uint32_t)__ffs(em) - 1u;
+      seen_empty = true;
     }
     const unsigned fm = __ballot_sync(kFull, fresh);
-    if (fm == 0u) continue;
-    // valid lanes are a prefix of the warp and span nodes jA and jA + 1
-    const uint32_t jA = __shfl_sync(kFull, j, 0);
-    const bool inA = j == jA;
-    const unsigned fa = fm & __ballot_sync(kFull, inA), fb = fm & ~fa;
-    // the fresh keys' term sums, per node of the step, go with their count
-    const uint64_t tm = fresh ? elem_term(kt, a.seed) : 0ull;
-    const uint32_t loA = __reduce_add_sync(kFull, inA ? (uint32_t)tm : 0u);
-    const uint32_t hiA = __reduce_add_sync(kFull, inA ? (uint32_t)(tm >> 32) : 0u);
-    const uint32_t loB = __reduce_add_sync(kFull, inA ? 0u : (uint32_t)tm);
-    const uint32_t hiB = __reduce_add_sync(kFull, inA ? 0u : (uint32_t)(tm >> 32));
-    uint32_t base = 0;
-    if (lane == 0 && fa) {
-      base = atomicAdd(&sm.cnt[jA], (uint32_t)__popc(fa));
-      atomicAdd(&sm.lo[jA], loA);
-      atomicAdd(&sm.hi[jA], hiA);
+    if (!alone && fresh) {
+      out[u + __popc(fm & lanes_below(lane))] = k;
+      const uint64_t tm = elem_term(k, a.seed);
+      l += (uint32_t)tm;
+      h += (uint32_t)(tm >> 32);
     }
-    if (lane == 31 && fb) {
-      base = atomicAdd(&sm.cnt[jA + 1], (uint32_t)__popc(fb));
-      atomicAdd(&sm.lo[jA + 1], loB);
-      atomicAdd(&sm.hi[jA + 1], hiB);
-    }
-    const uint32_t bA = __shfl_sync(kFull, base, 0), bB = __shfl_sync(kFull, base, 31);
-    if (fresh)
-      out[sm.off[j] + (inA ? bA + __popc(fa & lanes_below(lane)) : bB + __popc(fb & lanes_below(lane)))] = kt;
+    u += __popc(fm);
   }
-  __syncthreads();
-  // count and hash of each node of the chunk
-  for (uint32_t i = tid; i < nn; i += NT) {
-    const uint64_t p = first + i;
-    const uint32_t U = sm.cnt[i];
-    a.ucnt[p] = U;
-    a.hash[p] = node_hash(((uint64_t)sm.hi[i] << 32) | sm.lo[i], a.prev[p], U, a.seed, a.mask);
+  U = u;
+  if (!alone) {
+    lo = __reduce_add_sync(kFull, l);
+    hi = __reduce_add_sync(kFull, h);
+  }
+  __syncwarp();  // the set is cleared for the next node only after every insert
+}
+
+template <int MAXSTEPS, typename LabelT, typename K>
+__device__ __forceinline__ void sig_warp_block(const SigArgs& a, uint64_t first, uint64_t count, uint32_t per) {
+  __shared__ __align__(16) K sets[kNodeWarps][64 * MAXSTEPS];
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint64_t i0 = ((uint64_t)blockIdx.x * kNodeWarps + w) * per;
+  if (i0 >= count) return;
+  const uint32_t nn = (uint32_t)min((uint64_t)per, count - i0);
+  const uint64_t p0 = first + i0, p = p0 + min(lane, nn - 1);
+  const uint64_t b = a.off[p];
+  const uint32_t d_l = (uint32_t)(a.off[p + 1] - b);
+  const uint64_t base = __shfl_sync(kFull, b, 0);
+  const uint32_t r_l = (uint32_t)(b - base);
+  const bool mine = lane < nn && in_mask(a, p);
+  const bool alone_l = a.alone && a.alone[p];
+  unsigned todo = __ballot_sync(kFull, mine);
+  const unsigned alone_m = __ballot_sync(kFull, alone_l);
+  uint32_t U_l = 0, lo_l = 0, hi_l = 0;
+  const Policies pol;
+  K* set = sets[w];
+  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(set);
+  while (todo) {
+    const uint32_t j = (uint32_t)__ffs(todo) - 1u;
+    todo &= todo - 1;
+    const uint64_t e0 = base + __shfl_sync(kFull, r_l, j);
+    const uint32_t d = __shfl_sync(kFull, d_l, j);
+    const bool alone = (alone_m >> j) & 1u;
+    uint32_t U = 0, lo = 0, hi = 0;
+    if constexpr (MAXSTEPS == 8) {
+      if (d <= 128) sig_one_node<4, LabelT, K>(a, e0, d, alone, sbase, set, pol, U, lo, hi);
+      else sig_one_node<8, LabelT, K>(a, e0, d, alone, sbase, set, pol, U, lo, hi);
+    } else {
+      sig_one_node<MAXSTEPS, LabelT, K>(a, e0, d, alone, sbase, set, pol, U, lo, hi);
+    }
+    if (lane == j) {
+      U_l = U;
+      lo_l = lo;
+      hi_l = hi;
+    }
+  }
+  if (mine) {
+    a.ucnt[p] = U_l;
+    if (!alone_l) a.hash[p] = node_hash(((uint64_t)hi_l << 32) | lo_l, a.prev[p], U_l, a.seed, a.mask);
   }
 }
 
-template <int NT, int MIN_DEG, typename LabelT, typename K>
-__global__ void __launch_bounds__(NT) k_sig_chunk(SigArgs a, const uint2* chunks) {
+template <int MAXSTEPS, typename LabelT, typename K>
+__global__ void __launch_bounds__(kNodeWarps * 32, sizeof(K) == 4 ? 6 : 4) k_sig_warp(SigArgs a, uint64_t first, uint64_t count,
+                                                                uint32_t per) {
   overlap_next();
-  sig_chunk_block<NT, MIN_DEG, LabelT, K>(a, chunks);
+  sig_warp_block<MAXSTEPS, LabelT, K>(a, first, count, per);
+  overlap_wait();
+}
+
+// ---- out-degree 257..4096: a CTA per node ----------------------------------
+// As above with one set for the CTA; a warp inserts all its steps, then takes
+// the places of its fresh keys with one reservation on the node's count.
+constexpr int kCtaNodeItems = 8;  // edges per thread
+
+template <typename K>
+struct CtaNodeSmem {
+  uint32_t cnt, lo, hi, empty;
+  __device__ __forceinline__ K* set() { return reinterpret_cast<K*>(this + 1); }
+};
+
+template <int NT, typename K>
+__host__ __device__ constexpr size_t cta_node_smem() { return sizeof(CtaNodeSmem<K>) + 2 * (size_t)NT * kCtaNodeItems * sizeof(K); }
+
+template <int NT, int ITEMS, typename LabelT, typename K>
+__device__ __forceinline__ void sig_cta_node(const SigArgs& a, uint64_t p, uint64_t e0, uint32_t d, CtaNodeSmem<K>& sm) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31;
+  const bool alone = a.alone && a.alone[p];
+  const Policies pol;
+  K key[ITEMS];
+  edge_keys<ITEMS, 0, ITEMS, LabelT, K>(a, e0 + tid, NT, e0 + d, pol, key);
+  constexpr uint32_t kSlots = 2 * NT * ITEMS;
+  if (tid < 4) (&sm.cnt)[tid] = 0;
+  fill_empty<NT>(sm.set(), kSlots, tid);
+  __syncthreads();
+  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sm.set());
+  unsigned fms[ITEMS];
+  uint32_t lo = 0, hi = 0, total = 0;
+#pragma unroll
+  for (int t = 0; t < ITEMS; ++t) {
+    fms[t] = 0u;
+    if ((uint32_t)t * NT >= d) continue;  // the same for the whole CTA
+    const K k = key[t];
+    bool fresh = false;
+    if (tid + (uint32_t)t * NT < d)
+      fresh = k == KeyOps<K>::kEmpty ? atomicExch(&sm.empty, 1u) == 0u : pow2_insert(sbase, kSlots - 1, k) > 0;
+    fms[t] = __ballot_sync(kFull, fresh);
+    total += __popc(fms[t]);
+    if (!alone && fresh) {
+      const uint64_t tm = elem_term(k, a.seed);
+      lo += (uint32_t)tm;
+      hi += (uint32_t)(tm >> 32);
+    }
+  }
+  if (alone) {
+    if (lane == 0) atomicAdd(&sm.cnt, total);
+  } else if (total) {
+    uint32_t at = 0;
+    if (lane == 0) at = atomicAdd(&sm.cnt, total);
+    at = __shfl_sync(kFull, at, 0);
+    K* out = static_cast<K*>(a.sigkey) + e0;
+#pragma unroll
+    for (int t = 0; t < ITEMS; ++t) {
+      if ((fms[t] >> lane) & 1u) out[at + __popc(fms[t] & lanes_below(lane))] = key[t];
+      at += __popc(fms[t]);
+    }
+    lo = __reduce_add_sync(kFull, lo);
+    hi = __reduce_add_sync(kFull, hi);
+    if (lane == 0) {
+      atomicAdd(&sm.lo, lo);
+      atomicAdd(&sm.hi, hi);
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    a.ucnt[p] = sm.cnt;
+    if (!alone) a.hash[p] = node_hash(((uint64_t)sm.hi << 32) | sm.lo, a.prev[p], sm.cnt, a.seed, a.mask);
+  }
+}
+
+template <int NT, typename LabelT, typename K>
+__device__ __forceinline__ void sig_cta_block(const SigArgs& a, uint64_t first) {
+  extern __shared__ __align__(16) char smem_raw[];
+  CtaNodeSmem<K>& sm = *reinterpret_cast<CtaNodeSmem<K>*>(smem_raw);
+  const uint64_t p = first + blockIdx.x;
+  if (!in_mask(a, p)) return;
+  const uint64_t e0 = a.off[p];
+  const uint32_t d = (uint32_t)(a.off[p + 1] - e0);
+  if (d <= NT * kCtaNodeItems / 2) sig_cta_node<NT, kCtaNodeItems / 2, LabelT, K>(a, p, e0, d, sm);
+  else sig_cta_node<NT, kCtaNodeItems, LabelT, K>(a, p, e0, d, sm);
+}
+
+template <int NT, typename LabelT, typename K>
+__global__ void __launch_bounds__(NT) k_sig_cta(SigArgs a, uint64_t first) {
+  overlap_next();
+  sig_cta_block<NT, LabelT, K>(a, first);
   overlap_wait();
 }
 
@@ -789,7 +896,7 @@ constexpr uint32_t kHubScatterShiftMax = 2;  // bucket growth of a scattering hu
 
 template <typename K>
 __host__ __device__ constexpr size_t hub_chunk_smem() {
-  return sizeof(ChunkSmem<K, kChunkThreads, kChunkMinHub>) + (size_t)kHubChunk * sizeof(K) + 2 * kHubSmemBuckets * sizeof(uint32_t);
+  return sizeof(ChunkSmem<K>) + (size_t)kHubChunk * sizeof(K) + 2 * kHubSmemBuckets * sizeof(uint32_t);
 }
 
 
@@ -803,8 +910,8 @@ __global__ void __launch_bounds__(kChunkThreads) k_hub_chunk(SigArgs a, HubArgs 
   overlap_next();
   overlap_wait();
   extern __shared__ __align__(16) char smem_raw[];
-  ChunkSmem<K, kChunkThreads, kChunkMinHub>& sm = *reinterpret_cast<ChunkSmem<K, kChunkThreads, kChunkMinHub>*>(smem_raw);
-  K* list = reinterpret_cast<K*>(smem_raw + sizeof(ChunkSmem<K, kChunkThreads, kChunkMinHub>));
+  ChunkSmem<K>& sm = *reinterpret_cast<ChunkSmem<K>*>(smem_raw);
+  K* list = reinterpret_cast<K*>(smem_raw + sizeof(ChunkSmem<K>));
   uint32_t* bcnt = reinterpret_cast<uint32_t*>(list + kHubChunk);
   uint32_t* bpos = bcnt + kHubSmemBuckets;
   const uint4 c = h.chunks[blockIdx.x];
@@ -817,7 +924,8 @@ __global__ void __launch_bounds__(kChunkThreads) k_hub_chunk(SigArgs a, HubArgs 
   const uint32_t nb = 1u << bits;
   const bool in_smem = nb <= (uint32_t)kHubSmemBuckets;
   const uint32_t tid = threadIdx.x, lane = tid & 31;
-  chunk_clear(sm, (2 * E + 3) & ~3u);
+  fill_empty<kChunkThreads>(sm.slot, (2 * E + 3) & ~3u, tid);
+  if (tid == 0) sm.cnt = sm.empty = 0;
   if (in_smem)
     for (uint32_t i = tid; i < nb; i += kChunkThreads) bcnt[i] = 0;
   __syncthreads();
@@ -831,16 +939,16 @@ __global__ void __launch_bounds__(kChunkThreads) k_hub_chunk(SigArgs a, HubArgs 
     for (int q = 0; q + 1 < kChunkItems; ++q) key[q] = key[q + 1];
     bool fresh = false;
     if (tid + t * kChunkThreads < E)
-      fresh = kt == KeyOps<K>::kEmpty ? atomicExch(&sm.empty[0], 1u) == 0u : region_insert(sbase, 0u, 2 * E, kt);
+      fresh = kt == KeyOps<K>::kEmpty ? atomicExch(&sm.empty, 1u) == 0u : region_insert(sbase, 0u, 2 * E, kt);
     const unsigned fm = __ballot_sync(kFull, fresh);
     if (fm == 0u) continue;
     uint32_t base = 0;
-    if (lane == 0) base = atomicAdd(&sm.cnt[0], (uint32_t)__popc(fm));
+    if (lane == 0) base = atomicAdd(&sm.cnt, (uint32_t)__popc(fm));
     base = __shfl_sync(kFull, base, 0);
     if (fresh) list[base + __popc(fm & lanes_below(lane))] = kt;
   }
   __syncthreads();
-  const uint32_t U = sm.cnt[0];
+  const uint32_t U = sm.cnt;
   const uint32_t cap = h.hub_cap[hub];
   uint32_t* cur = h.cursor + h.hub_bbase[hub];
   K* tmp = static_cast<K*>(h.tmp) + h.hub_tbase[hub];
@@ -1009,24 +1117,6 @@ __global__ void __launch_bounds__(kChunkThreads) k_hub_scatter(SigArgs a, HubArg
     if (q < cap) tmp[(uint64_t)b * cap + q] = k;
     else hub_fail(a, h, hub, kErrHubOverflow);
   }
-}
-
-// Insert k (!= kEmpty) into a power-of-two set of hmask + 1 slots at
-// shared-window address `base`, home slot from the key's low bits (the keys of
-// one hub bucket share their top bits).  The compare-and-swap is the probe
-// itself: one shared access per probed slot, whether the slot is empty, holds
-// k or holds another key.  Returns 1 if this call inserted k, 0 if k was
-// present, -1 if the set is full.
-template <typename K>
-__device__ __forceinline__ int pow2_insert(uint32_t base, uint32_t hmask, K k) {
-  uint32_t s = key_h32(k) & hmask;
-  for (uint32_t t = 0; t <= hmask; ++t) {
-    const K cur = atoms_cas(base + s * (uint32_t)sizeof(K), KeyOps<K>::kEmpty, k);
-    if (cur == KeyOps<K>::kEmpty) return 1;
-    if (cur == k) return 0;
-    s = (s + 1) & hmask;
-  }
-  return -1;
 }
 
 constexpr int kBucketThreads = 256, kBucketItems = 8;
@@ -2156,17 +2246,10 @@ Status scan64(Store& s, uint64_t* a, uint64_t n, uint64_t* copy) {
   return launch_check("scan64");
 }
 
-template <int NT, int MIN_DEG, typename LabelT, typename K>
-cudaError_t set_chunk_attr() {
-  return cudaFuncSetAttribute(k_sig_chunk<NT, MIN_DEG, LabelT, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(ChunkSmem<K, NT, MIN_DEG>));
-}
-
 template <typename LabelT, typename K>
 cudaError_t set_smem_attrs_label() {
-  cudaError_t e = set_chunk_attr<kSmallChunkThreads, kChunkMin64, LabelT, K>();
-  if (e == cudaSuccess) e = set_chunk_attr<kSmallChunkThreads, kChunkMin1K, LabelT, K>();
-  if (e == cudaSuccess) e = set_chunk_attr<kChunkThreads, kChunkMin4K, LabelT, K>();
+  cudaError_t e = cudaFuncSetAttribute(k_sig_cta<kChunkThreads, LabelT, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)cta_node_smem<kChunkThreads, K>());
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_hub_chunk<LabelT, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)hub_chunk_smem<K>());
@@ -2645,27 +2728,35 @@ Status run_signatures(Store& s, const SigArgs& a, bool defer) {
     launch_if_overlapped(overlapped, s, kernel, blocks, threads, smem, args...);
     overlapped = true;
   };
+  // nodes a warp takes: up to 32 (one lane each), fewer where that would leave
+  // multiprocessors without two full waves of warps
+  auto warp_nodes = [&](auto kernel, uint64_t first, uint64_t count) {
+    const uint32_t per = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(32, count / ((uint64_t)sm_count(s.device) * 128)));
+    run(kernel, grid_for(count, kNodeWarps * per), kNodeWarps * 32, 0, a, first, count, per);
+  };
   {
-    TimedScope ts(s, KBISIM_KERNEL_SIG_SMALL, (n04 ? 1 : 0) + (n5 ? 1 : 0) + (n6 ? 1 : 0) + (s.n_mid_chunks[0] ? 1 : 0));
+    const uint64_t n64 = s.class_start[kClassWarp] - s.class_start[kSmallClasses - 1];
+    TimedScope ts(s, KBISIM_KERNEL_SIG_SMALL, (n04 ? 1 : 0) + (n5 ? 1 : 0) + (n6 ? 1 : 0) + (n64 ? 1 : 0));
     if (n04) run(k_sig_small<0, 4, LabelT, K>, n04, kSmallThreads, 0, a, L04);
     if (n5) run(k_sig_small<5, 5, LabelT, K>, n5, kSmallThreads, 0, a, L5);
     if (n6) run(k_sig_small<6, 6, LabelT, K>, n6, kSmallThreads, 0, a, L6);
-    if (s.n_mid_chunks[0])
-      run(k_sig_chunk<kSmallChunkThreads, kChunkMin64, LabelT, K>, (unsigned)s.n_mid_chunks[0], kSmallChunkThreads,
-          sizeof(ChunkSmem<K, kSmallChunkThreads, kChunkMin64>), a, ptr<uint2>(s.mid_chunks));
+    if (n64) warp_nodes(k_sig_warp<2, LabelT, K>, s.class_start[kSmallClasses - 1], n64);
   }
   if (!(st = launch_check("k_sig_small")).ok()) return st;
-  if (s.n_mid_chunks[1] + s.n_mid_chunks[2]) {
-    TimedScope ts(s, KBISIM_KERNEL_SIG_MEDIUM, (s.n_mid_chunks[1] ? 1 : 0) + (s.n_mid_chunks[2] ? 1 : 0));
-    if (s.n_mid_chunks[1])
-      run(k_sig_chunk<kSmallChunkThreads, kChunkMin1K, LabelT, K>, (unsigned)s.n_mid_chunks[1], kSmallChunkThreads,
-          sizeof(ChunkSmem<K, kSmallChunkThreads, kChunkMin1K>), a, ptr<uint2>(s.mid_chunks) + s.n_mid_chunks[0]);
-    if (s.n_mid_chunks[2])
-      run(k_sig_chunk<kChunkThreads, kChunkMin4K, LabelT, K>, (unsigned)s.n_mid_chunks[2], kChunkThreads,
-          sizeof(ChunkSmem<K, kChunkThreads, kChunkMin4K>), a,
-          ptr<uint2>(s.mid_chunks) + s.n_mid_chunks[0] + s.n_mid_chunks[1]);
+  const uint64_t n256 = s.class_start[kClassWarp2] - s.class_start[kClassWarp];
+  const uint64_t n1k = s.class_start[kClassBlock] - s.class_start[kClassWarp2];
+  const uint64_t n4k = s.class_start[kClassHub] - s.class_start[kClassBlock];
+  if (n256 + n1k + n4k) {
+    TimedScope ts(s, KBISIM_KERNEL_SIG_MEDIUM, (n256 ? 1 : 0) + (n1k ? 1 : 0) + (n4k ? 1 : 0));
+    if (n256) warp_nodes(k_sig_warp<8, LabelT, K>, s.class_start[kClassWarp], n256);
+    if (n1k)
+      run(k_sig_cta<kSmallChunkThreads, LabelT, K>, (unsigned)n1k, kSmallChunkThreads,
+          cta_node_smem<kSmallChunkThreads, K>(), a, s.class_start[kClassWarp2]);
+    if (n4k)
+      run(k_sig_cta<kChunkThreads, LabelT, K>, (unsigned)n4k, kChunkThreads, cta_node_smem<kChunkThreads, K>(), a,
+          s.class_start[kClassBlock]);
   }
-  if (!(st = launch_check("k_sig_chunk")).ok()) return st;
+  if (!(st = launch_check("k_sig_warp")).ok()) return st;
   if (s.n_hub) {
     if (!s.tune_now) return defer ? launch_hubs<LabelT, K>(s, a, true) : run_hubs<LabelT, K>(s, a);
     // tuning (once per handle, on a full round from level 2 on): each bucket
@@ -2817,19 +2908,9 @@ Status restore_hub_growth(Store& s, const HubGrowth& g, bool same_degree) {
 // ---------------------------------------------------------------------------
 // Relabelling and degree classes (once per graph)
 // ---------------------------------------------------------------------------
-// Work lists made from the offsets of the degree classes: hub chunks and the
-// hubs' bucket layout, and the chunks of whole nodes for out-degree 33..4096.
+// Work lists made from the hubs' offsets: their chunks and bucket layout.
 // `fresh`: a new graph (bucket growth learned on the previous one is dropped).
-// Offsets of the out-degree 33..4096 nodes, copied to the host for the chunk
-// plan, and the class bounds they cover.
-struct MidPlan {
-  std::vector<uint64_t> moff;
-  uint64_t mf = 0, mw = 0, mb = 0, me = 0;
-};
-
-// Hub chunk lists and layout, and the copy of the offsets the chunk plan of
-// the out-degree 33..4096 nodes needs (made with the hub offsets' copy).
-Status chunk_lists_hubs(Store& s, bool fresh, MidPlan* mp) {
+Status build_chunk_lists(Store& s, bool fresh) {
   Status st;
   // hubs: a contiguous internal id range; their offsets come in one copy
   s.n_hub = s.class_start[kClassHub + 1] - s.class_start[kClassHub];
@@ -2879,68 +2960,8 @@ Status chunk_lists_hubs(Store& s, bool fresh, MidPlan* mp) {
     if (!st.ok()) return st;
     if (!(st = hub_layout(s)).ok()) return st;
   }
-  // the out-degree 33..4096 nodes' offsets for their chunk plan
-  mp->mf = s.class_start[kSmallClasses - 1];
-  mp->mw = s.class_start[kClassWarp];
-  mp->mb = s.class_start[kClassBlock];
-  mp->me = s.class_start[kClassHub];
-  mp->moff.clear();
-  if (mp->me > mp->mf) {
-    mp->moff.resize(mp->me - mp->mf + 1);
-    st = cuda_check(cudaMemcpyAsync(mp->moff.data(), ptr<uint64_t>(s.offsets) + mp->mf,
-                                    (mp->me - mp->mf + 1) * 8, cudaMemcpyDeviceToHost, s.stream),
-                    "chunk offsets");
-    if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "sync");
-    if (!st.ok()) return st;
-  }
   return Status::Ok();
 }
-
-// out-degree 33..4096: runs of whole nodes; 33..64 and 65..1024 in chunks
-// of at most 1024 edges (128-thread CTAs), 1025..4096 in chunks of at most
-// 4096 edges (512-thread CTAs).  A host loop over the nodes' offsets (about
-// 2 ms for 640K nodes), so a load runs it while the GPU relabels the edges.
-Status chunk_lists_mid(Store& s, const MidPlan& mp) {
-  Status st;
-  s.n_mid_chunks[0] = s.n_mid_chunks[1] = s.n_mid_chunks[2] = 0;
-  const uint64_t mf = mp.mf, mw = mp.mw, mb = mp.mb, me = mp.me;
-  if (me > mf) {
-    const std::vector<uint64_t>& moff = mp.moff;
-    std::vector<uint2> mc;
-    mc.reserve((size_t)((moff[me - mf] - moff[0]) / 512 + (me - mf) / 16 + 16));
-    auto pack = [&](uint64_t lo, uint64_t hi, uint64_t max_edges, uint64_t max_nodes) {
-      for (uint64_t i = lo; i < hi;) {
-        uint64_t j = i + 1;
-        while (j < hi && j - i < max_nodes && moff[j + 1] - moff[i] <= max_edges) ++j;
-        mc.push_back(make_uint2((uint32_t)(mf + i), (uint32_t)(j - i)));
-        i = j;
-      }
-    };
-    using S64 = ChunkShape<kSmallChunkThreads, kChunkMin64>;
-    using S1K = ChunkShape<kSmallChunkThreads, kChunkMin1K>;
-    using S4K = ChunkShape<kChunkThreads, kChunkMin4K>;
-    pack(0, mw - mf, S64::kEdges, S64::kMaxNodes);
-    s.n_mid_chunks[0] = mc.size();
-    pack(mw - mf, mb - mf, S1K::kEdges, S1K::kMaxNodes);
-    s.n_mid_chunks[1] = mc.size() - s.n_mid_chunks[0];
-    pack(mb - mf, me - mf, S4K::kEdges, S4K::kMaxNodes);
-    s.n_mid_chunks[2] = mc.size() - s.n_mid_chunks[0] - s.n_mid_chunks[1];
-    if (!(st = ensure(s, s.mid_chunks, mc.size() * sizeof(uint2))).ok()) return st;
-    st = cuda_check(cudaMemcpyAsync(s.mid_chunks.p, mc.data(), mc.size() * sizeof(uint2), cudaMemcpyHostToDevice,
-                                    s.stream), "medium chunks");
-    if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "sync");  // mc is freed on return
-    if (!st.ok()) return st;
-  }
-  return Status::Ok();
-}
-
-Status build_chunk_lists(Store& s, bool fresh) {
-  MidPlan mp;
-  Status st = chunk_lists_hubs(s, fresh, &mp);
-  if (st.ok()) st = chunk_lists_mid(s, mp);
-  return st;
-}
-
 
 Status scan_u64(Store& s, uint64_t* a, uint64_t n) { return scan64(s, a, n, nullptr); }
 
@@ -2997,8 +3018,7 @@ Status relabel_graph(Store& s, const uint64_t* off0, const uint32_t* dst0, const
   if (!st.ok()) return st;
   if (!(st = scan64(s, ptr<uint64_t>(s.offsets), n + 1, nullptr)).ok()) return st;
   s.n_alone = 0;
-  MidPlan mp;
-  if (!(st = chunk_lists_hubs(s, true, &mp)).ok()) return st;
+  if (!(st = build_chunk_lists(s, true)).ok()) return st;
   // the edge labels (and with them the label width) from here on
   if (s.await_labels && !(st = s.await_labels(s)).ok()) return st;
   if (!(st = ensure(s, s.elabel, std::max<uint64_t>(1, m) * (s.label8 ? 1 : 4))).ok()) return st;
@@ -3015,8 +3035,6 @@ Status relabel_graph(Store& s, const uint64_t* off0, const uint32_t* dst0, const
     }
   }
   st = launch_check("relabel edges");
-  // the medium chunk plan on the host while the GPU relabels the edges
-  if (st.ok()) st = chunk_lists_mid(s, mp);
   if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "sync");
   return st;
 }
@@ -3247,6 +3265,7 @@ Status compute_round(Store& s, uint32_t i) {
   a.mask = s.hash_mask;
   a.err = ptr<uint32_t>(s.d_err);
   a.fmask = s.round_mask;
+  a.alone = ptr<uint8_t>(s.alone);
   // 32-bit signature words when (label, child id) fits in 32 bits
   const uint32_t pbits = bits_for(s.counts[i - 1] ? s.counts[i - 1] - 1 : 0);
   const bool key64 = pbits + s.label_bits > 32;
@@ -3319,6 +3338,7 @@ Status masked_signatures(Store& s, const uint32_t* prev, const uint32_t* fmask) 
   a.mask = s.hash_mask;
   a.err = ptr<uint32_t>(s.d_err);
   a.fmask = fmask;
+  a.alone = nullptr;
   if (s.mt.key32) {  // labels below 2^pbits (the stores' width)
     a.pbits = (int)s.mt.pbits;
     return s.label8 ? run_signatures<uint8_t, uint32_t>(s, a, false) : run_signatures<uint32_t, uint32_t>(s, a, false);

@@ -71,3 +71,50 @@ def test_frontier_groups_equal_new_signatures(width):
         ref = oracle.kbisim(g.num_nodes, g.node_label, src, dst, lab, 2)
         assert res.counts == ref.counts.tolist()
         assert np.array_equal(kb.all_pids(2), ref.pids)
+
+
+def _degree_graph(degrees, marker, wide, seed):
+    """Nodes of the given out-degrees over 2^11 targets that are blocks of their own at level 0, with repeated
+    elements.  `marker`: every other node also holds, twice, the element whose 32-bit word marks an empty slot."""
+    rng = np.random.default_rng(seed)
+    nt, pbits = 1 << 11, 11
+    degrees = np.repeat(degrees, 3)
+    packed = (0xFFFF0000 * pow(0x9E3779B1, -1, 1 << 32)) % (1 << 32)  # its word is all ones
+    src, dst, lab = [], [], []
+    for j, d in enumerate(degrees):
+        t = rng.integers(0, nt, d)
+        l = rng.integers(0, 3, d)
+        if marker and j % 2 and d >= 2:
+            t[:2], l[:2] = packed & (nt - 1), packed >> pbits
+        if j % 3 == 1:  # the same set as the node before, in another order
+            d0 = degrees[j - 1]
+            p = rng.permutation(d0)
+            t, l = dst[-1][p], lab[-1][p]
+        src.append(np.full(t.size, nt + j)), dst.append(t), lab.append(l)
+    src, dst, lab = (np.concatenate(x).astype(np.uint64) for x in (src, dst, lab))
+    if wide:
+        lab[0] = 0xFFFFFFFF
+    # nodes: targets first, labels 0..nt-1; the others reuse labels, so level 0 has 2^11 blocks
+    nlab = np.concatenate([np.arange(nt), np.full(degrees.size, 7)])
+    return synth.from_coo(nt + degrees.size, src, dst, lab.astype(np.uint32), nlab)
+
+
+@pytest.mark.parametrize("marker,wide", [(False, False), (True, False), (False, True)])
+def test_signatures_at_degree_class_edges(marker, wide):
+    """Out-degrees on both sides of every change of kernel and of steps within one."""
+    edges = [1, 2, 4, 8, 16, 32, 64, 96, 128, 160, 256, 512, 1024, 2048, 4096]
+    degrees = sorted({d + x for d in edges for x in (-1, 0, 1) if d + x > 0})
+    g = _degree_graph(degrees, marker, wide, seed=17)
+    with KBisim() as kb:
+        res = kb.build(g, 3)
+        assert_same(res, kb.all_pids(3), oracle_levels(g, 3))
+        assert [kb.round_stats(1)[f] for f in ("unique_keys", "max_signature")] == _set_sizes(g, kb.pids(0))
+        # level 2: most nodes are alone in their block by then
+        assert [kb.round_stats(2)[f] for f in ("unique_keys", "max_signature")] == _set_sizes(g, kb.pids(1))
+
+
+def _set_sizes(g, prev):
+    key = np.unique(np.stack([g.src().astype(np.uint64), g.edge_label.astype(np.uint64), prev[g.dst].astype(np.uint64)]),
+                    axis=1)
+    per = np.bincount(key[0].astype(np.int64))
+    return [int(per.sum()), int(per.max())]
