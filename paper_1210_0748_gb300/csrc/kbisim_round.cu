@@ -676,6 +676,17 @@ __device__ __forceinline__ void sig_one_node(const SigArgs& a, uint64_t e0, uint
   K* out = static_cast<K*>(a.sigkey) + e0;
   uint32_t u = 0, l = 0, h = 0;
   bool seen_empty = false;
+  if (alone) {  // only the number of distinct keys is needed
+#pragma unroll
+    for (int t = 0; t < STEPS; ++t) {
+      const K k = key[t];
+      if (lane + 32u * t >= d) continue;
+      if (k != KeyOps<K>::kEmpty) u += pow2_insert(sbase, 64u * STEPS - 1, k) > 0 ? 1u : 0u;
+      else seen_empty = true;
+    }
+    U = __reduce_add_sync(kFull, u) + (__any_sync(kFull, seen_empty) ? 1u : 0u);
+    return;
+  }
 #pragma unroll
   for (int t = 0; t < STEPS; ++t) {
     if (STEPS > 2 && 32u * t >= d) break;
@@ -689,7 +700,7 @@ __device__ __forceinline__ void sig_one_node(const SigArgs& a, uint64_t e0, uint
       seen_empty = true;
     }
     const unsigned fm = __ballot_sync(kFull, fresh);
-    if (!alone && fresh) {
+    if (fresh) {
       out[u + __popc(fm & lanes_below(lane))] = k;
       const uint64_t tm = elem_term(k, a.seed);
       l += (uint32_t)tm;
@@ -698,11 +709,8 @@ __device__ __forceinline__ void sig_one_node(const SigArgs& a, uint64_t e0, uint
     u += __popc(fm);
   }
   U = u;
-  if (!alone) {
-    lo = __reduce_add_sync(kFull, l);
-    hi = __reduce_add_sync(kFull, h);
-  }
-  __syncwarp();  // the set is cleared for the next node only after every insert
+  lo = __reduce_add_sync(kFull, l);
+  hi = __reduce_add_sync(kFull, h);
 }
 
 template <int MAXSTEPS, typename LabelT, typename K>
@@ -784,6 +792,21 @@ __device__ __forceinline__ void sig_cta_node(const SigArgs& a, uint64_t p, uint6
   fill_empty<NT>(sm.set(), kSlots, tid);
   __syncthreads();
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sm.set());
+  if (alone) {  // only the number of distinct keys is needed
+    uint32_t c = 0;
+#pragma unroll
+    for (int t = 0; t < ITEMS; ++t) {
+      if (tid + (uint32_t)t * NT >= d) continue;
+      const K k = key[t];
+      c += k == KeyOps<K>::kEmpty ? (atomicExch(&sm.empty, 1u) == 0u ? 1u : 0u)
+                                  : (pow2_insert(sbase, kSlots - 1, k) > 0 ? 1u : 0u);
+    }
+    c = __reduce_add_sync(kFull, c);
+    if (lane == 0) atomicAdd(&sm.cnt, c);
+    __syncthreads();
+    if (tid == 0) a.ucnt[p] = sm.cnt;
+    return;
+  }
   unsigned fms[ITEMS];
   uint32_t lo = 0, hi = 0, total = 0;
 #pragma unroll
@@ -796,15 +819,13 @@ __device__ __forceinline__ void sig_cta_node(const SigArgs& a, uint64_t p, uint6
       fresh = k == KeyOps<K>::kEmpty ? atomicExch(&sm.empty, 1u) == 0u : pow2_insert(sbase, kSlots - 1, k) > 0;
     fms[t] = __ballot_sync(kFull, fresh);
     total += __popc(fms[t]);
-    if (!alone && fresh) {
+    if (fresh) {
       const uint64_t tm = elem_term(k, a.seed);
       lo += (uint32_t)tm;
       hi += (uint32_t)(tm >> 32);
     }
   }
-  if (alone) {
-    if (lane == 0) atomicAdd(&sm.cnt, total);
-  } else if (total) {
+  if (total) {
     uint32_t at = 0;
     if (lane == 0) at = atomicAdd(&sm.cnt, total);
     at = __shfl_sync(kFull, at, 0);
@@ -824,7 +845,7 @@ __device__ __forceinline__ void sig_cta_node(const SigArgs& a, uint64_t p, uint6
   __syncthreads();
   if (tid == 0) {
     a.ucnt[p] = sm.cnt;
-    if (!alone) a.hash[p] = node_hash(((uint64_t)sm.hi << 32) | sm.lo, a.prev[p], sm.cnt, a.seed, a.mask);
+    a.hash[p] = node_hash(((uint64_t)sm.hi << 32) | sm.lo, a.prev[p], sm.cnt, a.seed, a.mask);
   }
 }
 
@@ -841,7 +862,7 @@ __device__ __forceinline__ void sig_cta_block(const SigArgs& a, uint64_t first) 
 }
 
 template <int NT, typename LabelT, typename K>
-__global__ void __launch_bounds__(NT) k_sig_cta(SigArgs a, uint64_t first) {
+__global__ void __launch_bounds__(NT, sizeof(K) == 4 ? 2048 / NT : 1536 / NT) k_sig_cta(SigArgs a, uint64_t first) {
   overlap_next();
   sig_cta_block<NT, LabelT, K>(a, first);
   overlap_wait();
@@ -1146,6 +1167,7 @@ __global__ void __launch_bounds__(kBucketThreads, sizeof(K) == 4 ? 6 : 3) k_hub_
   // loaded one bucket ahead, so that their latency overlaps the work on the
   // bucket before
   uint32_t nx_hub = 0, nx_n = 0;
+  bool nx_alone = false;
   const K* nx_tmp = nullptr;
   K kk[kBucketItems];
   auto fetch = [&](uint64_t bb) {
@@ -1153,6 +1175,7 @@ __global__ void __launch_bounds__(kBucketThreads, sizeof(K) == 4 ? 6 : 3) k_hub_
     const uint32_t cap = h.hub_cap[nx_hub];
     nx_tmp = static_cast<const K*>(h.tmp) + h.hub_tbase[nx_hub] + (bb - h.hub_bbase[nx_hub]) * cap;
     nx_n = min(h.cursor[bb], cap);
+    nx_alone = a.alone && a.alone[h.first + nx_hub];
 #pragma unroll
     for (int t = 0; t < kBucketItems; ++t) {
       const uint32_t i = tid + t * kBucketThreads;
@@ -1162,6 +1185,7 @@ __global__ void __launch_bounds__(kBucketThreads, sizeof(K) == 4 ? 6 : 3) k_hub_
   if (blockIdx.x < n_buckets) fetch(blockIdx.x);
   for (uint64_t b = blockIdx.x; b < n_buckets; b += gridDim.x) {
     const uint32_t hub = nx_hub, n = nx_n;
+    const bool alone = nx_alone;  // only the number of distinct keys is needed
     const uint64_t p = h.first + hub;
     const K* tmp = nx_tmp;
     if (n == 0) {  // nothing appended (a hub outside a frontier mask): no barrier, no output
@@ -1191,6 +1215,25 @@ __global__ void __launch_bounds__(kBucketThreads, sizeof(K) == 4 ? 6 : 3) k_hub_
           const uint32_t i = i0 + tid + t * kBucketThreads;
           kk[t] = i < n ? tmp[i] : (K)0;
         }
+      }
+      if (alone) {
+        uint32_t c = 0;
+#pragma unroll
+        for (int t = 0; t < kBucketItems; ++t) {
+          const uint32_t i = i0 + tid + t * kBucketThreads;
+          const K k = kk[t];
+          if (i >= n) continue;
+          if (k == KeyOps<K>::kEmpty) {
+            c += atomicExch(&sm.empty, 1u) == 0u ? 1u : 0u;
+          } else {
+            const int r = pow2_insert(sbase, hcap - 1, k);
+            c += r > 0 ? 1u : 0u;
+            if (r < 0) sm.full = 1u;
+          }
+        }
+        c = __reduce_add_sync(kFull, c);
+        if (lane == 0) atomicAdd(&sm.lo, c);
+        continue;
       }
       // the keys of kBucketItems steps are inserted first; then the warp
       // takes the places of all its fresh keys with one reservation on the
@@ -1243,8 +1286,13 @@ __global__ void __launch_bounds__(kBucketThreads, sizeof(K) == 4 ? 6 : 3) k_hub_
     __syncthreads();
     if (tid == 0) {
       if (sm.full) hub_fail(a, h, hub, kErrHubSet);  // more distinct keys than the set holds: the host adds buckets
-      atomicAdd(&h.hub_term[2 * hub], sm.lo);      // (a failed hub's sums are cleared before its repeat)
-      atomicAdd(&h.hub_term[2 * hub + 1], sm.hi);
+      // (a failed hub's sums are cleared before its repeat)
+      if (alone) {
+        atomicAdd(hcur, (unsigned long long)sm.lo);
+      } else {
+        atomicAdd(&h.hub_term[2 * hub], sm.lo);
+        atomicAdd(&h.hub_term[2 * hub + 1], sm.hi);
+      }
     }
     // no barrier here: thread 0 alone reads the bucket's totals, and the next
     // bucket's first barrier comes before anything is written to them again
