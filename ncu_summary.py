@@ -35,7 +35,7 @@ CLASS_OF = [
     (r"k_sig_small|k_sig_warp<2,|k_sig_chunk<128, 33,", "sig_small"),  # the library times out-degree 33..64 with <= 32
     (r"k_sig_warp|k_sig_cta|k_sig_chunk", "sig_medium"),
     (r"k_hub_sample|k_hub_chunk|k_hub_scatter|k_hub_bucket|k_hub_finish", "sig_hub"),
-    (r"k_group_insert", "group"),
+    (r"k_group_insert|k_group_filter|k_group_select|k_table_clear", "group"),
     (r"k_group_verify|k_verify_long", "verify"),
     (r"k_head_ranks|k_word_counts|k_tile_sum64|k_scan_tiles|k_tile_scan64|k_pid_fill|k_l0_fill", "renumber"),
 ]

@@ -1332,13 +1332,25 @@ struct GroupArgs {
   uint32_t* err;
   const uint8_t* alone;  // nodes alone in their previous block (may be null): heads, not grouped
   int read_first;        // few distinct hashes shared by many nodes (level 0): read a slot before any atomic
+  // number of listed nodes on the device (NULL = the launch's count); the table
+  // then has table_slots of it
+  const unsigned long long* d_count;
+  uint2* seen;           // filter: per 32 bits, (hash seen, hash seen twice); NULL = no filter
+  uint64_t seen_mask;    // bits - 1
 };
 
-__device__ __forceinline__ uint32_t table_insert(const GroupArgs& g, uint64_t h, uint32_t minid) {
+// Slots of a table for n nodes: a power of two, at most half full.
+__host__ __device__ __forceinline__ uint64_t table_slots(uint64_t n) {
+  uint64_t c = 1024;
+  while (c < 2 * n) c <<= 1;
+  return c;
+}
+
+__device__ __forceinline__ uint32_t table_insert(const GroupArgs& g, uint64_t tmask, uint64_t h, uint32_t minid) {
   const unsigned long long fp = (unsigned long long)(uint32_t)(h >> 32);
   const unsigned long long v = (fp << 32) | minid;
-  uint32_t s = (uint32_t)(mix64(h) & g.tmask);
-  for (uint64_t t = 0; t <= g.tmask; ++t) {
+  uint32_t s = (uint32_t)(mix64(h) & tmask);
+  for (uint64_t t = 0; t <= tmask; ++t) {
     // a slot already holding this fingerprint with an id no larger needs no atomic
     if (g.read_first) {
       const unsigned long long seen = *(volatile unsigned long long*)&g.table[s];
@@ -1350,7 +1362,7 @@ __device__ __forceinline__ uint32_t table_insert(const GroupArgs& g, uint64_t h,
       if ((uint32_t)cur > minid) atomicMin(&g.table[s], v);
       return s;
     }
-    s = (uint32_t)((s + 1) & g.tmask);
+    s = (uint32_t)((s + 1) & tmask);
   }
   atomicOr(g.err, kErrProbe);
   return 0;
@@ -1363,6 +1375,8 @@ constexpr int kInsThreads = 256, kInsItems = 4, kInsChunk = kInsThreads * kInsIt
 __global__ void __launch_bounds__(kInsThreads) k_group_insert(GroupArgs g, const uint32_t* list, uint64_t count) {
   overlap_next();
   overlap_wait();
+  if (g.d_count) count = *g.d_count;
+  const uint64_t tmask = g.d_count ? table_slots(count) - 1 : g.tmask;
   __shared__ unsigned long long skey[kInsSlots];
   __shared__ unsigned int smin[kInsSlots];
   __shared__ unsigned int sglob[kInsSlots];
@@ -1422,7 +1436,7 @@ __global__ void __launch_bounds__(kInsThreads) k_group_insert(GroupArgs g, const
     const uint32_t nu = n_used;
     for (uint32_t i = threadIdx.x; i < nu; i += kInsThreads) {
       const uint32_t sl = used[i];
-      sglob[sl] = table_insert(g, skey[sl], smin[sl]);
+      sglob[sl] = table_insert(g, tmask, skey[sl], smin[sl]);
     }
     __syncthreads();
 #pragma unroll
@@ -1490,6 +1504,115 @@ __device__ __forceinline__ void mark_member(const VerifyArgs& v, uint32_t r) {
   if (!*(volatile uint8_t*)&v.member[r]) v.member[r] = 1;
 }
 
+// Filter before the table, when the table would not stay in L2.  Where blocks
+// are small most hashes occur once, and a node alone with its hash is a head
+// that needs neither the table nor a comparison.  One pass notes every hash in
+// a bitmap of 8 to 16 bits per node, and in a second one the hashes met before;
+// the next pass settles the nodes whose bit was met once and lists the others
+// (those that share a hash, and one node in 16 to 8 by chance) for the grouping,
+// whose table is sized for them.
+// 16M random accesses cost 0.43 ms as compare-and-swaps in a table of 256 MB
+// and 0.25 ms as its loads, 0.14 and 0.07 ms in 32 MB.  Grouping and comparison
+// of the 16M-node powerlaw graph's four rounds: 1.95 -> 1.55 ms; 25.6M nodes of
+// the alpha = 2.0 one, five rounds: 5.2 -> 4.7 ms.  Up to 4M nodes the table
+// is as cheap (64 MB) and the two passes only cost.
+constexpr uint64_t kFilterNodes = 4u << 20;  // table above 64 MB
+constexpr int kFilThreads = 256, kFilItems = 4, kFilTile = kFilThreads * kFilItems;
+
+__device__ __forceinline__ uint64_t filter_bit(const GroupArgs& g, uint64_t h) { return (mix64(h) >> 32) & g.seen_mask; }
+
+__global__ void __launch_bounds__(kFilThreads) k_group_filter(GroupArgs g, uint64_t count) {
+  overlap_next();
+  overlap_wait();
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint64_t base = (uint64_t)blockIdx.x * kFilTile; base < count; base += (uint64_t)gridDim.x * kFilTile) {
+    uint64_t b[kFilItems];
+    bool act[kFilItems];
+    uint2 w[kFilItems];
+#pragma unroll
+    for (int t = 0; t < kFilItems; ++t) {
+      const uint64_t p = base + threadIdx.x + (uint64_t)t * kFilThreads;
+      act[t] = p < count && !(g.alone && g.alone[p]);
+      b[t] = act[t] ? filter_bit(g, g.hash[p]) : ~0ull;
+    }
+    // bits only get set, so a stale word can only cost an atomic
+#pragma unroll
+    for (int t = 0; t < kFilItems; ++t)
+      w[t] = act[t] ? g.seen[b[t] >> 5] : make_uint2(0u, 0u);
+#pragma unroll
+    for (int t = 0; t < kFilItems; ++t) {
+      // of a run of lanes with one hash, the first notes it as seen and the
+      // second as seen twice
+      const bool run = __shfl_up_sync(kFull, b[t], 1) == b[t] && lane > 0;
+      const bool rest = __shfl_up_sync(kFull, (uint32_t)run, 1) != 0u && lane > 0 && run;
+      if (!act[t] || rest) continue;
+      const uint32_t bit = 1u << (b[t] & 31);
+      uint2* at = &g.seen[b[t] >> 5];
+      if (w[t].y & bit) continue;
+      if (run || (w[t].x & bit) || (atomicOr(&at->x, bit) & bit)) atomicOr(&at->y, bit);
+    }
+  }
+}
+
+// Nodes alone in their previous block or with their hash: heads.  The others
+// are listed (a CTA takes its places together).
+__global__ void __launch_bounds__(kFilThreads) k_group_select(GroupArgs g, VerifyArgs v, uint64_t count, uint32_t* list,
+                                                              unsigned long long* n_list) {
+  overlap_next();
+  overlap_wait();
+  __shared__ uint32_t n_cta;
+  __shared__ unsigned long long at_cta;
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint64_t base = (uint64_t)blockIdx.x * kFilTile; base < count; base += (uint64_t)gridDim.x * kFilTile) {
+    if (threadIdx.x == 0) n_cta = 0;
+    __syncthreads();
+    uint32_t o[kFilItems], at[kFilItems];
+    uint64_t h[kFilItems];
+    bool act[kFilItems], cand[kFilItems];
+#pragma unroll
+    for (int t = 0; t < kFilItems; ++t) {
+      const uint64_t p = base + threadIdx.x + (uint64_t)t * kFilThreads;
+      act[t] = p < count;
+      cand[t] = act[t] && !(g.alone && g.alone[p]);
+      if (act[t]) o[t] = g.p2o[p];
+      if (cand[t]) h[t] = g.hash[p];
+    }
+#pragma unroll
+    for (int t = 0; t < kFilItems; ++t) {
+      if (cand[t]) {
+        const uint64_t b = filter_bit(g, h[t]);
+        cand[t] = (__ldcg(&g.seen[b >> 5].y) >> (b & 31)) & 1u;
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < kFilItems; ++t) {
+      const unsigned m = __ballot_sync(kFull, cand[t]);
+      uint32_t q = 0;
+      if (lane == 0 && m) q = atomicAdd(&n_cta, (uint32_t)__popc(m));
+      at[t] = __shfl_sync(kFull, q, 0) + __popc(m & lanes_below(lane));
+      if (act[t] && !cand[t]) {
+        g.rep[base + threadIdx.x + (uint64_t)t * kFilThreads] = (uint32_t)(base + threadIdx.x + (uint64_t)t * kFilThreads);
+        mark_head(v, o[t]);
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && n_cta) at_cta = atomicAdd(n_list, (unsigned long long)n_cta);
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < kFilItems; ++t)
+      if (cand[t]) list[at_cta + at[t]] = (uint32_t)(base + threadIdx.x + (uint64_t)t * kFilThreads);
+    __syncthreads();  // the CTA's count and place are read before the next tile's
+  }
+}
+
+__global__ void __launch_bounds__(kFilThreads) k_table_clear(GroupArgs g) {
+  overlap_next();
+  overlap_wait();
+  const uint64_t units = table_slots(*g.d_count) / 2;  // 16 bytes
+  for (uint64_t u = blockIdx.x * (uint64_t)kFilThreads + threadIdx.x; u < units; u += (uint64_t)gridDim.x * kFilThreads)
+    reinterpret_cast<uint4*>(g.table)[u] = make_uint4(~0u, ~0u, ~0u, ~0u);
+}
+
 constexpr int kMarkSeen = 256;  // heads a verification CTA remembers as marked
 
 __device__ __forceinline__ void mark_unresolved(const VerifyArgs& v, uint32_t* rep, uint32_t p) {
@@ -1508,6 +1631,7 @@ __global__ void __launch_bounds__(kVerNodeThreads) k_group_verify(GroupArgs g, V
                                                                    uint64_t count) {
   overlap_next();
   overlap_wait();
+  if (g.d_count) count = *g.d_count;
   // heads this CTA has marked as having members: a block of millions of
   // nodes (level 0) then costs one global access per CTA, not per member
   __shared__ uint32_t seen[kMarkSeen];
@@ -2362,11 +2486,7 @@ Status check_below(Store& s, const uint32_t* a, uint64_t n, uint64_t bound, cons
   return checked_outcome(s, what);
 }
 
-uint64_t table_capacity(uint64_t n) {
-  uint64_t c = 1024;
-  while (c < 2 * n) c <<= 1;
-  return c;
-}
+uint64_t table_capacity(uint64_t n) { return table_slots(n); }
 
 void launch_insert(Store& s, const GroupArgs& g, const uint32_t* list, uint64_t count) {
   static int cached[64];
@@ -2448,6 +2568,9 @@ GroupArgs group_args(Store& s, uint64_t slots) {
   g.err = ptr<uint32_t>(s.d_err);
   g.alone = nullptr;
   g.read_first = 0;
+  g.d_count = nullptr;
+  g.seen = nullptr;
+  g.seen_mask = 0;
   return g;
 }
 
@@ -2473,16 +2596,23 @@ VerifyArgs verify_args(Store& s, int mode, const uint32_t* prev, bool key64) {
   return v;
 }
 
+// Bits of the filter before the grouping of `ins` nodes (0 = none): 8 to 16 per
+// node, two bitmaps, so at most 4 of the 8 bytes per node of the pair lists,
+// which nothing uses before the comparison.
+uint64_t filter_bits(uint64_t ins) { return ins > kFilterNodes ? 4 * table_slots(ins) : 0; }
+
 // Clear what a level's signatures and grouping start from: error flags,
 // scalars, the marks of the canonical numbering, the hash table for `ins`
-// inserted nodes, and, with hubs, their buckets' cursors and totals.
-Status clear_round(Store& s, uint64_t ins, bool hubs) {
+// inserted nodes or the filter before it, and, with hubs, their buckets'
+// cursors and totals.
+Status clear_round(Store& s, uint64_t ins, bool filter, bool hubs) {
   ClearArgs c;
   c.add(s.d_err.p, 16, 0u);
   c.add(s.d_scalars.p, 16 * 8, 0u);
   c.add(s.hbits.p, (s.n + 31) / 32 * 4, 0u);
   c.add(s.member.p, s.n, 0u);
-  c.add(s.table.p, group_slots(s, ins) * 8, ~0u);
+  if (filter && filter_bits(ins)) c.add(s.long_pairs.p, filter_bits(ins) / 4, 0u);
+  else c.add(s.table.p, group_slots(s, ins) * 8, ~0u);
   if (hubs) {
     c.add(s.hub_cursor.p, s.n_hub_buckets * 4, 0u);
     c.add(s.hub_acc.p, s.n_hub * 24, 0u);
@@ -2514,7 +2644,8 @@ uint64_t insert_count(const Store& s, bool use_alone) {
 //  [1] unresolved after the first pass, [2] key total, [3] largest signature,
 //  [4] collided nodes, [5] unresolved after a repair pass, [6] and [10] pairs
 //  with long and with middle signatures, [7] error flags copy, [8] nodes alone
-//  in their block, [9] ticket of k_head_ranks, [15] the number of blocks.
+//  in their block, [9] ticket of k_head_ranks, [11] nodes the filter left to
+//  the grouping, [15] the number of blocks.
 Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint32_t* pid, uint64_t* blocks,
                       uint64_t* collided, bool with_stats, uint64_t* keys, uint64_t* maxsig, bool use_alone,
                       uint32_t* hub_flags) {
@@ -2553,14 +2684,34 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
                       kFillThreads, 0, r);
     return launch_check("renumber");
   };
+  const uint64_t bits = mode ? filter_bits(insert_count(s, use_alone)) : 0;
   if (na) {
+    const uint32_t* list = nullptr;
     {
-      TimedScope ts(s, KBISIM_KERNEL_GROUP, 1);
-      launch_insert(s, g, nullptr, na);
+      TimedScope ts(s, KBISIM_KERNEL_GROUP, bits ? 4 : 1);
+      if (bits) {
+        uint32_t* cand = ptr<uint32_t>(s.ulist[1]);
+        static int cf[64], cs[64];
+        g.seen = ptr<uint2>(s.long_pairs);
+        g.seen_mask = bits - 1;
+        const uint64_t tiles = grid_for(na, kFilTile);
+        launch_chained(s, k_group_filter,
+                       (unsigned)std::min<uint64_t>(tiles, resident_grid(k_group_filter, kFilThreads, 0, s.device, cf)),
+                       kFilThreads, 0, g, na);
+        launch_chained(s, k_group_select,
+                       (unsigned)std::min<uint64_t>(tiles, resident_grid(k_group_select, kFilThreads, 0, s.device, cs)),
+                       kFilThreads, 0, g, v, na, cand, sc + 11);
+        list = cand;
+        g.alone = nullptr;  // none of the listed nodes is
+        g.d_count = sc + 11;
+        launch_chained(s, k_table_clear, (unsigned)sm_count(s.device) * 8, kFilThreads, 0, g);
+      }
+      launch_insert(s, g, list, na);
     }
     if (!(st = launch_check("k_group_insert")).ok()) return st;
     TimedScope ts(s, KBISIM_KERNEL_VERIFY, mode ? 2 : 1);
-    if (!(st = launch_verify(s, g, v, nullptr, na)).ok()) return st;
+    if (!(st = launch_verify(s, g, v, list, na)).ok()) return st;
+    g.d_count = nullptr;
   }
   if (s.checked) {  // representatives are checked before the numbering uses them
     if (!(st = read_scalars(s, h)).ok()) return st;
@@ -3246,7 +3397,7 @@ Status compute_level0(Store& s) {
   if (done) return Status::Ok();
   const int sms = sm_count(s.device);
   const unsigned blocks = (unsigned)std::min<uint64_t>(grid_for(s.n_alive, 256), (uint64_t)sms * 16);
-  if (!(st = clear_round(s, s.n_alive, false)).ok()) return st;
+  if (!(st = clear_round(s, s.n_alive, false, false)).ok()) return st;
   {
     TimedScope ts(s, KBISIM_KERNEL_LABEL_GROUP, s.n_alive ? 1 : 0);
     if (s.n_alive)
@@ -3299,7 +3450,7 @@ Status compute_round(Store& s, uint32_t i) {
     return Status::Err(KBISIM_ERR_TIMEOUT, "injected timeout (KBISIM_FAULT_TIMEOUT_ROUND)");
   Status st = ensure_round_scratch(s);
   if (!st.ok()) return st;
-  if (!(st = clear_round(s, insert_count(s, true), s.n_hub != 0)).ok()) return st;
+  if (!(st = clear_round(s, insert_count(s, true), true, s.n_hub != 0)).ok()) return st;
   if (s.checked && !(st = check_round_inputs(s, i)).ok()) return st;
   SigArgs a;
   a.off = ptr<uint64_t>(s.offsets);
@@ -3354,7 +3505,7 @@ Status compute_round(Store& s, uint32_t i) {
     if (!hub_flags) break;
     if (attempt >= kHubAttempts) return Status::Err(KBISIM_ERR_TIMEOUT, "hub bucket overflow persists");
     if (!(st = grow_hubs(s, &a)).ok()) return st;
-    if (!(st = clear_round(s, insert_count(s, true), true)).ok()) return st;
+    if (!(st = clear_round(s, insert_count(s, true), true, true)).ok()) return st;
     if (!(st = typed(hubs_again)).ok()) return st;
   }
   if (i >= 2) s.hub_calm = !s.hub_grew;  // (level 1 has few distinct keys)

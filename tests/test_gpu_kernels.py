@@ -118,3 +118,20 @@ def _set_sizes(g, prev):
                     axis=1)
     per = np.bincount(key[0].astype(np.int64))
     return [int(per.sum()), int(per.max())]
+
+
+@pytest.mark.parametrize("hash_bits", [64, 22])
+def test_grouping_of_many_nodes_through_the_filter(hash_bits):
+    """Above 4M nodes the grouping filters out the hashes that occur once: blocks of one, of two, of hundreds and
+    of a million nodes (no out-edges), and hashes that collide."""
+    n, leaves, m = 4_400_000, 1_000_000, 6_000_000
+    rng = np.random.default_rng(29)
+    src = rng.integers(leaves, n, m).astype(np.uint32)
+    dst = rng.integers(0, n, m).astype(np.uint32)
+    src[:400_000] = leaves + np.arange(400_000) // 2  # pairs of nodes with the same two elements
+    dst[:400_000:4] = dst[2:400_000:4]
+    dst[1:400_000:4] = dst[3:400_000:4]
+    g = synth.from_coo(n, src, dst, rng.integers(0, 200, m).astype(np.uint32), (np.arange(n) % 5).astype(np.uint32))
+    with KBisim(hash_bits=hash_bits) as kb:
+        res = kb.build(g, 2)
+        assert_same(res, kb.all_pids(2), oracle_levels(g, 2))
