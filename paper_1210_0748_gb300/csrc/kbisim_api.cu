@@ -651,6 +651,7 @@ Status refine(Store& s, uint32_t k, kbisim_result* out) {
   s.stable = false;
   s.computed = 0;
   s.rounds_run = 0;
+  s.heads_level = -1;
   s.stats.clear();
   s.counts.assign(std::max<size_t>(snap.counts.size(), 1), 0);
   Status st = refine_levels(s, k);
@@ -675,6 +676,7 @@ Status extend(Store& s, uint32_t k_new, kbisim_result* out) {
   InUse use(s, kCacheSpare);
   Status st;
   const bool need = k_new > s.computed && !(s.early_stop && s.stable);
+  s.heads_level = -1;
   if (need) {
     if (!(st = ensure(s, s.spare_alone, s.n + 16)).ok()) return st;
     if (!(st = cuda_check(cudaMemcpyAsync(s.spare_alone.p, s.alone.p, s.n + 16, cudaMemcpyDeviceToDevice,

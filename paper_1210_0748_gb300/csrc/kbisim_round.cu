@@ -1473,6 +1473,9 @@ struct VerifyArgs {
   unsigned long long* n_long;
   uint32_t* hbits;          // head bitmap over original ids (canonical numbering)
   uint8_t* member;          // per internal id: this head has other members
+  // the marks and representatives of the nodes alone in their previous block
+  // stand since the level before (a head stays one: its block only splits)
+  bool keep;
 };
 
 constexpr uint32_t kShortSig = 8;   // compared by one thread
@@ -1574,6 +1577,7 @@ __global__ void __launch_bounds__(kFilThreads) k_group_select(GroupArgs g, Verif
       const uint64_t p = base + threadIdx.x + (uint64_t)t * kFilThreads;
       act[t] = p < count;
       cand[t] = act[t] && !(g.alone && g.alone[p]);
+      act[t] = act[t] && !(v.keep && !cand[t]);
       if (act[t]) o[t] = g.p2o[p];
       if (cand[t]) h[t] = g.hash[p];
     }
@@ -1649,6 +1653,7 @@ __global__ void __launch_bounds__(kVerNodeThreads) k_group_verify(GroupArgs g, V
     for (int t = 0; t < kVerItems; ++t) act[t] = p[t] != kNone32 && !(g.alone && g.alone[p[t]]);
 #pragma unroll
     for (int t = 0; t < kVerItems; ++t) {
+      if (!act[t] && v.keep) p[t] = kNone32;
       if (p[t] != kNone32) o[t] = g.p2o[p[t]];
       if (act[t]) x[t] = g.slot[p[t]];
     }
@@ -2077,10 +2082,25 @@ __global__ void k_label_hash(uint64_t n, const uint32_t* nlabel, uint64_t* hash,
     hash[p] = node_hash(0, nlabel[p], 0, seed, mask);
 }
 
-__global__ void k_unpermute(uint64_t n, const uint32_t* o2p, const uint32_t* lvl, uint32_t* out) {
-  for (uint64_t o = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; o < n;
-       o += (uint64_t)gridDim.x * blockDim.x)
-    out[o] = lvl[o2p[o]];
+// A level in original order: a coalesced read, a gather and a coalesced write
+// per node.  Four nodes per thread in flight (one a time left the loads' latency
+// bare: 58 us at 16M nodes).
+constexpr int kUnpItems = 4, kUnpThreads = 256;
+
+__global__ void __launch_bounds__(kUnpThreads) k_unpermute(uint64_t n, const uint32_t* o2p, const uint32_t* lvl, uint32_t* out) {
+  const uint64_t stride = (uint64_t)gridDim.x * kUnpThreads;
+  for (uint64_t o0 = blockIdx.x * (uint64_t)kUnpThreads + threadIdx.x; o0 < n; o0 += stride * kUnpItems) {
+    uint32_t x[kUnpItems];
+#pragma unroll
+    for (int t = 0; t < kUnpItems; ++t)
+      if (o0 + t * stride < n) x[t] = __ldg(o2p + o0 + t * stride);
+#pragma unroll
+    for (int t = 0; t < kUnpItems; ++t)
+      if (o0 + t * stride < n) x[t] = __ldg(lvl + x[t]);
+#pragma unroll
+    for (int t = 0; t < kUnpItems; ++t)
+      if (o0 + t * stride < n) out[o0 + t * stride] = x[t];
+  }
 }
 
 // --------------------------------------------------------------------------
@@ -2593,6 +2613,7 @@ VerifyArgs verify_args(Store& s, int mode, const uint32_t* prev, bool key64) {
   v.n_long = sc + 6;
   v.hbits = ptr<uint32_t>(s.hbits);
   v.member = ptr<uint8_t>(s.member);
+  v.keep = false;
   return v;
 }
 
@@ -2605,11 +2626,12 @@ uint64_t filter_bits(uint64_t ins) { return ins > kFilterNodes ? 4 * table_slots
 // scalars, the marks of the canonical numbering, the hash table for `ins`
 // inserted nodes or the filter before it, and, with hubs, their buckets'
 // cursors and totals.
-Status clear_round(Store& s, uint64_t ins, bool filter, bool hubs) {
+// `keep`: the head marks of the level before stay.
+Status clear_round(Store& s, uint64_t ins, bool filter, bool hubs, bool keep) {
   ClearArgs c;
   c.add(s.d_err.p, 16, 0u);
   c.add(s.d_scalars.p, 16 * 8, 0u);
-  c.add(s.hbits.p, (s.n + 31) / 32 * 4, 0u);
+  if (!keep) c.add(s.hbits.p, (s.n + 31) / 32 * 4, 0u);
   c.add(s.member.p, s.n, 0u);
   if (filter && filter_bits(ins)) c.add(s.long_pairs.p, filter_bits(ins) / 4, 0u);
   else c.add(s.table.p, group_slots(s, ins) * 8, ~0u);
@@ -2637,6 +2659,7 @@ uint64_t insert_count(const Store& s, bool use_alone) {
 // the comparison of long signatures takes its pairs' number from the device,
 // and the numbering is launched before the host knows whether a hash collision
 // left nodes unresolved; if one did they are settled and it runs again.
+// `keep`: hbits and rep hold the level before (Store::heads_level).
 // *hub_flags (mode 1): overflow flags of the hub passes before; when set, the
 // signatures were incomplete and nothing else is returned.
 //
@@ -2648,14 +2671,15 @@ uint64_t insert_count(const Store& s, bool use_alone) {
 //  the grouping, [15] the number of blocks.
 Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint32_t* pid, uint64_t* blocks,
                       uint64_t* collided, bool with_stats, uint64_t* keys, uint64_t* maxsig, bool use_alone,
-                      uint32_t* hub_flags) {
+                      bool keep, uint32_t* hub_flags) {
   const uint64_t n = s.n, na = s.n_alive;
   Status st;
   unsigned long long* sc = ptr<unsigned long long>(s.d_scalars);
   GroupArgs g = group_args(s, group_slots(s, insert_count(s, use_alone)));
   g.alone = use_alone ? ptr<uint8_t>(s.alone) : nullptr;
   g.read_first = mode == 0 ? 1 : 0;
-  const VerifyArgs v = verify_args(s, mode, prev, key64);
+  VerifyArgs v = verify_args(s, mode, prev, key64);
+  v.keep = keep;
   const uint64_t words = (n + 31) / 32;
   uint64_t h[16] = {0};
   // canonical renumbering
@@ -3397,7 +3421,7 @@ Status compute_level0(Store& s) {
   if (done) return Status::Ok();
   const int sms = sm_count(s.device);
   const unsigned blocks = (unsigned)std::min<uint64_t>(grid_for(s.n_alive, 256), (uint64_t)sms * 16);
-  if (!(st = clear_round(s, s.n_alive, false, false)).ok()) return st;
+  if (!(st = clear_round(s, s.n_alive, false, false, false)).ok()) return st;
   {
     TimedScope ts(s, KBISIM_KERNEL_LABEL_GROUP, s.n_alive ? 1 : 0);
     if (s.n_alive)
@@ -3407,7 +3431,7 @@ Status compute_level0(Store& s) {
   if (!(st = launch_check("k_label_hash")).ok()) return st;
   uint64_t blocks_out = 0, coll = 0;
   st = group_and_rank(s, 0, nullptr, false, ptr<uint32_t>(s.level[0]), &blocks_out, &coll, false, nullptr,
-                      nullptr, false, nullptr);
+                      nullptr, false, false, nullptr);
   if (!st.ok()) return st;
   s.counts[0] = blocks_out;
   return Status::Ok();
@@ -3450,7 +3474,9 @@ Status compute_round(Store& s, uint32_t i) {
     return Status::Err(KBISIM_ERR_TIMEOUT, "injected timeout (KBISIM_FAULT_TIMEOUT_ROUND)");
   Status st = ensure_round_scratch(s);
   if (!st.ok()) return st;
-  if (!(st = clear_round(s, insert_count(s, true), true, s.n_hub != 0)).ok()) return st;
+  bool keep = s.heads_level == (int64_t)i - 1;
+  s.heads_level = -1;
+  if (!(st = clear_round(s, insert_count(s, true), true, s.n_hub != 0, keep)).ok()) return st;
   if (s.checked && !(st = check_round_inputs(s, i)).ok()) return st;
   SigArgs a;
   a.off = ptr<uint64_t>(s.offsets);
@@ -3500,14 +3526,16 @@ Status compute_round(Store& s, uint32_t i) {
   for (int attempt = 0;; ++attempt) {
     uint32_t hub_flags = 0;
     st = group_and_rank(s, 1, a.prev, key64, ptr<uint32_t>(s.level[i]), &blocks, &coll, true, &keys, &maxsig, true,
-                        &hub_flags);
+                        keep, &hub_flags);
     if (!st.ok()) return st;
     if (!hub_flags) break;
     if (attempt >= kHubAttempts) return Status::Err(KBISIM_ERR_TIMEOUT, "hub bucket overflow persists");
     if (!(st = grow_hubs(s, &a)).ok()) return st;
-    if (!(st = clear_round(s, insert_count(s, true), true, true)).ok()) return st;
+    keep = false;  // heads were marked with incomplete signatures
+    if (!(st = clear_round(s, insert_count(s, true), true, true, false)).ok()) return st;
     if (!(st = typed(hubs_again)).ok()) return st;
   }
+  s.heads_level = i;
   if (i >= 2) s.hub_calm = !s.hub_grew;  // (level 1 has few distinct keys)
   s.counts[i] = blocks;
   kbisim_round_stats rs;
@@ -3574,8 +3602,8 @@ Status group_list(Store& s, const uint32_t* list, uint64_t count, const uint32_t
 Status unpermute_level(Store& s, uint32_t level, uint32_t* dst) {
   if (!s.n) return Status::Ok();
   const int sms = sm_count(s.device);
-  const unsigned gb = (unsigned)std::min<uint64_t>(grid_for(s.n, 256), (uint64_t)sms * 16);
-  k_unpermute<<<gb, 256, 0, s.stream>>>(s.n, ptr<uint32_t>(s.o2p), ptr<uint32_t>(s.level[level]), dst);
+  const unsigned gb = (unsigned)std::min<uint64_t>(grid_for(s.n, kUnpThreads * kUnpItems), (uint64_t)sms * 8);
+  k_unpermute<<<gb, kUnpThreads, 0, s.stream>>>(s.n, ptr<uint32_t>(s.o2p), ptr<uint32_t>(s.level[level]), dst);
   return launch_check("k_unpermute");
 }
 
