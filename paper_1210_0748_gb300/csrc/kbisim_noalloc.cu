@@ -31,14 +31,16 @@ namespace {
 
 constexpr uint64_t kMaxNodes = 1ull << 18;          // 262,144 nodes
 constexpr uint64_t kSlots = 2 * kMaxNodes;          // hash table slots (power of two)
-constexpr int kThreads = 1024;                      // rank kernels: one node per thread
+constexpr int kThreads = 1024;                      // head kernel: one node per thread
+static_assert(kThreads == 1024, "one warp sums the warps");
 constexpr uint64_t kTiles = kMaxNodes / kThreads;   // 256
 constexpr unsigned long long kEmptySlot = ~0ull;
 
 struct Scratch {
   unsigned long long table[kSlots];  // (label << 32) | smallest node id with that label
-  uint32_t rank[kMaxNodes];          // head flag, then the head's block id
-  uint32_t tile[kTiles + 1];         // heads per tile, then exclusive offsets; [kTiles] = total
+  uint32_t rank[kMaxNodes];          // of a head: heads before it in its tile
+  uint32_t tile[kTiles];             // heads per tile, then heads before the tile
+  uint32_t ticket;                   // tiles counted
 };
 
 static __device__ __align__(256) Scratch g_scratch;
@@ -78,76 +80,99 @@ __device__ __forceinline__ int64_t find_slot(Scratch* sc, uint32_t label, uint32
   return -1;
 }
 
+// Four launches, each started while the one before still runs
+// (programmatic dependent launch) and waiting for it before its first access:
+// at 262,144 nodes the work is a few microseconds a step, and six launches in
+// a row (with the tile scan and the ranks in launches of their own) took 33 us.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __global__ void k_na_clear(Scratch* sc, uint64_t slots) {
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < slots; i += (uint64_t)gridDim.x * blockDim.x)
-    sc->table[i] = kEmptySlot;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  ulonglong2* t = reinterpret_cast<ulonglong2*>(sc->table);
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < slots / 2; i += (uint64_t)gridDim.x * blockDim.x)
+    t[i] = make_ulonglong2(kEmptySlot, kEmptySlot);
+  if (blockIdx.x == 0 && threadIdx.x == 0) sc->ticket = 0;
 }
 
 __global__ void k_na_insert(Scratch* sc, const uint32_t* label, uint64_t n, uint64_t mask) {
+  after_previous();
   for (uint64_t u = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; u < n; u += (uint64_t)gridDim.x * blockDim.x)
     find_slot(sc, label[u], (uint32_t)u, mask, true);
 }
 
-// rank[u] = 1 if u is the smallest node with its label; per-tile head counts.
-__global__ void __launch_bounds__(kThreads) k_na_heads(Scratch* sc, const uint32_t* label, uint64_t n, uint64_t mask) {
+// Exclusive sum of v over the CTA of kThreads; *total gets the CTA's sum.
+__device__ __forceinline__ uint32_t cta_before(uint32_t v, uint32_t* warp_sum, uint32_t* total) {
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  uint32_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+    if (lane >= (uint32_t)o) x += y;
+  }
+  if (lane == 31) warp_sum[w] = x;
+  __syncthreads();
+  const uint32_t s = warp_sum[lane];  // kThreads / 32 = 32 warps
+  *total = __reduce_add_sync(0xFFFFFFFFu, s);
+  const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < w ? s : 0u);
+  __syncthreads();
+  return before + x - v;
+}
+
+// Heads (the smallest node of each label): their rank in their tile; the CTA
+// that comes last (a ticket: nothing waits) turns the tiles' head counts into
+// heads before each tile and writes the block count.
+__global__ void __launch_bounds__(kThreads) k_na_heads(Scratch* sc, const uint32_t* label, uint64_t n, uint64_t mask,
+                                                       uint32_t* count_out) {
+  after_previous();
   __shared__ uint32_t warp_sum[kThreads / 32];
+  __shared__ uint32_t last;
   const uint64_t u = (uint64_t)blockIdx.x * kThreads + threadIdx.x;
-  uint32_t head = 0;
+  uint32_t head = 0, total;
   if (u < n) {
     const int64_t s = find_slot(sc, label[u], (uint32_t)u, mask, false);
     head = (s >= 0 && (uint32_t)sc->table[s] == (uint32_t)u) ? 1u : 0u;
-    sc->rank[u] = head;
   }
-  uint32_t c = __popc(__ballot_sync(0xFFFFFFFFu, head));
-  if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = c;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t t = 0;
-    for (int w = 0; w < kThreads / 32; ++w) t += warp_sum[w];
-    sc->tile[blockIdx.x] = t;
-  }
-}
-
-// Exclusive scan of the tile counts (one CTA, at most kTiles tiles).
-__global__ void __launch_bounds__(kTiles) k_na_scan(Scratch* sc, uint64_t ntiles, uint32_t* count_out) {
-  __shared__ uint32_t v[kTiles];
-  const uint32_t i = threadIdx.x;
-  v[i] = i < ntiles ? sc->tile[i] : 0u;
-  __syncthreads();
-  for (uint32_t o = 1; o < kTiles; o <<= 1) {
-    const uint32_t add = i >= o ? v[i - o] : 0u;
-    __syncthreads();
-    v[i] += add;
-    __syncthreads();
-  }
-  if (i < ntiles) sc->tile[i] = v[i] - (i < ntiles ? sc->tile[i] : 0u);
-  __syncthreads();
-  if (i == 0) {
-    sc->tile[kTiles] = v[kTiles - 1];
-    if (count_out) *count_out = v[kTiles - 1];
-  }
-}
-
-// Heads get their block id: tile offset + heads before them in the tile.
-__global__ void __launch_bounds__(kThreads) k_na_rank(Scratch* sc, uint64_t n) {
-  __shared__ uint32_t warp_sum[kThreads / 32];
-  const uint64_t u = (uint64_t)blockIdx.x * kThreads + threadIdx.x;
-  const uint32_t head = u < n ? sc->rank[u] : 0u;
-  const unsigned lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const unsigned bal = __ballot_sync(0xFFFFFFFFu, head);
-  if (lane == 0) warp_sum[w] = __popc(bal);
-  __syncthreads();
-  uint32_t before = sc->tile[blockIdx.x];
-  for (unsigned i = 0; i < w; ++i) before += warp_sum[i];
-  before += __popc(bal & ((1u << lane) - 1u));
+  const uint32_t before = cta_before(head, warp_sum, &total);
   if (head) sc->rank[u] = before;
+  if (threadIdx.x == 0) {
+    sc->tile[blockIdx.x] = total;
+    __threadfence();
+    last = atomicAdd(&sc->ticket, 1u) == gridDim.x - 1 ? 1u : 0u;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const uint32_t t = threadIdx.x;
+  const uint32_t v = t < gridDim.x ? __ldcg(&sc->tile[t]) : 0u;
+  const uint32_t tb = cta_before(v, warp_sum, &total);
+  if (t < gridDim.x) sc->tile[t] = tb;
+  if (t == 0 && count_out) *count_out = total;
 }
 
 __global__ void k_na_assign(Scratch* sc, const uint32_t* label, uint64_t n, uint64_t mask, uint32_t* pid0) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   for (uint64_t u = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; u < n; u += (uint64_t)gridDim.x * blockDim.x) {
     const int64_t s = find_slot(sc, label[u], (uint32_t)u, mask, false);
-    pid0[u] = s >= 0 ? sc->rank[(uint32_t)sc->table[s]] : KBISIM_DELETED;
+    const uint32_t head = s >= 0 ? (uint32_t)sc->table[s] : 0u;
+    pid0[u] = s >= 0 ? sc->tile[head / kThreads] + sc->rank[head] : KBISIM_DELETED;
   }
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_after(cudaStream_t st, bool overlap, void (*kernel)(P...), unsigned blocks, unsigned threads, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(blocks);
+  c.blockDim = dim3(threads);
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kernel, P(args)...);
 }
 
 }  // namespace
@@ -184,11 +209,9 @@ extern "C" int kbisim_label_partition_noalloc(const uint32_t* node_label, uint64
   const uint64_t mask = slots - 1;
   const uint64_t ntiles = (num_nodes + kThreads - 1) / kThreads;
   const unsigned g = (unsigned)((num_nodes + 255) / 256);
-  k_na_clear<<<(unsigned)((slots + 255) / 256), 256, 0, st>>>(sc, slots);
-  k_na_insert<<<g, 256, 0, st>>>(sc, node_label, num_nodes, mask);
-  k_na_heads<<<(unsigned)ntiles, kThreads, 0, st>>>(sc, node_label, num_nodes, mask);
-  k_na_scan<<<1, (unsigned)kTiles, 0, st>>>(sc, ntiles, block_count);
-  k_na_rank<<<(unsigned)ntiles, kThreads, 0, st>>>(sc, num_nodes);
-  k_na_assign<<<g, 256, 0, st>>>(sc, node_label, num_nodes, mask, pid0);
+  launch_after(st, false, k_na_clear, (unsigned)((slots / 2 + 255) / 256), 256, sc, slots);
+  launch_after(st, true, k_na_insert, g, 256, sc, node_label, num_nodes, mask);
+  launch_after(st, true, k_na_heads, (unsigned)ntiles, kThreads, sc, node_label, num_nodes, mask, block_count);
+  launch_after(st, true, k_na_assign, g, 256, sc, node_label, num_nodes, mask, pid0);
   return cudaGetLastError() == cudaSuccess ? KBISIM_OK : KBISIM_ERR_CUDA;
 }
