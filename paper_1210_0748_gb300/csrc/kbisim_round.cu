@@ -3269,6 +3269,7 @@ Status relabel_graph(Store& s, const uint64_t* off0, const uint32_t* dst0, const
 // a shared copy, so the global table sees one update per label per CTA.  If a
 // shared or the global table fills (more labels than it holds) the general
 // path (hash, grouping, exact check, renumbering) computes the level instead.
+// The host waits once, for the block count.
 constexpr int kL0Slots = 4096;        // global table: labels at most kL0Slots / 2
 constexpr int kL0SmemSlots = 1024;    // per CTA
 constexpr int kL0Threads = 256;
@@ -3298,6 +3299,8 @@ __device__ __forceinline__ int l0_insert(unsigned long long* tab, uint32_t mask,
 
 __global__ void __launch_bounds__(kL0Threads) k_l0_collect(uint64_t n_alive, const uint32_t* nlabel, const uint32_t* p2o,
                                                            unsigned long long* gtab, uint32_t* gcnt, uint32_t* err) {
+  overlap_next();
+  overlap_wait();
   __shared__ unsigned long long tab[kL0SmemSlots];
   __shared__ uint32_t cnt[kL0SmemSlots];
   __shared__ uint32_t full;
@@ -3329,11 +3332,63 @@ __global__ void __launch_bounds__(kL0Threads) k_l0_collect(uint64_t n_alive, con
   }
 }
 
+// Block ids of the table's labels, ranked by smallest original id, by one CTA:
+// a label's rank is the number of labels with a smaller id (up to
+// kL0Slots / 2 of them, listed in shared memory; more set err).  On the device,
+// so that level 0 needs no copies of the table (three, a host sort and one copy
+// back took 50 us).  stats: [7] err, [8] nodes alone, [15] blocks.
+constexpr int kL0RankThreads = 1024;
+
+__global__ void __launch_bounds__(kL0RankThreads) k_l0_rank(const unsigned long long* gtab, const uint32_t* gcnt,
+                                                            uint32_t* rank, uint32_t* err, unsigned long long* stats) {
+  overlap_next();
+  overlap_wait();
+  __shared__ uint32_t ids[kL0Slots / 2];
+  __shared__ uint32_t n, alone;
+  if (threadIdx.x == 0) n = alone = 0;
+  __syncthreads();
+  constexpr int kPer = kL0Slots / kL0RankThreads;
+  unsigned long long v[kPer];
+#pragma unroll
+  for (int t = 0; t < kPer; ++t) {
+    v[t] = gtab[threadIdx.x + t * kL0RankThreads];
+    if (v[t] == kL0Empty) continue;
+    const uint32_t at = atomicAdd(&n, 1u);
+    if (at < (uint32_t)kL0Slots / 2) ids[at] = (uint32_t)v[t];
+    if (gcnt[threadIdx.x + t * kL0RankThreads] == 1u) atomicAdd(&alone, 1u);
+  }
+  __syncthreads();
+  const uint32_t found = n;
+  if (found > (uint32_t)kL0Slots / 2) {  // long probe runs: the general path
+    if (threadIdx.x == 0) {
+      *err = 1u;
+      stats[7] = 1ull;
+    }
+    return;
+  }
+#pragma unroll
+  for (int t = 0; t < kPer; ++t) {
+    if (v[t] == kL0Empty) continue;
+    uint32_t r = 0;
+    for (uint32_t j = 0; j < found; ++j) r += ids[j] < (uint32_t)v[t] ? 1u : 0u;
+    rank[threadIdx.x + t * kL0RankThreads] = r;
+  }
+  if (threadIdx.x == 0) {
+    stats[7] = *err;
+    stats[8] = alone;
+    stats[15] = found;
+  }
+}
+
 // pId_0 of every node from the ranked table: rank[slot] = block id, and the
 // node is alone in its block when its label's count is 1.
 __global__ void __launch_bounds__(kL0Threads) k_l0_fill(uint64_t n, uint64_t n_alive, const uint32_t* nlabel,
                                                         const unsigned long long* gtab, const uint32_t* rank,
-                                                        const uint32_t* gcnt, uint32_t* pid, uint8_t* alone) {
+                                                        const uint32_t* gcnt, const uint32_t* err, uint32_t* pid,
+                                                        uint8_t* alone) {
+  overlap_next();
+  overlap_wait();
+  if (*err) return;  // too many labels
   for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < n; p += (uint64_t)gridDim.x * blockDim.x) {
     if (p >= n_alive) {
       pid[p] = kDead;
@@ -3367,48 +3422,33 @@ Status level0_few_labels(Store& s, bool* done) {
   uint32_t* grank = gcnt + kL0Slots;
   uint32_t* err = grank + kL0Slots;
   const int sms = sm_count(s.device);
-  cudaMemsetAsync(s.d_err.p, 0, 4, s.stream);
+  unsigned long long* sc = ptr<unsigned long long>(s.d_scalars);
   {
-    TimedScope ts(s, KBISIM_KERNEL_LABEL_GROUP, 1);
-    cudaMemsetAsync(gtab, 0xFF, kL0Slots * 8, s.stream);
-    cudaMemsetAsync(gcnt, 0, kL0Slots * 4 * 2 + 16, s.stream);
+    TimedScope ts(s, KBISIM_KERNEL_LABEL_GROUP, 3);
+    ClearArgs c;
+    c.add(s.d_err.p, 16, 0u);
+    c.add(sc, 16 * 8, 0u);
+    c.add(gtab, kL0Slots * 8, ~0u);
+    c.add(gcnt, kL0Slots * 4 * 2 + 16, 0u);
+    k_clear<<<8, kClearThreads, 0, s.stream>>>(c);
     const unsigned g = (unsigned)std::min<uint64_t>(grid_for(na, 2048), (uint64_t)sms * 8);
-    k_l0_collect<<<g, kL0Threads, 0, s.stream>>>(na, ptr<uint32_t>(s.nlabel), ptr<uint32_t>(s.p2o), gtab, gcnt, err);
+    launch_chained(s, k_l0_collect, g, kL0Threads, 0, na, ptr<uint32_t>(s.nlabel), ptr<uint32_t>(s.p2o), gtab, gcnt, err);
+    launch_chained(s, k_l0_rank, 1, kL0RankThreads, 0, gtab, gcnt, grank, err, sc);
   }
   if (!(st = launch_check("k_l0_collect")).ok()) return st;
-  std::vector<unsigned long long> tab(kL0Slots);
-  std::vector<uint32_t> cnt(kL0Slots + 1);
-  st = cuda_check(cudaMemcpyAsync(tab.data(), gtab, kL0Slots * 8, cudaMemcpyDeviceToHost, s.stream), "level 0");
-  if (st.ok())
-    st = cuda_check(cudaMemcpyAsync(cnt.data(), gcnt, kL0Slots * 4, cudaMemcpyDeviceToHost, s.stream), "level 0");
-  if (st.ok()) st = cuda_check(cudaMemcpyAsync(&cnt[kL0Slots], err, 4, cudaMemcpyDeviceToHost, s.stream), "level 0");
-  if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "sync");
-  if (!st.ok() || cnt[kL0Slots]) return st;  // too many labels: the general path
-  // blocks ranked by their smallest original id
-  std::vector<std::pair<uint32_t, uint32_t>> heads;  // (smallest id, slot)
-  uint64_t alone = 0;
-  for (uint32_t i = 0; i < (uint32_t)kL0Slots; ++i)
-    if (tab[i] != kL0Empty) {
-      heads.push_back({(uint32_t)tab[i], i});
-      alone += cnt[i] == 1 ? 1 : 0;
-    }
-  if (heads.size() > (size_t)kL0Slots / 2) return Status::Ok();  // long probe runs: the general path
-  std::sort(heads.begin(), heads.end());
-  std::vector<uint32_t> rank(kL0Slots, 0);
-  for (size_t r = 0; r < heads.size(); ++r) rank[heads[r].second] = (uint32_t)r;
-  st = cuda_check(cudaMemcpyAsync(grank, rank.data(), kL0Slots * 4, cudaMemcpyHostToDevice, s.stream), "level 0");
-  if (!st.ok()) return st;
   {
     TimedScope ts(s, KBISIM_KERNEL_RENUMBER, 1);
     const unsigned g = (unsigned)std::min<uint64_t>(grid_for(n, kL0Threads), (uint64_t)sms * 16);
-    k_l0_fill<<<g, kL0Threads, 0, s.stream>>>(n, na, ptr<uint32_t>(s.nlabel), gtab, grank, gcnt,
-                                             ptr<uint32_t>(s.level[0]), ptr<uint8_t>(s.alone));
+    launch_chained(s, k_l0_fill, g, kL0Threads, 0, n, na, ptr<uint32_t>(s.nlabel), gtab, grank, gcnt, err,
+                   ptr<uint32_t>(s.level[0]), ptr<uint8_t>(s.alone));
   }
   if (!(st = launch_check("k_l0_fill")).ok()) return st;
-  if (s.checked && !(st = check_below(s, ptr<uint32_t>(s.level[0]), na, heads.size(), "identifiers")).ok())
-    return st;
-  s.counts[0] = heads.size();
-  s.n_alone = alone;
+  uint64_t h[16];
+  if (!(st = read_scalars(s, h)).ok()) return st;
+  if (h[7]) return Status::Ok();  // too many labels: the general path
+  if (s.checked && !(st = check_below(s, ptr<uint32_t>(s.level[0]), na, h[15], "identifiers")).ok()) return st;
+  s.counts[0] = h[15];
+  s.n_alone = h[8];
   *done = true;
   return Status::Ok();
 }

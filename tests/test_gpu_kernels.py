@@ -135,3 +135,33 @@ def test_grouping_of_many_nodes_through_the_filter(hash_bits):
     with KBisim(hash_bits=hash_bits) as kb:
         res = kb.build(g, 2)
         assert_same(res, kb.all_pids(2), oracle_levels(g, 2))
+
+
+@pytest.mark.parametrize("nodes,labels", [(1, 1), (2, 2), (31, 5), (1023, 1023), (1024, 3), (1025, 1025), (50_000, 50_000),
+                                          (262_143, 2047), (262_144, 262_144)])
+def test_label_partition_at_tile_edges(nodes, labels):
+    """The allocation-free partition and level 0 (label table up to 2048 labels, general path above)."""
+    import torch
+    from paper_1210_0748_gb300.kbisim import label_partition_noalloc
+    rng = np.random.default_rng(nodes + labels)
+    lab = rng.permutation(np.concatenate([np.arange(labels), rng.integers(0, labels, nodes - labels)]))
+    lab = (lab * 2_654_435_761 % (1 << 32)).astype(np.uint32)
+    ref = oracle.kbisim(nodes, lab, [], [], [], 0)
+    out = torch.full((nodes,), -1, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+    label_partition_noalloc(torch.from_numpy(lab.view(np.int32)).cuda(), out, cnt)
+    assert np.array_equal(out.cpu().numpy().view(np.uint32), ref.pids[0])
+    assert int(cnt.item()) == labels
+    with KBisim() as kb:
+        res = kb.build(synth.from_coo(nodes, [], [], [], lab), 0)
+        assert res.counts == [labels]
+        assert np.array_equal(kb.pids(0), ref.pids[0])
+
+
+@pytest.mark.parametrize("labels", [2047, 2048, 2049, 5000])
+def test_level0_table_limit(labels):
+    g = synth.random_small_graph(20_000, 40_000, node_labels=2, edge_labels=2, seed=1)
+    g.node_label = (np.arange(20_000) * 7919 % labels).astype(np.uint32)
+    with KBisim() as kb:
+        res = kb.build(g, 2)
+        assert_same(res, kb.all_pids(2), oracle_levels(g, 2))
