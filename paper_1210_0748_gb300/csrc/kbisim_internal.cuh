@@ -268,6 +268,7 @@ struct Store {
   Buf alone;                   // uint8 [n] node is alone in its block at the last computed level
   Buf hword;                   // uint64 [(n+31)/32] heads before each bitmap word
   uint64_t n_alone = 0;        // nodes alone in their block at the last computed level
+  bool pairs_last = true;      // the last round left signatures longer than a thread compares
   int64_t heads_level = -1;    // the level whose heads hbits and rep hold, while one call refines (-1 = none)
   Buf bsum;                    // uint64 scan block sums
   Buf long_pairs;              // uint32 [2n] (node, candidate) pairs with long signatures

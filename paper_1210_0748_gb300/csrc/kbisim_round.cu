@@ -882,7 +882,8 @@ __global__ void __launch_bounds__(NT, sizeof(K) == 4 ? 2048 / NT : 1536 / NT) k_
 // (kErrHubSet) gives its hub more buckets.  Pass 2 (k_hub_bucket):
 // one CTA per bucket deduplicates across chunks and appends the bucket's
 // distinct keys at the hub's CSR offset, adding to the hub's count and term
-// sums; k_hub_finish then writes each hub's count and hash.
+// sums; the CTA of a hub's last bucket, or k_hub_finish, writes its count and
+// hash.
 struct HubArgs {
   uint64_t first;           // internal id of hub 0
   const uint32_t* hub_bits;
@@ -894,6 +895,7 @@ struct HubArgs {
   uint32_t* cursor;              // per bucket: key words appended
   unsigned long long* hub_cur;   // per hub: distinct keys written
   uint32_t* hub_term;            // per hub: term sum halves (low, high)
+  uint32_t* done;                // per hub: buckets deduplicated (NULL: k_hub_finish follows)
   void* tmp;
   uint8_t* mode;                 // per hub: 1 = chunks skip their set (few repeated keys)
   const uint8_t* force;          // per hub: 1 = always the deduplicating chunk pass
@@ -927,10 +929,7 @@ __device__ __forceinline__ uint32_t hub_bucket(K k, uint32_t bits) {
 }
 
 template <typename LabelT, typename K>
-__global__ void __launch_bounds__(kChunkThreads) k_hub_chunk(SigArgs a, HubArgs h) {
-  overlap_next();
-  overlap_wait();
-  extern __shared__ __align__(16) char smem_raw[];
+__device__ __forceinline__ void hub_chunk_block(const SigArgs& a, const HubArgs& h, char* smem_raw) {
   ChunkSmem<K>& sm = *reinterpret_cast<ChunkSmem<K>*>(smem_raw);
   K* list = reinterpret_cast<K*>(smem_raw + sizeof(ChunkSmem<K>));
   uint32_t* bcnt = reinterpret_cast<uint32_t*>(list + kHubChunk);
@@ -990,6 +989,14 @@ __global__ void __launch_bounds__(kChunkThreads) k_hub_chunk(SigArgs a, HubArgs 
     if (q < cap) tmp[(uint64_t)b * cap + q] = v;
     else hub_fail(a, h, hub, kErrHubOverflow);
   }
+}
+
+template <typename LabelT, typename K>
+__global__ void __launch_bounds__(kChunkThreads) k_hub_chunk(SigArgs a, HubArgs h) {
+  overlap_next();
+  overlap_wait();
+  extern __shared__ __align__(16) char smem_raw[];
+  hub_chunk_block<LabelT, K>(a, h, smem_raw);
 }
 
 // Hub pieces without the chunk-level set, for hubs whose keys rarely repeat
@@ -1069,15 +1076,17 @@ __device__ __forceinline__ void cta_exclusive_scan(uint32_t* v, uint32_t n, uint
   __syncthreads();
 }
 
+template <typename K>
+struct ScatterSmem {
+  K stage[kHubChunk];
+  uint32_t bcnt[kHubSmemBuckets], bpos[kHubSmemBuckets], lstart[kHubSmemBuckets];
+  uint32_t wsum[kChunkThreads / 32];
+};
+
 template <typename LabelT, typename K>
-__global__ void __launch_bounds__(kChunkThreads) k_hub_scatter(SigArgs a, HubArgs h) {
-  overlap_next();
-  overlap_wait();
-  __shared__ uint32_t bcnt[kHubSmemBuckets];
-  __shared__ uint32_t bpos[kHubSmemBuckets];
-  __shared__ uint32_t lstart[kHubSmemBuckets];
-  __shared__ uint32_t wsum[kChunkThreads / 32];
-  __shared__ K stage[kHubChunk];
+__device__ __forceinline__ void hub_scatter_block(const SigArgs& a, const HubArgs& h, ScatterSmem<K>& sm) {
+  uint32_t *bcnt = sm.bcnt, *bpos = sm.bpos, *lstart = sm.lstart, *wsum = sm.wsum;
+  K* stage = sm.stage;
   const uint4 c = h.chunks[blockIdx.x];
   const uint32_t hub = c.x;
   if (!h.mode[hub]) return;  // this hub's chunks run k_hub_chunk
@@ -1140,6 +1149,28 @@ __global__ void __launch_bounds__(kChunkThreads) k_hub_scatter(SigArgs a, HubArg
   }
 }
 
+template <typename LabelT, typename K>
+__global__ void __launch_bounds__(kChunkThreads, sizeof(K) == 4 ? 4 : 3) k_hub_scatter(SigArgs a, HubArgs h) {
+  overlap_next();
+  overlap_wait();
+  __shared__ ScatterSmem<K> sm;
+  hub_scatter_block<LabelT, K>(a, h, sm);
+}
+
+// Both kinds of chunk in one launch, for graphs whose rounds are launches and
+// latency more than work (up to kChainEdges): one launch less per round.  Its
+// shared memory is the chunk set's, which above that size would take the L1
+// from the scatter's gathers.
+template <typename LabelT, typename K>
+__global__ void __launch_bounds__(kChunkThreads) k_hub_pieces(SigArgs a, HubArgs h) {
+  overlap_next();
+  overlap_wait();
+  extern __shared__ __align__(16) char smem_raw[];
+  static_assert(sizeof(ScatterSmem<K>) <= hub_chunk_smem<K>(), "the scatter fits the chunk set's memory");
+  if (h.mode[h.chunks[blockIdx.x].x]) hub_scatter_block<LabelT, K>(a, h, *reinterpret_cast<ScatterSmem<K>*>(smem_raw));
+  else hub_chunk_block<LabelT, K>(a, h, smem_raw);
+}
+
 constexpr int kBucketThreads = 256, kBucketItems = 8;
 
 template <typename K, int UCAP>
@@ -1147,6 +1178,36 @@ struct BucketSmem {
   K set[2 * UCAP];
   uint32_t empty, full, lo, hi;
 };
+
+// Count and hash of a hub (of the mask) from its buckets' totals.
+__device__ __forceinline__ void hub_finish(const SigArgs& a, const HubArgs& h, uint64_t hub) {
+  const uint64_t p = h.first + hub;
+  if (!in_mask(a, p)) return;
+  const unsigned long long tot = __ldcg(&h.hub_cur[hub]);
+  const uint64_t tsum = ((uint64_t)__ldcg(&h.hub_term[2 * hub + 1]) << 32) | __ldcg(&h.hub_term[2 * hub]);
+  a.ucnt[p] = (uint32_t)tot;
+  a.hash[p] = node_hash(tsum, a.prev[p], tot, a.seed, a.mask);
+}
+
+// A bucket of the hub is done (called by one thread of its CTA, after the
+// bucket's sums have been added): the hub's last one finishes the hub.  Saves
+// a launch per round, but costs a fence and an atomic per bucket (256M edges,
+// 40K buckets a round: 9.92 against 9.81 ms), so larger graphs have h.done NULL.
+__device__ __forceinline__ void hub_bucket_done(const SigArgs& a, const HubArgs& h, uint32_t hub) {
+  if (!h.done) return;
+  const uint32_t nb = (uint32_t)(h.hub_bbase[hub + 1] - h.hub_bbase[hub]);
+  __threadfence();
+  if (atomicAdd(&h.done[hub], 1u) != nb - 1) return;
+  __threadfence();
+  hub_finish(a, h, hub);
+}
+
+__global__ void k_hub_finish(SigArgs a, HubArgs h, uint64_t n_hub) {
+  overlap_next();
+  overlap_wait();
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n_hub; i += (uint64_t)gridDim.x * blockDim.x)
+    hub_finish(a, h, i);
+}
 
 // One CTA per hub bucket (grid-stride): distinct keys of the bucket into a
 // shared set; a warp appends the keys it finds fresh straight after the
@@ -1189,6 +1250,7 @@ __global__ void __launch_bounds__(kBucketThreads, sizeof(K) == 4 ? 6 : 3) k_hub_
     const uint64_t p = h.first + hub;
     const K* tmp = nx_tmp;
     if (n == 0) {  // nothing appended (a hub outside a frontier mask): no barrier, no output
+      if (tid == 0) hub_bucket_done(a, h, hub);
       if (b + gridDim.x < n_buckets) fetch(b + gridDim.x);
       continue;
     }
@@ -1293,24 +1355,10 @@ __global__ void __launch_bounds__(kBucketThreads, sizeof(K) == 4 ? 6 : 3) k_hub_
         atomicAdd(&h.hub_term[2 * hub], sm.lo);
         atomicAdd(&h.hub_term[2 * hub + 1], sm.hi);
       }
+      hub_bucket_done(a, h, hub);
     }
     // no barrier here: thread 0 alone reads the bucket's totals, and the next
     // bucket's first barrier comes before anything is written to them again
-  }
-}
-
-// Count and hash of every hub (of the mask) from its buckets' totals.
-__global__ void k_hub_finish(SigArgs a, HubArgs h, uint64_t n_hub) {
-  overlap_next();
-  overlap_wait();
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n_hub;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t p = h.first + i;
-    if (!in_mask(a, p)) continue;
-    const unsigned long long tot = h.hub_cur[i];
-    const uint64_t tsum = ((uint64_t)h.hub_term[2 * i + 1] << 32) | h.hub_term[2 * i];
-    a.ucnt[p] = (uint32_t)tot;
-    a.hash[p] = node_hash(tsum, a.prev[p], tot, a.seed, a.mask);
   }
 }
 
@@ -1825,7 +1873,14 @@ struct RankArgs {
   uint32_t* pid;           // output level, internal order
   const uint32_t* err;     // error flags, copied to stats[7]
   unsigned long long* stats;  // [2] key total, [3] max signature, [7] error flags, [8] nodes alone in their block
+  unsigned long long* host;   // pinned: all 16 scalars, by the last CTA
 };
+
+// The 16 scalars of a level into pinned host memory (a copy of its own took
+// 3.3 us a round).  For the CTA that ends last, after a fence.
+__device__ __forceinline__ void publish_scalars(const unsigned long long* stats, unsigned long long* host, uint32_t lane) {
+  if (lane < 16) host[lane] = __ldcg(stats + lane);
+}
 
 // Heads before every bitmap word, in one pass: a CTA takes a tile of kRankTile
 // words and writes each word beside the heads before it in the tile; the CTA
@@ -1950,7 +2005,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(uint64_t* bsum, uin
 // (1M nodes: 39 us a call, 16M: 106 us).
 constexpr int kFillThreads = 256, kFillItems = 4;
 
-__global__ void __launch_bounds__(kFillThreads) k_pid_fill(RankArgs r) {
+__global__ void __launch_bounds__(kFillThreads, 6) k_pid_fill(RankArgs r) {
   overlap_next();
   overlap_wait();
   __shared__ unsigned int s_alone, s_mx;
@@ -2017,6 +2072,13 @@ __global__ void __launch_bounds__(kFillThreads) k_pid_fill(RankArgs r) {
       atomicMax(&r.stats[3], (unsigned long long)s_mx);
     }
     if (blockIdx.x == 0) r.stats[7] = *r.err;
+    __threadfence();
+    s_mx = atomicAdd(&r.stats[12], 1ull) == gridDim.x - 1 ? 1u : 0u;
+  }
+  __syncthreads();
+  if (s_mx && threadIdx.x < 32) {
+    __threadfence();
+    publish_scalars(r.stats, r.host, threadIdx.x);
   }
 }
 
@@ -2445,6 +2507,9 @@ cudaError_t set_smem_attrs_label() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_hub_chunk<LabelT, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)hub_chunk_smem<K>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_hub_pieces<LabelT, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)hub_chunk_smem<K>());
   return e;
 }
 
@@ -2474,6 +2539,13 @@ Status set_smem_attrs(int device) {
   Status st = set_smem_attrs_for<uint32_t>();
   if (st.ok()) st = set_smem_attrs_for<uint64_t>();
   if (st.ok() && device >= 0 && device < 64) done[device] = true;
+  return st;
+}
+
+// Wait for the stream; the scalars are those its last kernel put into pinned memory.
+Status await_scalars(Store& s, uint64_t* out) {
+  Status st = cuda_check(cudaStreamSynchronize(s.stream), "stream sync");
+  if (st.ok()) std::memcpy(out, s.h_scalars.p, 16 * sizeof(uint64_t));
   return st;
 }
 
@@ -2523,18 +2595,23 @@ void launch_verify_long(Store& s, const GroupArgs& g, const VerifyArgs& v, uint6
                     verify_ws_bytes<K>(), g, v);
 }
 
+// The pairs k_group_verify left (at most `count`).
+Status launch_pairs(Store& s, const GroupArgs& g, const VerifyArgs& v, uint64_t count) {
+  if (v.key64) launch_verify_long<uint64_t>(s, g, v, count);
+  else launch_verify_long<uint32_t>(s, g, v, count);
+  return launch_check("k_verify_long");
+}
+
 // Exact comparison of `count` nodes (of `list`, or all) with the head of their
-// hash: the short signatures, then the pairs left to k_verify_long.
-Status launch_verify(Store& s, const GroupArgs& g, const VerifyArgs& v, const uint32_t* list, uint64_t count) {
+// hash: the short signatures, then (with_pairs) the others.
+Status launch_verify(Store& s, const GroupArgs& g, const VerifyArgs& v, const uint32_t* list, uint64_t count,
+                     bool with_pairs) {
   static int cached[64];
   const unsigned res = resident_grid(k_group_verify, kVerNodeThreads, 0, s.device, cached);
   launch_chained(s, k_group_verify, (unsigned)std::min<uint64_t>(grid_for(count, kVerTile), res), kVerNodeThreads,
                     0, g, v, list, count);
-  if (v.mode != 0) {
-    if (v.key64) launch_verify_long<uint64_t>(s, g, v, count);
-    else launch_verify_long<uint32_t>(s, g, v, count);
-  }
-  return launch_check("exact comparison");
+  Status st = launch_check("k_group_verify");
+  return st.ok() && v.mode != 0 && with_pairs ? launch_pairs(s, g, v, count) : st;
 }
 
 // After a first insert + verify pass (scalars in h): regroup the nodes a hash
@@ -2551,6 +2628,7 @@ Status settle_unresolved(Store& s, const GroupArgs& g, const VerifyArgs& v, uint
     const uint64_t cap = table_capacity(unresolved_n);
     GroupArgs g2 = g;
     g2.tmask = cap - 1;
+    g2.alone = nullptr;  // no listed node is (the flags may be the new level's already)
     VerifyArgs v2 = v;
     v2.out_list = ptr<uint32_t>(s.ulist[cur ^ 1]);
     v2.n_out = sc + 5;
@@ -2560,7 +2638,7 @@ Status settle_unresolved(Store& s, const GroupArgs& g, const VerifyArgs& v, uint
       cudaMemsetAsync(sc + 5, 0, 16, s.stream);   // [5] and [6]
       cudaMemsetAsync(sc + 10, 0, 8, s.stream);
       launch_insert(s, g2, ptr<uint32_t>(s.ulist[cur]), unresolved_n);
-      st = launch_verify(s, g2, v2, ptr<uint32_t>(s.ulist[cur]), unresolved_n);
+      st = launch_verify(s, g2, v2, ptr<uint32_t>(s.ulist[cur]), unresolved_n, true);
     }
     if (!st.ok()) return st;
     if (!(st = read_scalars(s, h)).ok()) return st;
@@ -2659,6 +2737,7 @@ uint64_t insert_count(const Store& s, bool use_alone) {
 // the comparison of long signatures takes its pairs' number from the device,
 // and the numbering is launched before the host knows whether a hash collision
 // left nodes unresolved; if one did they are settled and it runs again.
+// `first`: a level whose blocks are few, so that long signatures repeat.
 // `keep`: hbits and rep hold the level before (Store::heads_level).
 // *hub_flags (mode 1): overflow flags of the hub passes before; when set, the
 // signatures were incomplete and nothing else is returned.
@@ -2667,11 +2746,11 @@ uint64_t insert_count(const Store& s, bool use_alone) {
 //  [1] unresolved after the first pass, [2] key total, [3] largest signature,
 //  [4] collided nodes, [5] unresolved after a repair pass, [6] and [10] pairs
 //  with long and with middle signatures, [7] error flags copy, [8] nodes alone
-//  in their block, [9] ticket of k_head_ranks, [11] nodes the filter left to
+//  in their block, [9] and [12] tickets of k_head_ranks and k_pid_fill, [11] nodes the filter left to
 //  the grouping, [15] the number of blocks.
 Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint32_t* pid, uint64_t* blocks,
                       uint64_t* collided, bool with_stats, uint64_t* keys, uint64_t* maxsig, bool use_alone,
-                      bool keep, uint32_t* hub_flags) {
+                      bool first, bool keep, uint32_t* hub_flags) {
   const uint64_t n = s.n, na = s.n_alive;
   Status st;
   unsigned long long* sc = ptr<unsigned long long>(s.d_scalars);
@@ -2681,6 +2760,10 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
   VerifyArgs v = verify_args(s, mode, prev, key64);
   v.keep = keep;
   const uint64_t words = (n + 31) / 32;
+  // the comparison of longer signatures runs unless the level before had none
+  // (the host sees their number at the end, and then compares them and
+  // numbers the blocks again)
+  const bool with_pairs = first || s.checked || s.pairs_last;
   uint64_t h[16] = {0};
   // canonical renumbering
   RankArgs r;
@@ -2695,6 +2778,7 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
   r.member = ptr<uint8_t>(s.member);
   r.alone = ptr<uint8_t>(s.alone);
   r.pid = pid;
+  r.host = ptr<unsigned long long>(s.h_scalars);
   r.stats = sc;
   auto renumber = [&]() -> Status {
     static int cached[64];
@@ -2733,8 +2817,8 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
       launch_insert(s, g, list, na);
     }
     if (!(st = launch_check("k_group_insert")).ok()) return st;
-    TimedScope ts(s, KBISIM_KERNEL_VERIFY, mode ? 2 : 1);
-    if (!(st = launch_verify(s, g, v, list, na)).ok()) return st;
+    TimedScope ts(s, KBISIM_KERNEL_VERIFY, mode && with_pairs ? 2 : 1);
+    if (!(st = launch_verify(s, g, v, list, na, with_pairs)).ok()) return st;
     g.d_count = nullptr;
   }
   if (s.checked) {  // representatives are checked before the numbering uses them
@@ -2743,14 +2827,25 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
     if (!(st = check_below(s, g.rep, na, n, "block heads")).ok()) return st;
   }
   if (!(st = renumber()).ok()) return st;
-  if (!(st = read_scalars(s, h)).ok()) return st;
+  if (!n) {
+    *blocks = *collided = s.n_alone = 0;
+    return read_scalars(s, h);
+  }
+  if (!(st = await_scalars(s, h)).ok()) return st;
   if (hub_flags && (*hub_flags = (uint32_t)h[7] & (kErrHubOverflow | kErrHubSet))) return Status::Ok();
-  if (h[1] && !s.checked) {
+  const bool missed = !with_pairs && mode && (h[6] || h[10]);
+  s.pairs_last = h[6] || h[10];
+  if ((h[1] || missed) && !s.checked) {
+    if (missed) {
+      TimedScope ts(s, KBISIM_KERNEL_VERIFY, 1);
+      if (!(st = launch_pairs(s, g, v, na)).ok()) return st;
+      if (!(st = read_scalars(s, h)).ok()) return st;
+    }
     if (!(st = settle_unresolved(s, g, v, h)).ok()) return st;
-    cudaMemsetAsync(sc + 2, 0, 16, s.stream);  // [2] and [3]
-    cudaMemsetAsync(sc + 8, 0, 16, s.stream);  // [8] and [9]
+    cudaMemsetAsync(sc + 2, 0, 16, s.stream);      // [2] and [3]
+    cudaMemsetAsync(sc + 8, 0, 5 * 8, s.stream);   // [8] .. [12]
     if (!(st = renumber()).ok()) return st;
-    if (!(st = read_scalars(s, h)).ok()) return st;
+    if (!(st = await_scalars(s, h)).ok()) return st;
   }
   *collided = h[4];
   *blocks = n ? h[15] : 0;  // heads
@@ -2836,6 +2931,8 @@ Status launch_hubs(Store& s, const SigArgs& a, bool cleared) {
   h.cursor = ptr<uint32_t>(s.hub_cursor);
   h.hub_cur = ptr<unsigned long long>(s.hub_acc);
   h.hub_term = reinterpret_cast<uint32_t*>(h.hub_cur + s.n_hub);
+  const bool small = s.m <= kChainEdges;
+  h.done = small ? reinterpret_cast<uint32_t*>(h.hub_cur + 2 * s.n_hub) : nullptr;
   h.tmp = s.hub_tmp.p;
   h.mode = ptr<uint8_t>(s.hub_mode);
   h.force = ptr<uint8_t>(s.hub_force);
@@ -2843,19 +2940,23 @@ Status launch_hubs(Store& s, const SigArgs& a, bool cleared) {
   // each hub's chunks run either the deduplicating pass or the plain
   // scatter, as its key sample says; both kernels cover all chunks and
   // skip those of the other kind
-  TimedScope ts(s, KBISIM_KERNEL_SIG_HUB, 5);
+  TimedScope ts(s, KBISIM_KERNEL_SIG_HUB, small ? 3 : 5);
   if (!cleared) {
     cudaMemsetAsync(h.cursor, 0, s.n_hub_buckets * 4, s.stream);
     cudaMemsetAsync(s.hub_acc.p, 0, s.n_hub * 24, s.stream);
     cudaMemsetAsync(s.hub_err.p, 0, s.n_hub * 4, s.stream);
   }
   launch_chained(s, k_hub_sample<LabelT, K>, (unsigned)((s.n_hub + 7) / 8), 256, 0, a, h, s.n_hub);
-  launch_chained(s, k_hub_chunk<LabelT, K>, (unsigned)s.n_hub_chunks, kChunkThreads, hub_chunk_smem<K>(), a, h);
-  launch_chained(s, k_hub_scatter<LabelT, K>, (unsigned)s.n_hub_chunks, kChunkThreads, 0, a, h);
+  if (small) {
+    launch_chained(s, k_hub_pieces<LabelT, K>, (unsigned)s.n_hub_chunks, kChunkThreads, hub_chunk_smem<K>(), a, h);
+  } else {
+    launch_chained(s, k_hub_chunk<LabelT, K>, (unsigned)s.n_hub_chunks, kChunkThreads, hub_chunk_smem<K>(), a, h);
+    launch_chained(s, k_hub_scatter<LabelT, K>, (unsigned)s.n_hub_chunks, kChunkThreads, 0, a, h);
+  }
   if (s.hub_ucap == (uint32_t)kHubUcaps[1]) launch_hub_bucket<K, kHubUcaps[1]>(s, a, h);
   else if (s.hub_ucap == (uint32_t)kHubUcaps[2]) launch_hub_bucket<K, kHubUcaps[2]>(s, a, h);
   else launch_hub_bucket<K, kHubUcaps[0]>(s, a, h);
-  launch_chained(s, k_hub_finish, (unsigned)((s.n_hub + 255) / 256), 256, 0, a, h, s.n_hub);
+  if (!small) launch_chained(s, k_hub_finish, (unsigned)((s.n_hub + 255) / 256), 256, 0, a, h, s.n_hub);
   return launch_check("hub kernels");
 }
 
@@ -3341,6 +3442,7 @@ constexpr int kL0RankThreads = 1024;
 
 __global__ void __launch_bounds__(kL0RankThreads) k_l0_rank(const unsigned long long* gtab, const uint32_t* gcnt,
                                                             uint32_t* rank, uint32_t* err, unsigned long long* stats) {
+  // stats: pinned host memory
   overlap_next();
   overlap_wait();
   __shared__ uint32_t ids[kL0Slots / 2];
@@ -3433,7 +3535,8 @@ Status level0_few_labels(Store& s, bool* done) {
     k_clear<<<8, kClearThreads, 0, s.stream>>>(c);
     const unsigned g = (unsigned)std::min<uint64_t>(grid_for(na, 2048), (uint64_t)sms * 8);
     launch_chained(s, k_l0_collect, g, kL0Threads, 0, na, ptr<uint32_t>(s.nlabel), ptr<uint32_t>(s.p2o), gtab, gcnt, err);
-    launch_chained(s, k_l0_rank, 1, kL0RankThreads, 0, gtab, gcnt, grank, err, sc);
+    launch_chained(s, k_l0_rank, 1, kL0RankThreads, 0, gtab, gcnt, grank, err,
+                   ptr<unsigned long long>(s.h_scalars));
   }
   if (!(st = launch_check("k_l0_collect")).ok()) return st;
   {
@@ -3444,7 +3547,7 @@ Status level0_few_labels(Store& s, bool* done) {
   }
   if (!(st = launch_check("k_l0_fill")).ok()) return st;
   uint64_t h[16];
-  if (!(st = read_scalars(s, h)).ok()) return st;
+  if (!(st = await_scalars(s, h)).ok()) return st;
   if (h[7]) return Status::Ok();  // too many labels: the general path
   if (s.checked && !(st = check_below(s, ptr<uint32_t>(s.level[0]), na, h[15], "identifiers")).ok()) return st;
   s.counts[0] = h[15];
@@ -3471,7 +3574,7 @@ Status compute_level0(Store& s) {
   if (!(st = launch_check("k_label_hash")).ok()) return st;
   uint64_t blocks_out = 0, coll = 0;
   st = group_and_rank(s, 0, nullptr, false, ptr<uint32_t>(s.level[0]), &blocks_out, &coll, false, nullptr,
-                      nullptr, false, false, nullptr);
+                      nullptr, false, true, false, nullptr);
   if (!st.ok()) return st;
   s.counts[0] = blocks_out;
   return Status::Ok();
@@ -3566,7 +3669,7 @@ Status compute_round(Store& s, uint32_t i) {
   for (int attempt = 0;; ++attempt) {
     uint32_t hub_flags = 0;
     st = group_and_rank(s, 1, a.prev, key64, ptr<uint32_t>(s.level[i]), &blocks, &coll, true, &keys, &maxsig, true,
-                        keep, &hub_flags);
+                        i <= 1, keep, &hub_flags);
     if (!st.ok()) return st;
     if (!hub_flags) break;
     if (attempt >= kHubAttempts) return Status::Err(KBISIM_ERR_TIMEOUT, "hub bucket overflow persists");
@@ -3626,7 +3729,7 @@ Status group_list(Store& s, const uint32_t* list, uint64_t count, const uint32_t
   {
     TimedScope ts(s, KBISIM_KERNEL_GROUP, 3);
     launch_insert(s, g, list, count);
-    st = launch_verify(s, g, v, list, count);
+    st = launch_verify(s, g, v, list, count, true);
   }
   if (!st.ok()) return st;
   uint64_t h[16];

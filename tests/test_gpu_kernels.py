@@ -165,3 +165,28 @@ def test_level0_table_limit(labels):
     with KBisim() as kb:
         res = kb.build(g, 2)
         assert_same(res, kb.all_pids(2), oracle_levels(g, 2))
+
+
+@pytest.mark.parametrize("width", [12, 64, 70])
+@pytest.mark.parametrize("checked", [False, True])
+def test_long_signatures_that_first_repeat_at_level_2(width, checked):
+    """Level 1 leaves no long signatures to compare, level 2 does: pairs of nodes over the same `width` children,
+    which differ only in their own children."""
+    pairs = 30
+    child0, leaf0 = 2 * pairs, 2 * pairs + width
+    src, dst = [], []
+    for a in range(2 * pairs):
+        skip = a // 2 if a // 2 < width else None  # most pairs leave out one child: other signatures, same length
+        src += [a] * (width - (skip is not None))
+        dst += [child0 + j for j in range(width) if j != skip]
+    src += list(range(child0, leaf0))
+    dst += list(range(leaf0, leaf0 + width))
+    labels = [0] * (2 * pairs) + [1] * width + list(range(2, 2 + width))
+    g = synth.from_coo(leaf0 + width, src, dst, [0] * len(src), labels)
+    ref = oracle_levels(g, 4)
+    with KBisim(checked=checked) as kb:
+        for _ in range(2):
+            res = kb.build(g, 4)
+            assert_same(res, kb.all_pids(4), ref)
+            res = kb.refine(4)
+            assert_same(res, kb.all_pids(4), ref)
