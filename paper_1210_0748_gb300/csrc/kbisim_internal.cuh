@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -172,8 +173,8 @@ struct ManyState {
   Buf dstart;                                  // uint64 [G+1]
   Buf gid, gidp;                               // uint32 [n] graph of each original / internal node
   Buf tkey, tmin, slot;                        // (graph, union block) -> smallest original id
-  Buf hbits, hword, cnt;                       // head bitmap, per-word prefix, per-graph prefix
-  Buf live, live_mask;                         // uint8 [G] graph still refined; bitmap over internal ids
+  Buf hbits, hword, cnt;                       // head bitmap, per-word ranks, per-graph prefix and scalars (two levels)
+  Buf live, live_mask;                         // uint32 [G] k of each graph; bitmap over internal ids
   uint64_t live_graphs = 0;                    // graphs refined in the next round
 };
 
@@ -419,6 +420,20 @@ Status timer_collect(Store& s);
 void timer_destroy(Store& s);
 // Exclusive prefix sum of a uint64 array in place (kbisim_round.cu).
 Status scan_u64(Store& s, uint64_t* a, uint64_t n);
+// Up to 8 arrays filled with a word each, in one launch; their sizes are
+// rounded up to 16 bytes (the arrays must be allocated so).
+struct ClearRange {
+  void* p;
+  uint64_t bytes;
+  uint32_t word;
+};
+Status clear_arrays(Store& s, std::initializer_list<ClearRange> ranges);
+// Ranks of the heads marked in a bitmap over original ids: hrank[w] = (word w,
+// heads before it in its tile), s.bsum as uint32 = heads before each tile of
+// 2^kRankTileShift ids; ticket_total[0] must be zero, [1] receives the number
+// of heads.
+constexpr int kRankTileShift = 15;
+Status rank_heads(Store& s, const uint32_t* hbits, uint64_t words, uint2* hrank, unsigned long long* ticket_total);
 
 // Incremental maintenance (kbisim_maint.cu).  maint_build makes the state for
 // levels 1..k of the loaded graph from its canonical levels (which must be

@@ -46,19 +46,81 @@ __global__ void k_many_gid(uint64_t n, const uint64_t* start, uint32_t G, uint32
   }
 }
 
-// gidp[p] = graph of internal node p; every edge must stay in its graph.
-// One warp per node (hubs included).
-__global__ void k_many_check(uint64_t n, const uint64_t* off, const uint32_t* dst, const uint32_t* p2o,
-                             const uint32_t* gid, uint32_t* gidp, uint32_t* err) {
-  const uint32_t lane = threadIdx.x & 31;
-  const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x / 32);
+// gidp[p] = graph of internal node p.
+__global__ void k_many_gidp(uint64_t n, const uint32_t* p2o, const uint32_t* gid, uint32_t* gidp) {
+  for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < n; p += (uint64_t)gridDim.x * blockDim.x)
+    gidp[p] = gid[p2o[p]];
+}
+
+// Every edge must stay in its graph.  Bound by the gather of the target's
+// graph: one per edge, kCheckItems of a lane in flight.  (A warp per node,
+// whatever its degree, with two gathers per edge took 790 us for 4.6M nodes
+// and 37M edges.)
+constexpr int kCheckItems = 4;
+
+__device__ __forceinline__ bool check_run(uint64_t b, uint64_t e, uint32_t g, uint32_t rank, uint32_t threads,
+                                          const uint32_t* dst, const uint32_t* gidp) {
   bool bad = false;
-  for (uint64_t p = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / 32; p < n; p += warps) {
-    const uint32_t g = gid[p2o[p]];
-    if (lane == 0) gidp[p] = g;
-    for (uint64_t e = off[p] + lane; e < off[p + 1]; e += 32) bad |= gid[p2o[dst[e]]] != g;
+  for (uint64_t i0 = b + rank; i0 < e; i0 += (uint64_t)threads * kCheckItems) {
+    uint32_t v[kCheckItems];
+#pragma unroll
+    for (int t = 0; t < kCheckItems; ++t)
+      if (i0 + (uint64_t)t * threads < e) v[t] = dst[i0 + (uint64_t)t * threads];
+#pragma unroll
+    for (int t = 0; t < kCheckItems; ++t)
+      if (i0 + (uint64_t)t * threads < e) bad |= gidp[v[t]] != g;
+  }
+  return bad;
+}
+
+// Out-degree <= 64: a warp per 32 consecutive nodes, whose edges are one
+// contiguous range; an edge's node by binary search over the lanes' offsets.
+__global__ void k_many_check_small(uint64_t n, const uint64_t* off, const uint32_t* dst, const uint32_t* gidp,
+                                   uint32_t* err) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  bool bad = false;
+  for (uint64_t w = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w * 32 < n; w += warps) {
+    const uint64_t p = w * 32 + lane;
+    const uint64_t base = off[w * 32], end = off[min(w * 32 + 32, n)];
+    const uint32_t r = (uint32_t)((p < n ? off[p] : end) - base), T = (uint32_t)(end - base);
+    const uint32_t g = p < n ? gidp[p] : 0u;
+    for (uint32_t k0 = 0; k0 < T; k0 += 32 * kCheckItems) {
+      uint32_t v[kCheckItems], ge[kCheckItems];
+#pragma unroll
+      for (int t = 0; t < kCheckItems; ++t) {
+        const uint32_t k = min(k0 + 32 * t + lane, T - 1);
+        v[t] = dst[base + k];
+        uint32_t j = 0;
+#pragma unroll
+        for (uint32_t step = 16; step; step >>= 1)
+          if (__shfl_sync(kFullMask, r, j + step) <= k) j += step;
+        ge[t] = __shfl_sync(kFullMask, g, j);
+      }
+#pragma unroll
+      for (int t = 0; t < kCheckItems; ++t) bad |= gidp[v[t]] != ge[t];
+    }
   }
   if (__any_sync(kFullMask, bad) && lane == 0) atomicOr(err, kErrBadInput);
+}
+
+// Larger nodes p0 .. p1-1: a warp per node; hubs: a CTA per chunk.
+__global__ void k_many_check_large(uint64_t p0, uint64_t p1, const uint64_t* off, const uint32_t* dst,
+                                   const uint32_t* gidp, uint32_t* err) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  bool bad = false;
+  for (uint64_t p = p0 + (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); p < p1; p += warps)
+    bad |= check_run(off[p], off[p + 1], gidp[p], lane, 32u, dst, gidp);
+  if (__any_sync(kFullMask, bad) && lane == 0) atomicOr(err, kErrBadInput);
+}
+
+__global__ void k_many_check_hub(uint64_t hub_first, const uint4* chunks, const uint32_t* dst, const uint32_t* gidp,
+                                 uint32_t* err) {
+  const uint4 c = chunks[blockIdx.x];
+  const uint64_t b = ((uint64_t)c.z << 32) | c.y;
+  const bool bad = check_run(b, b + c.w, gidp[hub_first + c.x], threadIdx.x, blockDim.x, dst, gidp);
+  if (__any_sync(kFullMask, bad) && (threadIdx.x & 31) == 0) atomicOr(err, kErrBadInput);
 }
 
 struct ManyArgs {
@@ -74,7 +136,8 @@ struct ManyArgs {
   uint64_t tmask;
   uint32_t* slot;          // per internal node: its key's slot
   uint32_t* hbits;         // head bitmap over original ids
-  const uint64_t* hword;   // heads before each bitmap word
+  const uint2* hrank;      // (bitmap word, heads before it in its tile)
+  const uint32_t* tbase;   // heads before each tile
   uint32_t* err;
 };
 
@@ -99,27 +162,39 @@ __global__ void __launch_bounds__(kThreads) k_many_insert(ManyArgs a) {
   __shared__ unsigned int smin[kAggSlots];
   __shared__ unsigned int sglob[kAggSlots];
   for (uint64_t base = (uint64_t)blockIdx.x * kAggChunk; base < a.n_alive; base += (uint64_t)gridDim.x * kAggChunk) {
+    uint32_t ls[kAggItems], oo[kAggItems];
+    uint64_t pp[kAggItems];
+    unsigned long long kk[kAggItems];
+    bool any = false;
+#pragma unroll
+    for (int t = 0; t < kAggItems; ++t) {
+      const uint64_t p = base + threadIdx.x + (uint64_t)t * kThreads;
+      ls[t] = p < a.n_alive && !a.alone[p] ? 0u : kNone32;
+      pp[t] = p;
+      any |= ls[t] == 0u;
+    }
+    if (!__syncthreads_or(any)) continue;  // (most chunks of a late level)
+#pragma unroll
+    for (int t = 0; t < kAggItems; ++t) {
+      if (ls[t] == kNone32) continue;
+      kk[t] = ((unsigned long long)a.gidp[pp[t]] << 32) | a.lvl[pp[t]];
+      oo[t] = a.p2o[pp[t]];
+    }
     for (int i = threadIdx.x; i < kAggSlots; i += kThreads) {
       skey[i] = kEmpty64;
       smin[i] = kNone32;
     }
     __syncthreads();
-    uint32_t ls[kAggItems];
-    uint64_t pp[kAggItems];
 #pragma unroll
     for (int t = 0; t < kAggItems; ++t) {
-      const uint64_t p = base + threadIdx.x + (uint64_t)t * kThreads;
-      ls[t] = kNone32;
-      pp[t] = p;
-      if (p >= a.n_alive || a.alone[p]) continue;
-      const unsigned long long key = ((unsigned long long)a.gidp[p] << 32) | a.lvl[p];
-      uint32_t s = (uint32_t)(mix64(key) & (kAggSlots - 1));
+      if (ls[t] == kNone32) continue;
+      uint32_t s = (uint32_t)(mix64(kk[t]) & (kAggSlots - 1));
       for (int q = 0; q < kAggSlots; ++q) {  // at most kAggChunk distinct keys: always room
-        const unsigned long long cur = atomicCAS(&skey[s], (unsigned long long)kEmpty64, key);
-        if (cur == kEmpty64 || cur == key) break;
+        const unsigned long long cur = atomicCAS(&skey[s], (unsigned long long)kEmpty64, kk[t]);
+        if (cur == kEmpty64 || cur == kk[t]) break;
         s = (s + 1) & (kAggSlots - 1);
       }
-      atomicMin(&smin[s], a.p2o[p]);
+      atomicMin(&smin[s], oo[t]);
       ls[t] = s;
     }
     __syncthreads();
@@ -142,14 +217,9 @@ __global__ void k_many_heads(ManyArgs a) {
   }
 }
 
-__global__ void k_many_word_counts(const uint32_t* hbits, uint64_t words, uint64_t* hword) {
-  for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w < words; w += (uint64_t)gridDim.x * blockDim.x)
-    hword[w] = __popc(hbits[w]);
-}
-
 __device__ __forceinline__ uint64_t heads_before(const ManyArgs& a, uint64_t x) {
-  const uint64_t w = x >> 5;
-  return a.hword[w] + (uint64_t)__popc(a.hbits[w] & ((1u << (x & 31)) - 1u));
+  const uint2 r = a.hrank[x >> 5];
+  return (uint64_t)a.tbase[x >> kRankTileShift] + r.y + (uint64_t)__popc(r.x & ((1u << (x & 31)) - 1u));
 }
 
 // Per-graph identifier of every node (original order): rank of its head
@@ -166,57 +236,33 @@ __global__ void k_many_pid(ManyArgs a, uint64_t n, const uint64_t* start, uint32
   }
 }
 
-// cnt[j] = heads before start[j] (j <= G).
+// cnt[j] = heads before start[j] (j <= G); cnt[G + 1] = the error flags.
 __global__ void k_many_counts(ManyArgs a, const uint64_t* start, uint32_t G, unsigned long long* cnt) {
   for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j <= G; j += gridDim.x * blockDim.x)
     cnt[j] = heads_before(a, start[j]);
+  if (blockIdx.x == 0 && threadIdx.x == 0) cnt[G + 1] = *a.err;
 }
 
-// Work list of the next round: nodes of the graphs still refined.
-__global__ void k_many_live_mask(uint64_t n_alive, const uint32_t* gidp, const uint8_t* live, uint32_t* mask) {
-  for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w * 32 < n_alive;
-       w += (uint64_t)gridDim.x * blockDim.x) {
-    uint32_t bits = 0;
-    for (uint32_t b = 0; b < 32; ++b) {
-      const uint64_t p = w * 32 + b;
-      if (p < n_alive && live[gidp[p]]) bits |= 1u << b;
+// Work list of the next round: nodes of the graphs still refined after level l
+// (l < k, and with early stop the level before had fewer blocks), from the
+// counts of this level and the one before, so that the host need not be asked.
+__global__ void k_many_live_mask(uint64_t n_alive, const uint32_t* gidp, const uint32_t* k, uint32_t l, bool early_stop,
+                                 const unsigned long long* cnt, const unsigned long long* cnt_before, uint32_t* mask) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  for (uint64_t w = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w * 32 < n_alive; w += warps) {
+    const uint64_t p = w * 32 + lane;
+    bool live = false;
+    if (p < n_alive) {
+      const uint32_t g = gidp[p];
+      live = l < k[g] && !(early_stop && l >= 1 && cnt[g + 1] - cnt[g] == cnt_before[g + 1] - cnt_before[g]);
     }
-    mask[w] = bits;
+    const uint32_t bits = __ballot_sync(kFullMask, live);
+    if (lane == 0) mask[w] = bits;
   }
 }
 
 }  // namespace
-
-// After level l: the graphs that still need a round (l < k_j, and with early
-// stop not yet stable) form the next round's work list; the others keep their
-// blocks (their nodes are not signed again).  Only set while some graph has
-// stopped and others go on.
-Status many_work_list(Store& s, uint32_t l) {
-  ManyState& m = s.many;
-  s.round_mask = nullptr;
-  std::vector<uint8_t> live(m.G, 0);
-  uint64_t nlive = 0;
-  for (uint32_t j = 0; j < m.G; ++j) {
-    bool go = l < m.k[j];
-    if (go && s.early_stop && l >= 1 && m.counts[l][j] == m.counts[l - 1][j]) go = false;
-    live[j] = go ? 1 : 0;
-    nlive += go ? 1 : 0;
-  }
-  m.live_graphs = nlive;
-  if (nlive == 0 || nlive == m.G) return Status::Ok();
-  Status st;
-  const uint64_t words = s.n_alive / 32 + 1;
-  if (!(st = ensure(s, m.live, m.G)).ok()) return st;
-  if (!(st = ensure(s, m.live_mask, words * 4)).ok()) return st;
-  st = cuda_check(cudaMemcpyAsync(m.live.p, live.data(), m.G, cudaMemcpyHostToDevice, s.stream), "live graphs");
-  if (!st.ok()) return st;
-  k_many_live_mask<<<grid_for(words, kThreads, s.sms * 16), kThreads, 0, s.stream>>>(
-      s.n_alive, ptr<uint32_t>(m.gidp), ptr<uint8_t>(m.live), ptr<uint32_t>(m.live_mask));
-  st = cuda_check(cudaGetLastError(), "live mask");
-  if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "live mask");  // the host vector goes away
-  if (st.ok()) s.round_mask = ptr<uint32_t>(m.live_mask);
-  return st;
-}
 
 // Per-graph renumbering of level l (called right after the union computed it).
 Status many_level(Store& s, uint32_t l) {
@@ -226,15 +272,19 @@ Status many_level(Store& s, uint32_t l) {
   Status st;
   if (m.lvl.size() < (size_t)l + 1) m.lvl.resize(l + 1);
   if (!(st = ensure(s, m.lvl[l], std::max<uint64_t>(n, 1) * 4)).ok()) return st;
-  if (!(st = ensure(s, m.hbits, words * 4)).ok()) return st;
+  if (!(st = ensure(s, m.hbits, words * 4 + 16)).ok()) return st;
   if (!(st = ensure(s, m.hword, words * 8)).ok()) return st;
-  if (!(st = ensure(s, m.cnt, (m.G + 1) * 8)).ok()) return st;
+  const uint64_t per = m.G + 4;  // counts of a level: [G + 1], error flags, ticket, number of heads
+  if (!(st = ensure(s, m.cnt, 2 * per * 8)).ok()) return st;
+  if (!(st = ensure(s, m.live_mask, (na / 32 + 1) * 4)).ok()) return st;
   const uint64_t ins = na - std::min(na, s.n_alone);
   uint64_t cap = 1024;
   while (cap < 2 * ins) cap <<= 1;
   if (!(st = ensure(s, m.tkey, cap * 8)).ok()) return st;
   if (!(st = ensure(s, m.tmin, cap * 4)).ok()) return st;
   if (!(st = ensure(s, m.slot, std::max<uint64_t>(na, 1) * 4)).ok()) return st;
+  unsigned long long* cnt = ptr<unsigned long long>(m.cnt) + (l & 1) * per;
+  const unsigned long long* cnt_before = ptr<unsigned long long>(m.cnt) + ((l + 1) & 1) * per;
   ManyArgs a;
   a.n_alive = na;
   a.lvl = ptr<uint32_t>(s.level[l]);
@@ -248,41 +298,43 @@ Status many_level(Store& s, uint32_t l) {
   a.tmask = cap - 1;
   a.slot = ptr<uint32_t>(m.slot);
   a.hbits = ptr<uint32_t>(m.hbits);
-  a.hword = ptr<uint64_t>(m.hword);
+  a.hrank = ptr<uint2>(m.hword);
   a.err = ptr<uint32_t>(s.d_err);
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s.device);
-  if (sms <= 0) sms = 132;
-  cudaMemsetAsync(m.tkey.p, 0xFF, cap * 8, s.stream);
-  cudaMemsetAsync(m.tmin.p, 0xFF, cap * 4, s.stream);
-  cudaMemsetAsync(m.hbits.p, 0, words * 4, s.stream);
+  cudaMemsetAsync(cnt + m.G + 2, 0, 8, s.stream);  // the ranks' ticket
+  if (!(st = clear_arrays(s, {{m.tkey.p, cap * 8, ~0u}, {m.tmin.p, cap * 4, ~0u}, {m.hbits.p, words * 4, 0u}})).ok())
+    return st;
   if (na) {
-    k_many_insert<<<grid_for(na, kAggChunk, (int)resident_blocks(k_many_insert, kThreads, 0, sms)), kThreads, 0,
+    k_many_insert<<<grid_for(na, kAggChunk, (int)resident_blocks(k_many_insert, kThreads, 0, s.sms)), kThreads, 0,
                     s.stream>>>(a);
-    k_many_heads<<<grid_for(na, kThreads, sms * 16), kThreads, 0, s.stream>>>(a);
+    k_many_heads<<<grid_for(na, kThreads, s.sms * 16), kThreads, 0, s.stream>>>(a);
   }
-  k_many_word_counts<<<grid_for(words, kThreads, sms * 16), kThreads, 0, s.stream>>>(ptr<uint32_t>(m.hbits), words,
-                                                                                      ptr<uint64_t>(m.hword));
-  if (!(st = scan_u64(s, ptr<uint64_t>(m.hword), words)).ok()) return st;
+  if (!(st = rank_heads(s, ptr<uint32_t>(m.hbits), words, ptr<uint2>(m.hword), cnt + m.G + 2)).ok()) return st;
+  a.tbase = ptr<uint32_t>(s.bsum);
+  k_many_counts<<<grid_for(m.G + 1, kThreads, 64), kThreads, 0, s.stream>>>(a, ptr<uint64_t>(m.dstart), m.G, cnt);
   if (n)
-    k_many_pid<<<grid_for(n, kThreads, sms * 16), kThreads, 0, s.stream>>>(a, n, ptr<uint64_t>(m.dstart),
+    k_many_pid<<<grid_for(n, kThreads, s.sms * 16), kThreads, 0, s.stream>>>(a, n, ptr<uint64_t>(m.dstart),
                                                                              ptr<uint32_t>(m.lvl[l]));
-  k_many_counts<<<grid_for(m.G + 1, kThreads, 64), kThreads, 0, s.stream>>>(a, ptr<uint64_t>(m.dstart), m.G,
-                                                                             ptr<unsigned long long>(m.cnt));
+  // the next round's work list, used while some graphs have stopped and others
+  // go on: the nodes of the others keep their blocks
+  if (na)
+    k_many_live_mask<<<grid_for(na, kThreads, s.sms * 16), kThreads, 0, s.stream>>>(
+        na, ptr<uint32_t>(m.gidp), ptr<uint32_t>(m.live), l, s.early_stop, cnt, cnt_before, ptr<uint32_t>(m.live_mask));
   if (!(st = cuda_check(cudaGetLastError(), "per-graph renumbering")).ok()) return st;
-  std::vector<uint64_t> c(m.G + 1);
-  st = cuda_check(cudaMemcpyAsync(c.data(), m.cnt.p, (m.G + 1) * 8, cudaMemcpyDeviceToHost, s.stream), "counts");
+  std::vector<uint64_t> c(m.G + 2);
+  st = cuda_check(cudaMemcpyAsync(c.data(), cnt, (m.G + 2) * 8, cudaMemcpyDeviceToHost, s.stream), "counts");
   if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "sync");
   if (!st.ok()) return st;
-  uint32_t e = 0;
-  st = cuda_check(cudaMemcpy(&e, s.d_err.p, 4, cudaMemcpyDeviceToHost), "error flags");
-  if (!st.ok()) return st;
-  if (e & kErrProbe) return Status::Err(KBISIM_ERR_TIMEOUT, "hash table probe bound exceeded");
+  if (c[m.G + 1] & kErrProbe) return Status::Err(KBISIM_ERR_TIMEOUT, "hash table probe bound exceeded");
   if (m.counts.size() < (size_t)l + 1) m.counts.resize(l + 1);
   m.counts[l].resize(m.G);
   for (uint32_t j = 0; j < m.G; ++j) m.counts[l][j] = c[j + 1] - c[j];
   m.levels = l + 1;
-  return many_work_list(s, l);
+  uint64_t nlive = 0;
+  for (uint32_t j = 0; j < m.G; ++j)
+    nlive += l < m.k[j] && !(s.early_stop && l >= 1 && m.counts[l][j] == m.counts[l - 1][j]) ? 1 : 0;
+  m.live_graphs = nlive;
+  s.round_mask = nlive && nlive < m.G ? ptr<uint32_t>(m.live_mask) : nullptr;
+  return Status::Ok();
 }
 
 Status many_check_args(const kbisim_graph* g, const uint64_t* start, uint32_t G, const uint32_t* k,
@@ -316,15 +368,24 @@ Status many_setup(Store& s, const uint64_t* start, uint32_t G, const uint32_t* k
   if (!(st = ensure(s, m.gidp, std::max<uint64_t>(n, 1) * 4)).ok()) return st;
   cudaMemcpyAsync(m.dstart.p, m.start.data(), (G + 1) * 8, cudaMemcpyHostToDevice, s.stream);
   cudaMemsetAsync(s.d_err.p, 0, 4, s.stream);
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s.device);
-  if (sms <= 0) sms = 132;
+  if (!(st = ensure(s, m.live, G * 4)).ok()) return st;
+  cudaMemcpyAsync(m.live.p, m.k.data(), G * 4, cudaMemcpyHostToDevice, s.stream);
   if (n) {
-    k_many_gid<<<grid_for(n, kThreads, sms * 16), kThreads, 0, s.stream>>>(n, ptr<uint64_t>(m.dstart), G,
-                                                                            ptr<uint32_t>(m.gid));
-    k_many_check<<<(unsigned)sms * 16, kThreads, 0, s.stream>>>(n, ptr<uint64_t>(s.offsets), ptr<uint32_t>(s.dst),
-                                                                 ptr<uint32_t>(s.p2o), ptr<uint32_t>(m.gid),
-                                                                 ptr<uint32_t>(m.gidp), ptr<uint32_t>(s.d_err));
+    const uint32_t* gidp = ptr<uint32_t>(m.gidp);
+    const uint64_t* off = ptr<uint64_t>(s.offsets);
+    const uint32_t* dst = ptr<uint32_t>(s.dst);
+    uint32_t* err = ptr<uint32_t>(s.d_err);
+    k_many_gid<<<grid_for(n, kThreads, s.sms * 16), kThreads, 0, s.stream>>>(n, ptr<uint64_t>(m.dstart), G,
+                                                                             ptr<uint32_t>(m.gid));
+    k_many_gidp<<<grid_for(n, kThreads, s.sms * 16), kThreads, 0, s.stream>>>(n, ptr<uint32_t>(s.p2o),
+                                                                              ptr<uint32_t>(m.gid), ptr<uint32_t>(m.gidp));
+    const uint64_t small = s.class_start[kClassWarp], hub = s.class_start[kClassHub];
+    if (small) k_many_check_small<<<grid_for(small, kThreads, s.sms * 16), kThreads, 0, s.stream>>>(small, off, dst, gidp, err);
+    if (hub > small)
+      k_many_check_large<<<grid_for((hub - small) * 32, kThreads, s.sms * 16), kThreads, 0, s.stream>>>(small, hub, off,
+                                                                                                        dst, gidp, err);
+    if (s.n_hub_chunks)
+      k_many_check_hub<<<(unsigned)s.n_hub_chunks, kThreads, 0, s.stream>>>(hub, ptr<uint4>(s.hub_chunks), dst, gidp, err);
   }
   uint32_t e = 0;
   st = cuda_check(cudaGetLastError(), "graph ids");

@@ -1890,7 +1890,6 @@ __device__ __forceinline__ void publish_scalars(const unsigned long long* stats,
 // launch instead of a word count, two tile passes and a scan of the tiles:
 // bound by launch latency (31K words at 1M nodes; 9.5 us for the four before).
 constexpr int kRankThreads = 256, kRankItems = 4, kRankTile = kRankThreads * kRankItems;
-constexpr int kRankTileShift = 10 + 5;  // original ids of a tile: 2^15
 static_assert(kRankTile * 32 == 1 << kRankTileShift, "tile of original ids");
 
 // Exclusive sum of v over the CTA; *total gets the CTA's sum.  red: NT / 32 words.
@@ -3288,6 +3287,27 @@ Status build_chunk_lists(Store& s, bool fresh) {
 }
 
 Status scan_u64(Store& s, uint64_t* a, uint64_t n) { return scan64(s, a, n, nullptr); }
+
+Status clear_arrays(Store& s, std::initializer_list<ClearRange> ranges) {
+  ClearArgs c;
+  uint64_t units = 0;
+  for (const ClearRange& r : ranges) {
+    c.add(r.p, r.bytes, r.word);
+    units += (r.bytes + 15) / 16;
+  }
+  k_clear<<<(unsigned)std::min<uint64_t>(grid_for(units, kClearThreads), (uint64_t)sm_count(s.device) * 8),
+            kClearThreads, 0, s.stream>>>(c);
+  return launch_check("k_clear");
+}
+
+Status rank_heads(Store& s, const uint32_t* hbits, uint64_t words, uint2* hrank, unsigned long long* ticket_total) {
+  const uint64_t tiles = (words + kRankTile - 1) / kRankTile;
+  Status st = ensure(s, s.bsum, std::max<uint64_t>(tiles, 64) * 8);
+  if (!st.ok()) return st;
+  launch_chained(s, k_head_ranks, (unsigned)tiles, kRankThreads, 0, hbits, words, hrank, ptr<uint32_t>(s.bsum),
+                 ticket_total, ticket_total + 1);
+  return launch_check("k_head_ranks");
+}
 
 Status relabel_graph(Store& s, const uint64_t* off0, const uint32_t* dst0, const void* lab0,
                      const uint32_t* nlab0, const uint8_t* alive0, uint32_t lab_bytes) {

@@ -190,3 +190,31 @@ def test_long_signatures_that_first_repeat_at_level_2(width, checked):
             assert_same(res, kb.all_pids(4), ref)
             res = kb.refine(4)
             assert_same(res, kb.all_pids(4), ref)
+
+
+@pytest.mark.parametrize("degree", [1, 40, 64, 65, 300, 4096, 4097, 9000])
+@pytest.mark.parametrize("bad", [False, True])
+def test_batch_finds_the_one_edge_between_graphs(degree, bad):
+    """An edge that leaves its graph is found whatever the out-degree of its source."""
+    from paper_1210_0748_gb300.kbisim import KBisimError, concat_graphs
+    rng = np.random.default_rng(degree)
+
+    def one(seed):
+        src = np.concatenate([np.zeros(degree, np.uint32), rng.integers(0, 200, 300).astype(np.uint32)])
+        dst = rng.integers(0, 200, src.size).astype(np.uint32)
+        return synth.from_coo(200, src, dst, rng.integers(0, 3, src.size), rng.integers(0, 3, 200))
+
+    graphs = [one(0), one(1), one(2)]
+    union, starts = concat_graphs(graphs)
+    if bad:
+        union.dst[int(union.offsets[200]) + degree - 1] = 199  # the last listed edges of graph 1's node 0 are its own
+    with KBisim() as kb:
+        if bad:
+            with pytest.raises(KBisimError):
+                kb.build_many(None, [2, 3, 1], union=(union, starts))
+            return
+        kb.build_many(None, [2, 3, 1], union=(union, starts))
+        for j, (g, k) in enumerate(zip(graphs, [2, 3, 1])):
+            ref = oracle_levels(g, k)
+            assert kb.many_info(j)[1].tolist() == ref.counts.tolist()
+            assert np.array_equal(kb.many_pids(j, k), ref.pids[k])
