@@ -1416,6 +1416,17 @@ __device__ __forceinline__ uint32_t table_insert(const GroupArgs& g, uint64_t tm
   return 0;
 }
 
+// Whether the CTA's tile of `tile` nodes from base on (a multiple of 4) holds a
+// node not alone in its previous block, by 4 flags a thread; called by the whole
+// CTA.  In late rounds most tiles hold none, and the grouping would pass through
+// its barriers for nothing (16M nodes, four rounds: 373 -> 252 us).
+__device__ __forceinline__ bool tile_has_work(const uint8_t* alone, uint64_t base, uint32_t tile, uint64_t count) {
+  if (base + tile > count) return true;
+  const bool mine = threadIdx.x * 4 < tile &&
+                    (reinterpret_cast<const uint32_t*>(alone + base)[threadIdx.x] & 0x01010101u) != 0x01010101u;
+  return __syncthreads_or(mine);
+}
+
 // A CTA takes 1024 nodes, combines equal hashes in shared memory (smallest
 // original id per hash), then inserts each distinct hash once.
 constexpr int kInsThreads = 256, kInsItems = 4, kInsChunk = kInsThreads * kInsItems, kInsSlots = 2 * kInsChunk;
@@ -1438,6 +1449,7 @@ __global__ void __launch_bounds__(kInsThreads) k_group_insert(GroupArgs g, const
   if (threadIdx.x == 0) n_used = 0;
   __syncthreads();
   for (uint64_t base = (uint64_t)blockIdx.x * kInsChunk; base < count; base += (uint64_t)gridDim.x * kInsChunk) {
+    if (g.alone && !list && !tile_has_work(g.alone, base, kInsChunk, count)) continue;
     // loads of all items first (node ids, then alone flags, then hashes and
     // original ids of the nodes that are grouped), so that they overlap
     uint32_t ls[kInsItems], pp[kInsItems], oo[kInsItems];
@@ -1679,7 +1691,7 @@ __device__ __forceinline__ void mark_unresolved(const VerifyArgs& v, uint32_t* r
 // ids and table slots; representatives; their fields; the short key lists).
 constexpr int kVerNodeThreads = 256, kVerItems = 2, kVerTile = kVerNodeThreads * kVerItems;
 
-__global__ void __launch_bounds__(kVerNodeThreads) k_group_verify(GroupArgs g, VerifyArgs v, const uint32_t* list,
+__global__ void __launch_bounds__(kVerNodeThreads, 5) k_group_verify(GroupArgs g, VerifyArgs v, const uint32_t* list,
                                                                    uint64_t count) {
   overlap_next();
   overlap_wait();
@@ -1699,6 +1711,12 @@ __global__ void __launch_bounds__(kVerNodeThreads) k_group_verify(GroupArgs g, V
     }
 #pragma unroll
     for (int t = 0; t < kVerItems; ++t) act[t] = p[t] != kNone32 && !(g.alone && g.alone[p[t]]);
+    if (v.keep) {  // (most warps of a late round; no barrier: warps go on by themselves)
+      bool any = false;
+#pragma unroll
+      for (int t = 0; t < kVerItems; ++t) any |= act[t];
+      if (!__any_sync(kFull, any)) continue;
+    }
 #pragma unroll
     for (int t = 0; t < kVerItems; ++t) {
       if (!act[t] && v.keep) p[t] = kNone32;
@@ -1999,12 +2017,13 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(uint64_t* bsum, uin
 // thread takes kFillItems nodes at a time and issues each step's loads for
 // all of them together (representatives; their original ids; the bitmap
 // words), so the three dependent gathers of a node overlap with the others'.
-// The grid is one resident wave and a CTA adds its counts with one atomic per
-// statistic: with one per warp the same-address atomics took most of the time
-// (1M nodes: 39 us a call, 16M: 106 us).
+// No load waits behind a store of the item before (the arrays might alias, so
+// the compiler keeps that order).  The grid is one resident wave and a CTA adds
+// its counts with one atomic per statistic: with one per warp the same-address
+// atomics took most of the time at 1M nodes (39 us a call).
 constexpr int kFillThreads = 256, kFillItems = 4;
 
-__global__ void __launch_bounds__(kFillThreads, 6) k_pid_fill(RankArgs r) {
+__global__ void __launch_bounds__(kFillThreads, 4) k_pid_fill(RankArgs r) {
   overlap_next();
   overlap_wait();
   __shared__ unsigned int s_alone, s_mx;
@@ -2018,14 +2037,20 @@ __global__ void __launch_bounds__(kFillThreads, 6) k_pid_fill(RankArgs r) {
   unsigned long long keys = 0;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t p0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p0 < r.n; p0 += stride * kFillItems) {
-    uint32_t h[kFillItems], o[kFillItems];
+    uint32_t h[kFillItems], o[kFillItems], u[kFillItems];
+    uint8_t mem[kFillItems];
     uint2 hr[kFillItems];
     bool live[kFillItems];
 #pragma unroll
     for (int t = 0; t < kFillItems; ++t) {
       const uint64_t p = p0 + (uint64_t)t * stride;
       live[t] = p < r.n_alive;
-      if (live[t]) h[t] = r.rep[p];
+      u[t] = 0;
+      if (live[t]) {
+        h[t] = r.rep[p];
+        mem[t] = r.member[p];
+        if (r.ucnt) u[t] = r.ucnt[p];
+      }
     }
     // a hash collision leaves nodes without a head: the fill runs again once
     // they are settled
@@ -2033,20 +2058,21 @@ __global__ void __launch_bounds__(kFillThreads, 6) k_pid_fill(RankArgs r) {
     for (int t = 0; t < kFillItems; ++t)
       if (live[t]) o[t] = h[t] < r.n_alive ? r.p2o[h[t]] : 0u;
 #pragma unroll
-    for (int t = 0; t < kFillItems; ++t)
-      if (live[t]) hr[t] = r.hrank[o[t] >> 5];
+    for (int t = 0; t < kFillItems; ++t) {
+      if (live[t]) {
+        hr[t] = r.hrank[o[t] >> 5];
+        hr[t].y += r.tbase[o[t] >> kRankTileShift];
+      }
+    }
 #pragma unroll
     for (int t = 0; t < kFillItems; ++t) {
       const uint64_t p = p0 + (uint64_t)t * stride;
       if (p >= r.n) break;
       if (live[t]) {
-        if (r.ucnt) {
-          const uint32_t q = r.ucnt[p];
-          keys += q;
-          mx = max(mx, q);
-        }
-        r.pid[p] = r.tbase[o[t] >> kRankTileShift] + hr[t].y + (uint32_t)__popc(hr[t].x & ((1u << (o[t] & 31)) - 1u));
-        const bool al = h[t] == (uint32_t)p && !r.member[p];
+        keys += u[t];
+        mx = max(mx, u[t]);
+        r.pid[p] = hr[t].y + (uint32_t)__popc(hr[t].x & ((1u << (o[t] & 31)) - 1u));
+        const bool al = h[t] == (uint32_t)p && !mem[t];
         r.alone[p] = al ? 1 : 0;
         n_alone += al ? 1u : 0u;
       } else {
