@@ -106,6 +106,9 @@ void trim_caches(Store& s) {
     for (Buf& b : s.spare_level) release(s, b);
     s.spare_level.clear();
     release(s, s.spare_alone);
+    release(s, s.dup);  // (only rounds use them)
+    release(s, s.alone_bits);
+    s.dup_valid = false;
   }
   // copies in original order whose results are no longer valid
   for (size_t l = 0; l < s.out_level.size(); ++l)
@@ -302,7 +305,7 @@ void free_graph(Store& s, bool keep_buffers) {
                  &s.hub_bbase, &s.hub_cap, &s.hub_tbase, &s.hub_chunks, &s.hub_cstart, &s.sigkey, &s.ucnt, &s.hash, &s.table,
                  &s.slot, &s.rep, &s.ulist[0], &s.ulist[1], &s.hbits, &s.member, &s.alone, &s.hword, &s.bsum,
                  &s.long_pairs, &s.hub_cursor, &s.bucket_hub, &s.hub_acc, &s.hub_mode, &s.hub_force, &s.hub_err, &s.hub_retry, &s.hub_tmp, &s.alive_o,
-                 &s.rl_tcnt, &s.rl_hot, &s.rl_ost};
+                 &s.rl_tcnt, &s.rl_hot, &s.rl_ost, &s.dup, &s.alone_bits};
   if (!keep_buffers) {
     for (Buf* b : bufs) release(s, *b);
     release(s, s.spare_alone);
@@ -654,7 +657,10 @@ Status refine(Store& s, uint32_t k, kbisim_result* out) {
   s.heads_level = -1;
   s.stats.clear();
   s.counts.assign(std::max<size_t>(snap.counts.size(), 1), 0);
-  Status st = refine_levels(s, k);
+  // the second refinement of an edge table marks its duplicate edges for this
+  // and later ones
+  Status st = s.refined && !s.dup_valid && k >= 2 ? mark_duplicates(s) : Status::Ok();
+  if (st.ok()) st = refine_levels(s, k);
   if (!st.ok()) {
     std::swap(s.level, s.spare_level);
     std::swap(s.alone, s.spare_alone);
@@ -664,6 +670,7 @@ Status refine(Store& s, uint32_t k, kbisim_result* out) {
   }
   invalidate_outputs(s);
   s.has_levels = true;
+  s.refined = true;
   fill_result(s, k, out);
   return timer_collect(s);
 }

@@ -235,6 +235,7 @@ struct Store {
   uint64_t hub_tmp_words = 0;  // key words of all hub buckets
   uint64_t n_hub_buckets = 0;
   uint64_t hub_edges = 0;
+  uint64_t hub_edge0 = 0;      // first hub edge
   std::vector<uint32_t> h_hub_xbits;  // per hub: more buckets, after a bucket's set filled
   std::vector<uint32_t> h_hub_shift;  // per hub: larger buckets, after a bucket's capacity was exceeded
   std::vector<uint8_t> h_hub_force;   // per hub: deduplicating chunk pass, after a scatter overflowed
@@ -269,6 +270,10 @@ struct Store {
   Buf alone;                   // uint8 [n] node is alone in its block at the last computed level
   Buf hword;                   // uint64 [(n+31)/32] heads before each bitmap word
   uint64_t n_alone = 0;        // nodes alone in their block at the last computed level
+  Buf dup;                     // bit per edge: repeats an earlier (label, target) of its node (out-degree > 32)
+  Buf alone_bits;              // alone as a bitmap, while dup is in use
+  bool dup_valid = false, dup_hubs = false;  // dup describes the edge table; the hubs' edges too
+  bool refined = false;        // the edge table has been refined from level 0
   bool pairs_last = true;      // the last round left signatures longer than a thread compares
   int64_t heads_level = -1;    // the level whose heads hbits and rep hold, while one call refines (-1 = none)
   Buf bsum;                    // uint64 scan block sums
@@ -391,6 +396,9 @@ Status relabel_graph(Store& s, const uint64_t* off0, const uint32_t* dst0, const
 // the store with the updated graph loaded and no levels.
 Status apply_batch(Store& s, const kbisim_batch* b, uint64_t* missing);
 Status compute_level0(Store& s);                  // pId_0 into level[0]
+// Mark the edges that repeat an earlier (label, target) of their node, for the
+// rounds of this edge table (once per table, when it is refined again).
+Status mark_duplicates(Store& s);
 // Work lists of the degree classes from s.offsets (after a relabel, or after
 // a batch applied in place); `fresh` drops what hub buckets learned.
 Status build_chunk_lists(Store& s, bool fresh);

@@ -351,6 +351,15 @@ struct SigArgs {
   // nodes alone in their previous block (NULL = not known): they stay alone, so
   // nothing reads their keys or hash, only their number of distinct elements
   const uint8_t* alone;
+  // With the edges that repeat an earlier (label, target) of their node marked
+  // (dup) and the nodes alone in their block as a bitmap (alone_bits), an
+  // unmarked edge to such a node is a distinct element by itself: nothing else
+  // of its node can equal it, so a node that only counts needs neither its key
+  // nor a place in a set for it.  NULL = not known.
+  const uint32_t* dup;
+  const uint32_t* alone_bits;
+  bool dup_hubs;    // the hubs' edges are marked too
+  uint32_t* mark;   // marking pass: output, a bit per edge (prev = identity, every node counts)
 };
 
 // The node is to be signed this pass (every node unless a frontier mask is set).
@@ -394,6 +403,51 @@ __device__ __forceinline__ void edge_key_batches(const SigArgs& a, uint64_t off,
     edge_keys<B, O, S, LabelT, K>(a, off + O, 1u, end, pol, key);
     edge_key_batches<O + B, B, S, LabelT, K>(a, off, end, pol, key);
   }
+}
+
+// Variants of the kernels for out-degree 33..4096: without marks, with a.dup
+// set, and the marking pass itself (each carries only its own code).
+enum { kPlain = 0, kWithDup = 1, kMarking = 2 };
+
+__device__ __forceinline__ void mark_dup(const SigArgs& a, uint64_t e) { atomicOr(&a.mark[e >> 5], 1u << (e & 31)); }
+
+// For a node that only counts: of N edges base + i * stride below end, the
+// number of unmarked ones to nodes alone in their block, and the keys of the
+// other unmarked ones (bits of the returned mask), for a set.  In late rounds
+// that is hardly any, and an edge costs its target, two bits and no label.
+template <int N, typename LabelT, typename K>
+__device__ __forceinline__ uint32_t edge_rest(const SigArgs& a, uint64_t base, uint32_t stride, uint64_t end,
+                                              const Policies& pol, K (&key)[N], uint32_t& count) {
+  uint32_t t[N], d[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const uint64_t e = base + (uint64_t)i * stride;
+    t[i] = ld_hint_if(a.dst + e, pol.stream, e < end);
+    d[i] = ld_hint_if(a.dup + (e >> 5), pol.stream, e < end);
+  }
+  uint32_t ok = 0, rest = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const uint64_t e = base + (uint64_t)i * stride;
+    if (e < end && !((d[i] >> (e & 31)) & 1u)) ok |= 1u << i;
+    d[i] = ld_hint_if(a.alone_bits + (t[i] >> 5), pol.keep, (ok >> i) & 1u);
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (((ok >> i) & 1u) && !((d[i] >> (t[i] & 31)) & 1u)) rest |= 1u << i;
+  count += __popc(ok & ~rest);
+  if (__any_sync(kFull, rest)) {
+    const LabelT* lab = static_cast<const LabelT*>(a.lab);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const bool r = (rest >> i) & 1u;
+      d[i] = ld_hint_if(lab + base + (uint64_t)i * stride, pol.stream, r);
+      t[i] = ld_hint_if(a.prev + t[i], pol.keep, r);
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) key[i] = KeyOps<K>::make(d[i], t[i], a.pbits);
+  }
+  return rest;
 }
 
 // Out-degree <= 64: one thread per node, its keys in registers (S = 2^c
@@ -665,7 +719,33 @@ __device__ __forceinline__ int pow2_insert(uint32_t base, uint32_t hmask, K k) {
 // atomics; a step that belongs to one node needs about 70.  
 constexpr int kNodeWarps = 8;  // per CTA
 
-template <int STEPS, typename LabelT, typename K>
+// Distinct elements of a node that only counts, with its duplicates marked: the
+// set (of SLOTS slots) is needed for targets not alone in their block only.
+template <uint32_t SLOTS, int PART, typename LabelT, typename K>
+__device__ __forceinline__ uint32_t count_one_node(const SigArgs& a, uint64_t e0, uint32_t d, uint32_t sbase, K* set,
+                                                   const Policies& pol) {
+  const uint32_t lane = threadIdx.x & 31;
+  uint32_t c = 0;
+  bool empty = false, cleared = false;
+#pragma unroll 1
+  for (uint32_t i0 = 0; i0 < d; i0 += 32 * PART) {
+    K key[PART];
+    const uint32_t rest = edge_rest<PART, LabelT, K>(a, e0 + i0 + lane, 32u, e0 + d, pol, key, c);
+    if (!__any_sync(kFull, rest)) continue;
+    if (!cleared) fill_empty<32>(set, SLOTS, lane);
+    cleared = true;
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < PART; ++t) {
+      if (!((rest >> t) & 1u)) continue;
+      if (key[t] != KeyOps<K>::kEmpty) c += pow2_insert(sbase, SLOTS - 1, key[t]) > 0 ? 1u : 0u;
+      else empty = true;
+    }
+  }
+  return __reduce_add_sync(kFull, c) + (__any_sync(kFull, empty) ? 1u : 0u);
+}
+
+template <int STEPS, int MODE, typename LabelT, typename K>
 __device__ __forceinline__ void sig_one_node(const SigArgs& a, uint64_t e0, uint32_t d, bool alone, uint32_t sbase,
                                              K* set, const Policies& pol, uint32_t& U, uint32_t& lo, uint32_t& hi) {
   const uint32_t lane = threadIdx.x & 31;
@@ -676,15 +756,22 @@ __device__ __forceinline__ void sig_one_node(const SigArgs& a, uint64_t e0, uint
   K* out = static_cast<K*>(a.sigkey) + e0;
   uint32_t u = 0, l = 0, h = 0;
   bool seen_empty = false;
-  if (alone) {  // only the number of distinct keys is needed
+  if (MODE != kWithDup && alone) {  // only the number of distinct keys is needed (with duplicates marked: count_one_node)
 #pragma unroll
     for (int t = 0; t < STEPS; ++t) {
       const K k = key[t];
-      if (lane + 32u * t >= d) continue;
-      if (k != KeyOps<K>::kEmpty) u += pow2_insert(sbase, 64u * STEPS - 1, k) > 0 ? 1u : 0u;
-      else seen_empty = true;
+      const bool valid = lane + 32u * t < d, empty = valid && k == KeyOps<K>::kEmpty;
+      bool fresh = false;
+      if (valid && !empty) fresh = pow2_insert(sbase, 64u * STEPS - 1, k) > 0;
+      const unsigned em = __ballot_sync(kFull, empty);
+      if (em) {
+        fresh |= !seen_empty && lane == (uint32_t)__ffs(em) - 1u;
+        seen_empty = true;
+      }
+      u += fresh ? 1u : 0u;
+      if (MODE == kMarking && valid && !fresh) mark_dup(a, e0 + lane + 32u * t);
     }
-    U = __reduce_add_sync(kFull, u) + (__any_sync(kFull, seen_empty) ? 1u : 0u);
+    U = __reduce_add_sync(kFull, u);
     return;
   }
 #pragma unroll
@@ -713,7 +800,7 @@ __device__ __forceinline__ void sig_one_node(const SigArgs& a, uint64_t e0, uint
   hi = __reduce_add_sync(kFull, h);
 }
 
-template <int MAXSTEPS, typename LabelT, typename K>
+template <int MAXSTEPS, int MODE, typename LabelT, typename K>
 __device__ __forceinline__ void sig_warp_block(const SigArgs& a, uint64_t first, uint64_t count, uint32_t per) {
   __shared__ __align__(16) K sets[kNodeWarps][64 * MAXSTEPS];
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -740,11 +827,13 @@ __device__ __forceinline__ void sig_warp_block(const SigArgs& a, uint64_t first,
     const uint32_t d = __shfl_sync(kFull, d_l, j);
     const bool alone = (alone_m >> j) & 1u;
     uint32_t U = 0, lo = 0, hi = 0;
-    if constexpr (MAXSTEPS == 8) {
-      if (d <= 128) sig_one_node<4, LabelT, K>(a, e0, d, alone, sbase, set, pol, U, lo, hi);
-      else sig_one_node<8, LabelT, K>(a, e0, d, alone, sbase, set, pol, U, lo, hi);
+    if (MODE == kWithDup && alone) {
+      U = count_one_node<64u * MAXSTEPS, (MAXSTEPS < 4 ? MAXSTEPS : 4), LabelT, K>(a, e0, d, sbase, set, pol);
+    } else if constexpr (MAXSTEPS == 8) {
+      if (d <= 128) sig_one_node<4, MODE, LabelT, K>(a, e0, d, alone, sbase, set, pol, U, lo, hi);
+      else sig_one_node<8, MODE, LabelT, K>(a, e0, d, alone, sbase, set, pol, U, lo, hi);
     } else {
-      sig_one_node<MAXSTEPS, LabelT, K>(a, e0, d, alone, sbase, set, pol, U, lo, hi);
+      sig_one_node<MAXSTEPS, MODE, LabelT, K>(a, e0, d, alone, sbase, set, pol, U, lo, hi);
     }
     if (lane == j) {
       U_l = U;
@@ -758,11 +847,11 @@ __device__ __forceinline__ void sig_warp_block(const SigArgs& a, uint64_t first,
   }
 }
 
-template <int MAXSTEPS, typename LabelT, typename K>
+template <int MAXSTEPS, int MODE, typename LabelT, typename K>
 __global__ void __launch_bounds__(kNodeWarps * 32, sizeof(K) == 4 ? 6 : 4) k_sig_warp(SigArgs a, uint64_t first, uint64_t count,
                                                                 uint32_t per) {
   overlap_next();
-  sig_warp_block<MAXSTEPS, LabelT, K>(a, first, count, per);
+  sig_warp_block<MAXSTEPS, MODE, LabelT, K>(a, first, count, per);
   overlap_wait();
 }
 
@@ -780,26 +869,46 @@ struct CtaNodeSmem {
 template <int NT, typename K>
 __host__ __device__ constexpr size_t cta_node_smem() { return sizeof(CtaNodeSmem<K>) + 2 * (size_t)NT * kCtaNodeItems * sizeof(K); }
 
-template <int NT, int ITEMS, typename LabelT, typename K>
+template <int NT, int ITEMS, int MODE, typename LabelT, typename K>
 __device__ __forceinline__ void sig_cta_node(const SigArgs& a, uint64_t p, uint64_t e0, uint32_t d, CtaNodeSmem<K>& sm) {
   const uint32_t tid = threadIdx.x, lane = tid & 31;
   const bool alone = a.alone && a.alone[p];
   const Policies pol;
   K key[ITEMS];
-  edge_keys<ITEMS, 0, ITEMS, LabelT, K>(a, e0 + tid, NT, e0 + d, pol, key);
   constexpr uint32_t kSlots = 2 * NT * ITEMS;
+  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sm.set());
   if (tid < 4) (&sm.cnt)[tid] = 0;
+  if (MODE == kWithDup && alone) {
+    uint32_t c = 0;
+    const uint32_t rest = edge_rest<ITEMS, LabelT, K>(a, e0 + tid, NT, e0 + d, pol, key, c);
+    if (__syncthreads_or(rest != 0)) {
+      fill_empty<NT>(sm.set(), kSlots, tid);
+      __syncthreads();
+#pragma unroll
+      for (int t = 0; t < ITEMS; ++t) {
+        if (!((rest >> t) & 1u)) continue;
+        c += key[t] == KeyOps<K>::kEmpty ? (atomicExch(&sm.empty, 1u) == 0u ? 1u : 0u)
+                                         : (pow2_insert(sbase, kSlots - 1, key[t]) > 0 ? 1u : 0u);
+      }
+    }
+    c = __reduce_add_sync(kFull, c);
+    if (lane == 0 && c) atomicAdd(&sm.cnt, c);
+    __syncthreads();
+    if (tid == 0) a.ucnt[p] = sm.cnt;
+    return;
+  }
+  edge_keys<ITEMS, 0, ITEMS, LabelT, K>(a, e0 + tid, NT, e0 + d, pol, key);
   fill_empty<NT>(sm.set(), kSlots, tid);
   __syncthreads();
-  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sm.set());
-  if (alone) {  // only the number of distinct keys is needed
+  if (MODE != kWithDup && alone) {  // only the number of distinct keys is needed
     uint32_t c = 0;
 #pragma unroll
     for (int t = 0; t < ITEMS; ++t) {
       if (tid + (uint32_t)t * NT >= d) continue;
       const K k = key[t];
-      c += k == KeyOps<K>::kEmpty ? (atomicExch(&sm.empty, 1u) == 0u ? 1u : 0u)
-                                  : (pow2_insert(sbase, kSlots - 1, k) > 0 ? 1u : 0u);
+      const bool fresh = k == KeyOps<K>::kEmpty ? atomicExch(&sm.empty, 1u) == 0u : pow2_insert(sbase, kSlots - 1, k) > 0;
+      c += fresh ? 1u : 0u;
+      if (MODE == kMarking && !fresh) mark_dup(a, e0 + tid + (uint32_t)t * NT);
     }
     c = __reduce_add_sync(kFull, c);
     if (lane == 0) atomicAdd(&sm.cnt, c);
@@ -849,7 +958,7 @@ __device__ __forceinline__ void sig_cta_node(const SigArgs& a, uint64_t p, uint6
   }
 }
 
-template <int NT, typename LabelT, typename K>
+template <int NT, int MODE, typename LabelT, typename K>
 __device__ __forceinline__ void sig_cta_block(const SigArgs& a, uint64_t first) {
   extern __shared__ __align__(16) char smem_raw[];
   CtaNodeSmem<K>& sm = *reinterpret_cast<CtaNodeSmem<K>*>(smem_raw);
@@ -857,14 +966,14 @@ __device__ __forceinline__ void sig_cta_block(const SigArgs& a, uint64_t first) 
   if (!in_mask(a, p)) return;
   const uint64_t e0 = a.off[p];
   const uint32_t d = (uint32_t)(a.off[p + 1] - e0);
-  if (d <= NT * kCtaNodeItems / 2) sig_cta_node<NT, kCtaNodeItems / 2, LabelT, K>(a, p, e0, d, sm);
-  else sig_cta_node<NT, kCtaNodeItems, LabelT, K>(a, p, e0, d, sm);
+  if (d <= NT * kCtaNodeItems / 2) sig_cta_node<NT, kCtaNodeItems / 2, MODE, LabelT, K>(a, p, e0, d, sm);
+  else sig_cta_node<NT, kCtaNodeItems, MODE, LabelT, K>(a, p, e0, d, sm);
 }
 
-template <int NT, typename LabelT, typename K>
+template <int NT, int MODE, typename LabelT, typename K>
 __global__ void __launch_bounds__(NT, sizeof(K) == 4 ? 2048 / NT : 1536 / NT) k_sig_cta(SigArgs a, uint64_t first) {
   overlap_next();
-  sig_cta_block<NT, LabelT, K>(a, first);
+  sig_cta_block<NT, MODE, LabelT, K>(a, first);
   overlap_wait();
 }
 
@@ -928,7 +1037,29 @@ __device__ __forceinline__ uint32_t hub_bucket(K k, uint32_t bits) {
   return bits ? (uint32_t)(k >> (KeyOps<K>::kBits - bits)) : 0u;
 }
 
-template <typename LabelT, typename K>
+// Keys of a hub piece's edges that go to the hub's buckets (bits of the
+// returned mask); a hub that only counts adds its edges to nodes alone in their
+// block straight to its count.
+template <int MODE, typename LabelT, typename K>
+__device__ __forceinline__ uint32_t hub_piece_keys(const SigArgs& a, const HubArgs& h, uint32_t hub, uint64_t ebase,
+                                                   uint32_t E, K (&key)[kChunkItems]) {
+  const uint32_t tid = threadIdx.x;
+  if (MODE == kWithDup && a.alone[h.first + hub]) {
+    const Policies pol;
+    uint32_t c = 0;
+    const uint32_t rest = edge_rest<kChunkItems, LabelT, K>(a, ebase + tid, kChunkThreads, ebase + E, pol, key, c);
+    c = __reduce_add_sync(kFull, c);
+    if ((tid & 31) == 0 && c) atomicAdd(&h.hub_cur[hub], (unsigned long long)c);
+    return rest;
+  }
+  chunk_keys<kChunkThreads, LabelT, K>(a, ebase, E, key);
+  uint32_t m = 0;
+#pragma unroll
+  for (int t = 0; t < kChunkItems; ++t) m |= tid + t * kChunkThreads < E ? 1u << t : 0u;
+  return m;
+}
+
+template <int MODE, typename LabelT, typename K>
 __device__ __forceinline__ void hub_chunk_block(const SigArgs& a, const HubArgs& h, char* smem_raw) {
   ChunkSmem<K>& sm = *reinterpret_cast<ChunkSmem<K>*>(smem_raw);
   K* list = reinterpret_cast<K*>(smem_raw + sizeof(ChunkSmem<K>));
@@ -950,7 +1081,7 @@ __device__ __forceinline__ void hub_chunk_block(const SigArgs& a, const HubArgs&
     for (uint32_t i = tid; i < nb; i += kChunkThreads) bcnt[i] = 0;
   __syncthreads();
   K key[kChunkItems];
-  chunk_keys<kChunkThreads, LabelT, K>(a, ebase, E, key);
+  uint32_t todo = hub_piece_keys<MODE, LabelT, K>(a, h, hub, ebase, E, key);
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sm.slot);
 #pragma unroll 1
   for (int t = 0; t < kChunkItems; ++t) {
@@ -958,8 +1089,9 @@ __device__ __forceinline__ void hub_chunk_block(const SigArgs& a, const HubArgs&
 #pragma unroll
     for (int q = 0; q + 1 < kChunkItems; ++q) key[q] = key[q + 1];
     bool fresh = false;
-    if (tid + t * kChunkThreads < E)
+    if (todo & 1u)
       fresh = kt == KeyOps<K>::kEmpty ? atomicExch(&sm.empty, 1u) == 0u : region_insert(sbase, 0u, 2 * E, kt);
+    todo >>= 1;
     const unsigned fm = __ballot_sync(kFull, fresh);
     if (fm == 0u) continue;
     uint32_t base = 0;
@@ -991,12 +1123,12 @@ __device__ __forceinline__ void hub_chunk_block(const SigArgs& a, const HubArgs&
   }
 }
 
-template <typename LabelT, typename K>
+template <int MODE, typename LabelT, typename K>
 __global__ void __launch_bounds__(kChunkThreads) k_hub_chunk(SigArgs a, HubArgs h) {
   overlap_next();
   overlap_wait();
   extern __shared__ __align__(16) char smem_raw[];
-  hub_chunk_block<LabelT, K>(a, h, smem_raw);
+  hub_chunk_block<MODE, LabelT, K>(a, h, smem_raw);
 }
 
 // Hub pieces without the chunk-level set, for hubs whose keys rarely repeat
@@ -1083,7 +1215,7 @@ struct ScatterSmem {
   uint32_t wsum[kChunkThreads / 32];
 };
 
-template <typename LabelT, typename K>
+template <int MODE, typename LabelT, typename K>
 __device__ __forceinline__ void hub_scatter_block(const SigArgs& a, const HubArgs& h, ScatterSmem<K>& sm) {
   uint32_t *bcnt = sm.bcnt, *bpos = sm.bpos, *lstart = sm.lstart, *wsum = sm.wsum;
   K* stage = sm.stage;
@@ -1101,7 +1233,8 @@ __device__ __forceinline__ void hub_scatter_block(const SigArgs& a, const HubArg
     for (uint32_t i = tid; i < nb; i += kChunkThreads) bcnt[i] = 0;
   __syncthreads();
   K key[kChunkItems];
-  chunk_keys<kChunkThreads, LabelT, K>(a, ebase, E, key);
+  const uint32_t todo = hub_piece_keys<MODE, LabelT, K>(a, h, hub, ebase, E, key);
+  if (MODE == kWithDup && !__syncthreads_or(todo != 0)) return;
   const uint32_t cap = h.hub_cap[hub];
   uint32_t* cur = h.cursor + h.hub_bbase[hub];
   K* tmp = static_cast<K*>(h.tmp) + h.hub_tbase[hub];
@@ -1111,7 +1244,7 @@ __device__ __forceinline__ void hub_scatter_block(const SigArgs& a, const HubArg
 #pragma unroll
   for (int t = 0; t < kChunkItems; ++t) {
     rank[t] = 0;
-    if (tid + t * kChunkThreads < E) {
+    if ((todo >> t) & 1u) {
       const uint32_t b = hub_bucket(key[t], bits);
       rank[t] = in_smem ? atomicAdd(&bcnt[b], 1u) : atomicAdd(&cur[b], 1u);
     }
@@ -1119,7 +1252,7 @@ __device__ __forceinline__ void hub_scatter_block(const SigArgs& a, const HubArg
   if (!in_smem) {
 #pragma unroll
     for (int t = 0; t < kChunkItems; ++t) {
-      if (tid + t * kChunkThreads >= E) continue;
+      if (!((todo >> t) & 1u)) continue;
       const uint32_t b = hub_bucket(key[t], bits);
       if (rank[t] < cap) tmp[(uint64_t)b * cap + rank[t]] = key[t];
       else hub_fail(a, h, hub, kErrHubOverflow);
@@ -1138,9 +1271,10 @@ __device__ __forceinline__ void hub_scatter_block(const SigArgs& a, const HubArg
   cta_exclusive_scan<kChunkThreads>(lstart, nb, wsum);
 #pragma unroll
   for (int t = 0; t < kChunkItems; ++t)
-    if (tid + t * kChunkThreads < E) stage[lstart[hub_bucket(key[t], bits)] + rank[t]] = key[t];
+    if ((todo >> t) & 1u) stage[lstart[hub_bucket(key[t], bits)] + rank[t]] = key[t];
+  const uint32_t staged = lstart[nb - 1] + bcnt[nb - 1];
   __syncthreads();
-  for (uint32_t i = tid; i < E; i += kChunkThreads) {
+  for (uint32_t i = tid; i < staged; i += kChunkThreads) {
     const K k = stage[i];
     const uint32_t b = hub_bucket(k, bits);
     const uint32_t q = bpos[b] + (i - lstart[b]);
@@ -1149,26 +1283,26 @@ __device__ __forceinline__ void hub_scatter_block(const SigArgs& a, const HubArg
   }
 }
 
-template <typename LabelT, typename K>
+template <int MODE, typename LabelT, typename K>
 __global__ void __launch_bounds__(kChunkThreads, sizeof(K) == 4 ? 4 : 3) k_hub_scatter(SigArgs a, HubArgs h) {
   overlap_next();
   overlap_wait();
   __shared__ ScatterSmem<K> sm;
-  hub_scatter_block<LabelT, K>(a, h, sm);
+  hub_scatter_block<MODE, LabelT, K>(a, h, sm);
 }
 
 // Both kinds of chunk in one launch, for graphs whose rounds are launches and
 // latency more than work (up to kChainEdges): one launch less per round.  Its
 // shared memory is the chunk set's, which above that size would take the L1
 // from the scatter's gathers.
-template <typename LabelT, typename K>
-__global__ void __launch_bounds__(kChunkThreads) k_hub_pieces(SigArgs a, HubArgs h) {
+template <int MODE, typename LabelT, typename K>
+__global__ void __launch_bounds__(kChunkThreads, sizeof(K) == 4 ? 4 : 3) k_hub_pieces(SigArgs a, HubArgs h) {
   overlap_next();
   overlap_wait();
   extern __shared__ __align__(16) char smem_raw[];
   static_assert(sizeof(ScatterSmem<K>) <= hub_chunk_smem<K>(), "the scatter fits the chunk set's memory");
-  if (h.mode[h.chunks[blockIdx.x].x]) hub_scatter_block<LabelT, K>(a, h, *reinterpret_cast<ScatterSmem<K>*>(smem_raw));
-  else hub_chunk_block<LabelT, K>(a, h, smem_raw);
+  if (h.mode[h.chunks[blockIdx.x].x]) hub_scatter_block<MODE, LabelT, K>(a, h, *reinterpret_cast<ScatterSmem<K>*>(smem_raw));
+  else hub_chunk_block<MODE, LabelT, K>(a, h, smem_raw);
 }
 
 constexpr int kBucketThreads = 256, kBucketItems = 8;
@@ -1360,6 +1494,52 @@ __global__ void __launch_bounds__(kBucketThreads, sizeof(K) == 4 ? 6 : 3) k_hub_
     // no barrier here: thread 0 alone reads the bucket's totals, and the next
     // bucket's first barrier comes before anything is written to them again
   }
+}
+
+// Marks the edges of hubs that repeat an earlier (label, target) of their hub:
+// a set in global memory, two 32-bit slots per edge at the hub's place in the
+// key buffer (all ones before).  Once per loaded graph; bound by the L2's
+// atomics (the word is read first, which spares them for repeats).
+template <typename LabelT>
+__global__ void __launch_bounds__(kChunkThreads) k_mark_hubs(SigArgs a, uint64_t first, const uint4* chunks,
+                                                             uint32_t* empty_seen) {
+  const uint4 c = chunks[blockIdx.x];
+  const uint64_t p = first + c.x, ebase = ((uint64_t)c.z << 32) | c.y;
+  const uint64_t off = a.off[p];
+  const uint32_t slots = (uint32_t)min((uint64_t)0xFFFFFFFEu, 2 * (a.off[p + 1] - off));
+  uint32_t* set = static_cast<uint32_t*>(a.sigkey) + 2 * off;
+  uint32_t key[kChunkItems];
+  chunk_keys<kChunkThreads, LabelT, uint32_t>(a, ebase, c.w, key);
+#pragma unroll 1
+  for (int t = 0; t < kChunkItems; ++t) {
+    const uint32_t i = threadIdx.x + t * kChunkThreads;
+    if (i >= c.w) break;
+    const uint32_t k = key[0];
+#pragma unroll
+    for (int q = 0; q + 1 < kChunkItems; ++q) key[q] = key[q + 1];
+    bool fresh = false;
+    if (k == KeyOps<uint32_t>::kEmpty) {
+      fresh = atomicExch(&empty_seen[c.x], 1u) == 0u;
+    } else {
+      uint32_t s = region_home(k, slots);
+      for (uint32_t q = 0; q < slots; ++q) {  // at most half full: ends at k or at an empty slot
+        uint32_t cur = *(volatile uint32_t*)&set[s];
+        if (cur == KeyOps<uint32_t>::kEmpty) cur = atomicCAS(&set[s], KeyOps<uint32_t>::kEmpty, k);
+        if (cur == KeyOps<uint32_t>::kEmpty) {
+          fresh = true;
+          break;
+        }
+        if (cur == k) break;
+        if (++s == slots) s = 0;
+      }
+    }
+    if (!fresh) mark_dup(a, ebase + i);
+  }
+}
+
+__global__ void k_iota(uint64_t n, uint32_t* a) {
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
+    a[i] = (uint32_t)i;
 }
 
 // --------------------------------------------------------------------------
@@ -1892,6 +2072,7 @@ struct RankArgs {
   const uint32_t* err;     // error flags, copied to stats[7]
   unsigned long long* stats;  // [2] key total, [3] max signature, [7] error flags, [8] nodes alone in their block
   unsigned long long* host;   // pinned: all 16 scalars, by the last CTA
+  uint32_t* alone_bits;       // [(n + 31) / 32] alone as a bitmap (may be null)
 };
 
 // The 16 scalars of a level into pinned host memory (a copy of its own took
@@ -2036,7 +2217,9 @@ __global__ void __launch_bounds__(kFillThreads, 4) k_pid_fill(RankArgs r) {
   unsigned int n_alone = 0, mx = 0;
   unsigned long long keys = 0;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t p0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p0 < r.n; p0 += stride * kFillItems) {
+  const uint32_t lane = threadIdx.x & 31;
+  // (the whole warp goes through the loop together)
+  for (uint64_t p0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p0 - lane < r.n; p0 += stride * kFillItems) {
     uint32_t h[kFillItems], o[kFillItems], u[kFillItems];
     uint8_t mem[kFillItems];
     uint2 hr[kFillItems];
@@ -2067,16 +2250,20 @@ __global__ void __launch_bounds__(kFillThreads, 4) k_pid_fill(RankArgs r) {
 #pragma unroll
     for (int t = 0; t < kFillItems; ++t) {
       const uint64_t p = p0 + (uint64_t)t * stride;
-      if (p >= r.n) break;
+      bool al = false;
       if (live[t]) {
         keys += u[t];
         mx = max(mx, u[t]);
         r.pid[p] = hr[t].y + (uint32_t)__popc(hr[t].x & ((1u << (o[t] & 31)) - 1u));
-        const bool al = h[t] == (uint32_t)p && !mem[t];
+        al = h[t] == (uint32_t)p && !mem[t];
         r.alone[p] = al ? 1 : 0;
         n_alone += al ? 1u : 0u;
-      } else {
+      } else if (p < r.n) {
         r.pid[p] = kDead;
+      }
+      if (r.alone_bits) {  // a warp's 32 nodes are one word
+        const uint32_t bits = __ballot_sync(kFull, al);
+        if (lane == 0 && p < r.n) r.alone_bits[p >> 5] = bits;
       }
     }
   }
@@ -2527,14 +2714,15 @@ Status scan64(Store& s, uint64_t* a, uint64_t n, uint64_t* copy) {
 
 template <typename LabelT, typename K>
 cudaError_t set_smem_attrs_label() {
-  cudaError_t e = cudaFuncSetAttribute(k_sig_cta<kChunkThreads, LabelT, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)cta_node_smem<kChunkThreads, K>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_hub_chunk<LabelT, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)hub_chunk_smem<K>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_hub_pieces<LabelT, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)hub_chunk_smem<K>());
+  cudaError_t e = cudaSuccess;
+  for (auto kernel : {k_sig_cta<kChunkThreads, kPlain, LabelT, K>, k_sig_cta<kChunkThreads, kWithDup, LabelT, K>,
+                      k_sig_cta<kChunkThreads, kMarking, LabelT, K>})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cta_node_smem<kChunkThreads, K>());
+  for (auto kernel : {k_hub_chunk<kPlain, LabelT, K>, k_hub_chunk<kWithDup, LabelT, K>, k_hub_pieces<kPlain, LabelT, K>,
+                      k_hub_pieces<kWithDup, LabelT, K>})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hub_chunk_smem<K>());
   return e;
 }
 
@@ -2802,6 +2990,7 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
   r.err = ptr<uint32_t>(s.d_err);
   r.member = ptr<uint8_t>(s.member);
   r.alone = ptr<uint8_t>(s.alone);
+  r.alone_bits = s.dup_valid ? ptr<uint32_t>(s.alone_bits) : nullptr;
   r.pid = pid;
   r.host = ptr<unsigned long long>(s.h_scalars);
   r.stats = sc;
@@ -2972,11 +3161,16 @@ Status launch_hubs(Store& s, const SigArgs& a, bool cleared) {
     cudaMemsetAsync(s.hub_err.p, 0, s.n_hub * 4, s.stream);
   }
   launch_chained(s, k_hub_sample<LabelT, K>, (unsigned)((s.n_hub + 7) / 8), 256, 0, a, h, s.n_hub);
+  const bool dup = a.dup && a.dup_hubs;
+  const unsigned pieces = (unsigned)s.n_hub_chunks;
   if (small) {
-    launch_chained(s, k_hub_pieces<LabelT, K>, (unsigned)s.n_hub_chunks, kChunkThreads, hub_chunk_smem<K>(), a, h);
+    launch_chained(s, dup ? k_hub_pieces<kWithDup, LabelT, K> : k_hub_pieces<kPlain, LabelT, K>, pieces, kChunkThreads,
+                   hub_chunk_smem<K>(), a, h);
   } else {
-    launch_chained(s, k_hub_chunk<LabelT, K>, (unsigned)s.n_hub_chunks, kChunkThreads, hub_chunk_smem<K>(), a, h);
-    launch_chained(s, k_hub_scatter<LabelT, K>, (unsigned)s.n_hub_chunks, kChunkThreads, 0, a, h);
+    launch_chained(s, dup ? k_hub_chunk<kWithDup, LabelT, K> : k_hub_chunk<kPlain, LabelT, K>, pieces, kChunkThreads,
+                   hub_chunk_smem<K>(), a, h);
+    launch_chained(s, dup ? k_hub_scatter<kWithDup, LabelT, K> : k_hub_scatter<kPlain, LabelT, K>, pieces, kChunkThreads,
+                   0, a, h);
   }
   if (s.hub_ucap == (uint32_t)kHubUcaps[1]) launch_hub_bucket<K, kHubUcaps[1]>(s, a, h);
   else if (s.hub_ucap == (uint32_t)kHubUcaps[2]) launch_hub_bucket<K, kHubUcaps[2]>(s, a, h);
@@ -3027,6 +3221,12 @@ Status grow_hubs(Store& s, SigArgs* a) {
 
 constexpr int kHubAttempts = 40;
 constexpr uint64_t kHubCalmNodes = 4u << 20;
+// Edges from which a graph's duplicates are marked: refining the 16M-edge
+// powerlaw graph again takes 1.21 against 1.30 ms, the uniform one 1.50 against
+// 1.54, 256M edges 8.51 against 9.58; below, a round is latency and the extra
+// words only cost.  Marking takes about one pass over the signatures, so a
+// graph refined once is not marked.
+constexpr uint64_t kMarkEdges = 8u << 20;
 
 // Hub passes until no bucket overflows, the host waiting for each.
 template <typename LabelT, typename K>
@@ -3086,10 +3286,14 @@ Status run_signatures(Store& s, const SigArgs& a, bool defer) {
   {
     const uint64_t n64 = s.class_start[kClassWarp] - s.class_start[kSmallClasses - 1];
     TimedScope ts(s, KBISIM_KERNEL_SIG_SMALL, (n04 ? 1 : 0) + (n5 ? 1 : 0) + (n6 ? 1 : 0) + (n64 ? 1 : 0));
-    if (n04) run(k_sig_small<0, 4, LabelT, K>, n04, kSmallThreads, 0, a, L04);
-    if (n5) run(k_sig_small<5, 5, LabelT, K>, n5, kSmallThreads, 0, a, L5);
-    if (n6) run(k_sig_small<6, 6, LabelT, K>, n6, kSmallThreads, 0, a, L6);
-    if (n64) warp_nodes(k_sig_warp<2, LabelT, K>, s.class_start[kSmallClasses - 1], n64);
+    if (n04 && !a.mark) run(k_sig_small<0, 4, LabelT, K>, n04, kSmallThreads, 0, a, L04);
+    if (n5 && !a.mark) run(k_sig_small<5, 5, LabelT, K>, n5, kSmallThreads, 0, a, L5);
+    if (n6 && !a.mark) run(k_sig_small<6, 6, LabelT, K>, n6, kSmallThreads, 0, a, L6);
+    if (n64)
+      warp_nodes(a.mark  ? k_sig_warp<2, kMarking, LabelT, K>
+                 : a.dup ? k_sig_warp<2, kWithDup, LabelT, K>
+                         : k_sig_warp<2, kPlain, LabelT, K>,
+                 s.class_start[kSmallClasses - 1], n64);
   }
   if (!(st = launch_check("k_sig_small")).ok()) return st;
   const uint64_t n256 = s.class_start[kClassWarp2] - s.class_start[kClassWarp];
@@ -3097,15 +3301,32 @@ Status run_signatures(Store& s, const SigArgs& a, bool defer) {
   const uint64_t n4k = s.class_start[kClassHub] - s.class_start[kClassBlock];
   if (n256 + n1k + n4k) {
     TimedScope ts(s, KBISIM_KERNEL_SIG_MEDIUM, (n256 ? 1 : 0) + (n1k ? 1 : 0) + (n4k ? 1 : 0));
-    if (n256) warp_nodes(k_sig_warp<8, LabelT, K>, s.class_start[kClassWarp], n256);
+    if (n256)
+      warp_nodes(a.mark  ? k_sig_warp<8, kMarking, LabelT, K>
+                 : a.dup ? k_sig_warp<8, kWithDup, LabelT, K>
+                         : k_sig_warp<8, kPlain, LabelT, K>,
+                 s.class_start[kClassWarp], n256);
     if (n1k)
-      run(k_sig_cta<kSmallChunkThreads, LabelT, K>, (unsigned)n1k, kSmallChunkThreads,
-          cta_node_smem<kSmallChunkThreads, K>(), a, s.class_start[kClassWarp2]);
+      run(a.mark  ? k_sig_cta<kSmallChunkThreads, kMarking, LabelT, K>
+          : a.dup ? k_sig_cta<kSmallChunkThreads, kWithDup, LabelT, K>
+                  : k_sig_cta<kSmallChunkThreads, kPlain, LabelT, K>,
+          (unsigned)n1k, kSmallChunkThreads, cta_node_smem<kSmallChunkThreads, K>(), a, s.class_start[kClassWarp2]);
     if (n4k)
-      run(k_sig_cta<kChunkThreads, LabelT, K>, (unsigned)n4k, kChunkThreads, cta_node_smem<kChunkThreads, K>(), a,
+      run(a.mark  ? k_sig_cta<kChunkThreads, kMarking, LabelT, K>
+          : a.dup ? k_sig_cta<kChunkThreads, kWithDup, LabelT, K>
+                  : k_sig_cta<kChunkThreads, kPlain, LabelT, K>, (unsigned)n4k, kChunkThreads, cta_node_smem<kChunkThreads, K>(), a,
           s.class_start[kClassBlock]);
   }
   if (!(st = launch_check("k_sig_warp")).ok()) return st;
+  if (s.n_hub && a.mark) {
+    if (!a.dup_hubs) return Status::Ok();
+    TimedScope ts(s, KBISIM_KERNEL_OTHER, 1);
+    const uint64_t first = s.class_start[kClassHub];
+    cudaMemsetAsync(s.hub_err.p, 0, s.n_hub * 4, s.stream);
+    k_mark_hubs<LabelT><<<(unsigned)s.n_hub_chunks, kChunkThreads, 0, s.stream>>>(a, first, ptr<uint4>(s.hub_chunks),
+                                                                                  ptr<uint32_t>(s.hub_err));
+    return launch_check("k_mark_hubs");
+  }
   if (s.n_hub) {
     if (!s.tune_now) return defer ? launch_hubs<LabelT, K>(s, a, true) : run_hubs<LabelT, K>(s, a);
     // tuning (once per handle, on a full round from level 2 on): each bucket
@@ -3261,6 +3482,8 @@ Status restore_hub_growth(Store& s, const HubGrowth& g, bool same_degree) {
 // `fresh`: a new graph (bucket growth learned on the previous one is dropped).
 Status build_chunk_lists(Store& s, bool fresh) {
   Status st;
+  s.dup_valid = false;  // another edge table
+  s.refined = false;
   // hubs: a contiguous internal id range; their offsets come in one copy
   s.n_hub = s.class_start[kClassHub + 1] - s.class_start[kClassHub];
   if (fresh || s.h_hub_xbits.size() != s.n_hub) {  // bucket growth learned on this graph is kept otherwise
@@ -3279,6 +3502,7 @@ Status build_chunk_lists(Store& s, bool fresh) {
                                     (s.n_hub + 1) * 8, cudaMemcpyDeviceToHost, s.stream), "hub offsets");
     if (st.ok()) st = cuda_check(cudaStreamSynchronize(s.stream), "sync");
     if (!st.ok()) return st;
+    s.hub_edge0 = hoff[0];
     std::vector<uint4> chunks;
     std::vector<uint32_t> cstart(s.n_hub + 1, 0);
     for (uint64_t i = 0; i < s.n_hub; ++i) {
@@ -3680,6 +3904,10 @@ Status compute_round(Store& s, uint32_t i) {
   a.err = ptr<uint32_t>(s.d_err);
   a.fmask = s.round_mask;
   a.alone = ptr<uint8_t>(s.alone);
+  a.dup = s.dup_valid && keep ? ptr<uint32_t>(s.dup) : nullptr;  // (keep: alone_bits is the level before's)
+  a.alone_bits = ptr<uint32_t>(s.alone_bits);
+  a.dup_hubs = s.dup_hubs;
+  a.mark = nullptr;
   // 32-bit signature words when (label, child id) fits in 32 bits
   const uint32_t pbits = bits_for(s.counts[i - 1] ? s.counts[i - 1] - 1 : 0);
   const bool key64 = pbits + s.label_bits > 32;
@@ -3738,6 +3966,49 @@ Status compute_round(Store& s, uint32_t i) {
   return Status::Ok();
 }
 
+Status mark_duplicates(Store& s) {
+  s.dup_valid = false;
+  if (!s.n || s.m < kMarkEdges || s.budget || s.checked || s.fault_alloc >= 0) return Status::Ok();
+  Status st = ensure_round_scratch(s);
+  if (!st.ok()) return st;
+  const uint64_t words = s.m / 32 + 1;
+  if (!ensure(s, s.dup, words * 4 + 16).ok() || !ensure(s, s.alone_bits, s.n / 32 * 4 + 16).ok()) {
+    release(s, s.dup);
+    return Status::Ok();  // no room: every round runs without the marks
+  }
+  const uint32_t pbits = bits_for(s.n - 1);
+  const bool key64 = pbits + s.label_bits > 32;
+  SigArgs a = {};
+  a.off = ptr<uint64_t>(s.offsets);
+  a.dst = ptr<uint32_t>(s.dst);
+  a.lab = s.elabel.p;
+  a.prev = ptr<uint32_t>(s.slot);     // the identity
+  a.alone = ptr<uint8_t>(s.member);   // every node only counts
+  a.sigkey = s.sigkey.p;
+  a.ucnt = ptr<uint32_t>(s.ucnt);
+  a.hash = ptr<uint64_t>(s.hash);
+  a.pbits = (int)pbits;
+  a.err = ptr<uint32_t>(s.d_err);
+  a.mark = ptr<uint32_t>(s.dup);
+  a.dup_hubs = !key64;  // (a hub's set has 32-bit slots)
+  TimedScope ts(s, KBISIM_KERNEL_OTHER, 1);
+  cudaMemsetAsync(s.dup.p, 0, words * 4, s.stream);
+  cudaMemsetAsync(s.member.p, 1, s.n, s.stream);
+  if (s.n_hub && a.dup_hubs)
+    cudaMemsetAsync(static_cast<char*>(s.sigkey.p) + s.hub_edge0 * 8, 0xFF, s.hub_edges * 8, s.stream);
+  k_iota<<<(unsigned)std::min<uint64_t>(grid_for(s.n, 256), (uint64_t)sm_count(s.device) * 16), 256, 0, s.stream>>>(
+      s.n, ptr<uint32_t>(s.slot));
+  if (!(st = launch_check("mark duplicates")).ok()) return st;
+  if (s.label8)
+    st = key64 ? run_signatures<uint8_t, uint64_t>(s, a, false) : run_signatures<uint8_t, uint32_t>(s, a, false);
+  else
+    st = key64 ? run_signatures<uint32_t, uint64_t>(s, a, false) : run_signatures<uint32_t, uint32_t>(s, a, false);
+  if (!st.ok()) return st;
+  s.dup_hubs = a.dup_hubs;
+  s.dup_valid = true;
+  return Status::Ok();
+}
+
 Status masked_signatures(Store& s, const uint32_t* prev, const uint32_t* fmask) {
   Status st = ensure_round_scratch(s);
   if (!st.ok()) return st;
@@ -3755,6 +4026,9 @@ Status masked_signatures(Store& s, const uint32_t* prev, const uint32_t* fmask) 
   a.err = ptr<uint32_t>(s.d_err);
   a.fmask = fmask;
   a.alone = nullptr;
+  a.dup = a.alone_bits = nullptr;
+  a.dup_hubs = false;
+  a.mark = nullptr;
   if (s.mt.key32) {  // labels below 2^pbits (the stores' width)
     a.pbits = (int)s.mt.pbits;
     return s.label8 ? run_signatures<uint8_t, uint32_t>(s, a, false) : run_signatures<uint32_t, uint32_t>(s, a, false);

@@ -218,3 +218,42 @@ def test_batch_finds_the_one_edge_between_graphs(degree, bad):
             ref = oracle_levels(g, k)
             assert kb.many_info(j)[1].tolist() == ref.counts.tolist()
             assert np.array_equal(kb.many_pids(j, k), ref.pids[k])
+
+
+@pytest.mark.parametrize("edge_labels", [3, 5000])
+def test_refining_again_with_duplicates_marked(edge_labels):
+    """From 8M edges on, the second refinement of an edge table marks the edges that repeat an earlier (label, target)
+    of their node and later rounds skip set inserts for targets alone in their block: levels and round statistics stay
+    those of the first, also after a batch (a new table) and with k extended."""
+    n, m = 150_000, 9_000_000
+    rng = np.random.default_rng(31)
+    deg = np.maximum(1, np.rint((1 - rng.random(n)) ** (-1 / 1.1))).astype(np.int64)
+    deg = np.minimum((deg * (m / deg.sum())).astype(np.int64) + 1, 300_000)
+    deg[:3] = 70_000
+    src = np.repeat(np.arange(n, dtype=np.uint32), deg)
+    dst = (n * rng.random(src.size) ** 3).astype(np.uint32)  # skewed: many repeated triples
+    lab = rng.integers(0, edge_labels, src.size).astype(np.uint32)
+    dst[:70_000] = rng.integers(0, 40, 70_000)  # a hub with few targets, one with a dominant target
+    dst[70_000:100_000] = 7
+    g = synth.Graph(n, np.concatenate([[0], np.cumsum(deg)]).astype(np.uint64), dst,
+                    lab.astype(np.uint8 if edge_labels < 256 else np.uint32), rng.integers(0, 4, n).astype(np.uint32))
+
+    def result(kb, res):
+        return res.counts, res.rounds_run, [kb.round_stats(r) for r in range(1, res.rounds_run + 1)], kb.all_pids(4)
+
+    def same(x, y):
+        assert x[:3] == y[:3]
+        assert np.array_equal(x[3], y[3])
+
+    with KBisim(early_stop=False) as kb:
+        first = result(kb, kb.build(g, 4))
+        assert_same(type("R", (), {"counts": first[0], "rounds_run": first[1]}), first[3], oracle_levels(g, 4, early_stop=False))
+        for _ in range(2):
+            same(result(kb, kb.refine(4)), first)
+        kb.refine(2)
+        same(result(kb, kb.extend(4)), first)
+        ins = (np.array([5, 6], np.uint32), np.array([1, 2], np.uint32), np.array([0, 1], np.uint32))
+        kb.update(4, ins=ins)
+        kb.update(4, dels=ins)
+        for _ in range(2):
+            same(result(kb, kb.refine(4)), first)
