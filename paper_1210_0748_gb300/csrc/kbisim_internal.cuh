@@ -21,7 +21,7 @@ constexpr uint32_t kNone32 = 0xFFFFFFFFu;
 constexpr uint32_t kDead = KBISIM_DELETED;
 
 // Degree classes of the signature kernels.
-constexpr int kSmallMax = 64;      // out-degree <= 32: one thread per node, keys in registers; 33..64: a warp per node
+constexpr int kSmallMax = 64;      // out-degree <= 16: one thread per node, keys in registers; 17..64: a warp per node
 constexpr int kWarpMax = 256;      // 65..256: a warp per node
 constexpr int kWarp2Max = 1024;    // 257..1024 and 1025..4096: a CTA per node
 constexpr int kBlockMax = 4096;
@@ -270,7 +270,7 @@ struct Store {
   Buf alone;                   // uint8 [n] node is alone in its block at the last computed level
   Buf hword;                   // uint64 [(n+31)/32] heads before each bitmap word
   uint64_t n_alone = 0;        // nodes alone in their block at the last computed level
-  Buf dup;                     // bit per edge: repeats an earlier (label, target) of its node (out-degree > 32)
+  Buf dup;                     // bit per edge: repeats an earlier (label, target) of its node (out-degree > 16)
   Buf alone_bits;              // alone as a bitmap, while dup is in use
   bool dup_valid = false, dup_hubs = false;  // dup describes the edge table; the hubs' edges too
   bool refined = false;        // the edge table has been refined from level 0

@@ -5,9 +5,8 @@
 //   (a) gather: for every edge e = (u, l, v) of the source-sorted edge table,
 //       the element (l, pId_{i-1}(v))  -- Algorithm 1 fills pId_old(tId) by a
 //       merge join of the edge and node tables; here it is a direct gather;
-//   (b) per source node: drop duplicate elements and sort the rest (the
-//       sorted, duplicate-free F of Algorithm 1), written at the node's CSR
-//       offset;
+//   (b) per source node: drop duplicate elements (the duplicate-free F of
+//       Algorithm 1, unsorted), written at the node's CSR offset;
 //   (c) a 64-bit hash of (pId_{i-1}(u), the element set)  -- it only routes
 //       nodes to candidate groups; it stands in for the signature store S
 //       (Section 3, "Data structures for S");
@@ -18,11 +17,11 @@
 //   (e) the caller stops when the block count is unchanged.
 // Level 0 groups nodes by label the same way (Algorithm 1, k = 0 branch).
 //
-// Degree tiers of step (a)-(c): out-degree <= 32 uses P = 2^c lanes per node
-// and a bitonic network in registers; 33..256 one warp per node; 257..4096
-// one CTA per node (both with a shared-memory hash set, then a counting sort);
-// larger "hubs" are partitioned by key bits into buckets of about 2048
-// distinct keys, each bucket deduplicated and sorted by one CTA.
+// Degree tiers of steps (a) to (c): out-degree <= 16 one thread per node with
+// its elements in registers, 17..256 one warp and 257..4096 one CTA per node,
+// both with a shared-memory hash set; larger "hubs" are partitioned by key bits
+// into buckets, each deduplicated by one CTA.  A node's distinct elements are
+// kept in any order and compared as sets.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -367,7 +366,6 @@ __device__ __forceinline__ bool in_mask(const SigArgs& a, uint64_t p) {
   return !a.fmask || ((a.fmask[p >> 5] >> (p & 31)) & 1u);
 }
 
-constexpr int kLoadBatch = 16;  // edges whose loads a thread-per-node kernel issues together
 
 struct Policies {
   uint64_t stream, keep;
@@ -395,17 +393,7 @@ __device__ __forceinline__ void edge_keys(const SigArgs& a, uint64_t base, uint3
   for (int i = 0; i < N; ++i) key[O + i] = KeyOps<K>::make(l[i], t[i], a.pbits);
 }
 
-// Keys of edges off .. off + S (those below end) in batches of B.
-template <int O, int B, int S, typename LabelT, typename K>
-__device__ __forceinline__ void edge_key_batches(const SigArgs& a, uint64_t off, uint64_t end, const Policies& pol,
-                                                 K (&key)[S]) {
-  if constexpr (O < S) {
-    edge_keys<B, O, S, LabelT, K>(a, off + O, 1u, end, pol, key);
-    edge_key_batches<O + B, B, S, LabelT, K>(a, off, end, pol, key);
-  }
-}
-
-// Variants of the kernels for out-degree 33..4096: without marks, with a.dup
+// Variants of the kernels for out-degree 17..4096: without marks, with a.dup
 // set, and the marking pass itself (each carries only its own code).
 enum { kPlain = 0, kWithDup = 1, kMarking = 2 };
 
@@ -450,42 +438,18 @@ __device__ __forceinline__ uint32_t edge_rest(const SigArgs& a, uint64_t base, u
   return rest;
 }
 
-// Out-degree <= 64: one thread per node, its keys in registers (S = 2^c
-// slots, S >= out-degree).  A key is kept unless an earlier slot holds the
-// same key, so no shuffles, sorting or shared memory are needed.
-template <int S, typename LabelT, typename K>
-__device__ __forceinline__ void sig_thread_node(const SigArgs& a, uint64_t p, const Policies& pol) {
-  if (!in_mask(a, p)) return;
-  const uint64_t off = a.off[p];
-  const uint32_t d = (uint32_t)(a.off[p + 1] - off);
-  K k[S];
-  edge_key_batches<0, (S < kLoadBatch ? S : kLoadBatch), S, LabelT, K>(a, off, off + d, pol, k);
-  K* out = static_cast<K*>(a.sigkey) + off;
-  uint64_t term = 0;
-  uint32_t U = 0;
-#pragma unroll
-  for (int i = 0; i < S; ++i) {
-    bool keep = i < (int)d;
-#pragma unroll
-    for (int j = 0; j < i; ++j) keep = keep && k[j] != k[i];
-    if (keep) {
-      out[U] = k[i];
-      term = term_add(term, elem_term(k[i], a.seed));
-      ++U;
-    }
-  }
-  a.ucnt[p] = U;
-  a.hash[p] = node_hash(term, a.prev[p], U, a.seed, a.mask);
-}
-
-// The same for the 32 nodes of a warp (consecutive internal ids, so their
-// edges are one contiguous range of at most 32 * S edges), with the edges
-// staged through the warp's shared-memory buffer: the warp loads the range
-// coalesced (lane l takes edges l, l + 32, ...) and makes the keys, each
-// thread reads its node's keys back, keeps the distinct ones as above and
-// writes them over its own keys, and the warp stores the whole range
-// coalesced (slots past a node's distinct count keep leftovers that nothing
-// reads).  Lanes past the class end take part without a node.
+// Out-degree <= 16: a thread per node for the 32 nodes of a warp (consecutive
+// internal ids, so their edges are one contiguous range of at most 32 * S
+// edges), with the edges staged through the warp's shared-memory buffer: the
+// warp loads the range coalesced (lane l takes edges l, l + 32, ...) and makes
+// the keys, each thread reads its node's keys back into registers (S = 2^c
+// slots, S >= out-degree) and keeps a key unless an earlier slot holds it, so
+// no sorting or set is needed; it writes the distinct ones over its own keys,
+// and the warp stores the whole range coalesced (slots past a node's distinct
+// count keep leftovers that nothing reads).  A node alone in its block only
+// counts.  Lanes past the class end take part without a node.
+// Bound by the L1's data pipe (81% at out-degree <= 8: about 0.75 of 1.4
+// wavefronts per edge are the identifier gather).
 template <int S, typename LabelT, typename K>
 __device__ __forceinline__ void sig_warp_staged(const SigArgs& a, uint64_t p_first, uint32_t nvalid, K* wsm,
                                                 const Policies& pol) {
@@ -505,6 +469,7 @@ __device__ __forceinline__ void sig_warp_staged(const SigArgs& a, uint64_t p_fir
   }
   __syncwarp();
   uint32_t r0 = 0, d = 0;
+  const bool full = valid && !(a.alone && a.alone[p]);  // its keys and hash are needed
   if (valid) {
     const uint64_t o = a.off[p];
     r0 = (uint32_t)(o - base);
@@ -522,27 +487,22 @@ __device__ __forceinline__ void sig_warp_staged(const SigArgs& a, uint64_t p_fir
 #pragma unroll
     for (int j = 0; j < i; ++j) keep = keep && k[j] != k[i];
     if (keep) {
-      wsm[r0 + U] = k[i];
-      term = term_add(term, elem_term(k[i], a.seed));
+      if (full) {
+        wsm[r0 + U] = k[i];
+        term = term_add(term, elem_term(k[i], a.seed));
+      }
       ++U;
     }
   }
-  __syncwarp();
-  K* out = static_cast<K*>(a.sigkey) + base;
+  if (__any_sync(kFull, full)) {
+    __syncwarp();
+    K* out = static_cast<K*>(a.sigkey) + base;
 #pragma unroll
-  for (int t = 0; t < S; ++t)
-    if (lane + 32u * t < T) out[lane + 32u * t] = wsm[lane + 32u * t];
-  if (valid) {
-    a.ucnt[p] = U;
-    a.hash[p] = node_hash(term, a.prev[p], U, a.seed, a.mask);
+    for (int t = 0; t < S; ++t)
+      if (lane + 32u * t < T) out[lane + 32u * t] = wsm[lane + 32u * t];
   }
-}
-
-// Largest S staged through shared memory (out-degree 9..16); the 17..32 class
-// keeps one node per thread, whose registers a staged copy would double.
-template <typename K>
-__host__ __device__ constexpr int staged_max_s() {
-  return 16;
+  if (valid) a.ucnt[p] = U;
+  if (full) a.hash[p] = node_hash(term, a.prev[p], U, a.seed, a.mask);
 }
 
 // Resident CTAs per multiprocessor the small-class kernels are compiled for:
@@ -550,7 +510,7 @@ __host__ __device__ constexpr int staged_max_s() {
 // keys sit in registers.
 template <int LAST, typename K>
 __host__ __device__ constexpr int small_min_blocks() {
-  return LAST <= 4 ? (sizeof(K) == 4 ? 8 : 6) : (LAST == 5 ? 4 : (sizeof(K) == 4 ? 4 : 2));
+  return LAST <= 4 ? (sizeof(K) == 4 ? 8 : 6) : 4;
 }
 
 struct SmallLaunch {
@@ -561,16 +521,13 @@ struct SmallLaunch {
 
 constexpr int kSmallThreads = 256;
 
-// Class 0 (no out-edges): signature (pId_{i-1}(u), {}); classes 1..7
-// (out-degree 1..64): one node per thread.  Classes FIRST..LAST per launch,
-// so the 64-slot class (most registers) does not limit the occupancy of the
-// others.
+// Class 0 (no out-edges): signature (pId_{i-1}(u), {}); classes 1..5
+// (out-degree 1..16): one node per thread.  Classes FIRST..LAST per launch, so
+// that each kernel carries only its own unrolled code.
 template <int FIRST, int LAST, typename LabelT, typename K>
 __device__ __forceinline__ void sig_small_block(const SigArgs& a, const SmallLaunch& L) {
-  // per-warp staging buffer for the largest class of this launch that is staged
   constexpr int kSLast = LAST == 0 ? 1 : (1 << (LAST - 1));
-  constexpr int kSBuf = kSLast <= staged_max_s<K>() ? kSLast : 1;
-  __shared__ K stage[kSmallThreads / 32][32 * kSBuf];
+  __shared__ K stage[kSmallThreads / 32][32 * kSLast];  // per warp, for the largest class of this launch
   int c = FIRST;
   while (c < LAST && blockIdx.x >= L.bstart[c + 1]) ++c;
   const uint32_t lane = threadIdx.x & 31;
@@ -582,12 +539,9 @@ __device__ __forceinline__ void sig_small_block(const SigArgs& a, const SmallLau
   const uint64_t p = L.start[c] + idx;
   const Policies pol;
   K* wsm = stage[threadIdx.x >> 5];
-#define KB_SMALL_CLASS(C, S)                                                                  \
-  case C:                                                                                     \
-    if constexpr (LAST >= C) {                                                                \
-      if constexpr (S <= kSBuf) sig_warp_staged<S, LabelT, K>(a, L.start[c] + widx, nvalid, wsm, pol); \
-      else if (idx < L.count[c]) sig_thread_node<S, LabelT, K>(a, p, pol);                    \
-    }                                                                                         \
+#define KB_SMALL_CLASS(C, S)                                                                                  \
+  case C:                                                                                                     \
+    if constexpr (LAST >= C) sig_warp_staged<S, LabelT, K>(a, L.start[c] + widx, nvalid, wsm, pol);            \
     break;
   switch (c) {
     case 0:
@@ -601,11 +555,6 @@ __device__ __forceinline__ void sig_small_block(const SigArgs& a, const SmallLau
     KB_SMALL_CLASS(3, 4)
     KB_SMALL_CLASS(4, 8)
     KB_SMALL_CLASS(5, 16)
-    KB_SMALL_CLASS(6, 32)
-    default:
-      if constexpr (LAST >= 7)
-        if (idx < L.count[c]) sig_thread_node<64, LabelT, K>(a, p, pol);
-      break;
   }
 #undef KB_SMALL_CLASS
 }
@@ -705,7 +654,7 @@ __device__ __forceinline__ int pow2_insert(uint32_t base, uint32_t hmask, K k) {
   return -1;
 }
 
-// ---- out-degree 33..256: a warp per node ----------------------------------
+// ---- out-degree 17..256: a warp per node ----------------------------------
 // A warp takes `per` consecutive nodes (at most 32; lane j holds the bounds and
 // results of node j) and signs them one after the other: the node's edges come
 // coalesced, STEPS per lane, their gathers all in flight; every key is inserted
@@ -713,10 +662,13 @@ __device__ __forceinline__ int pow2_insert(uint32_t base, uint32_t hmask, K k) {
 // insert was the first writes the key out behind those found before.  Count and
 // term sums stay in registers, and the hashes of the warp's nodes are made
 // together at the end, a lane per node.
-// Bound by instruction issue.  Chunks of whole nodes in a CTA-wide set, where a
-// step of 32 edges could meet two nodes, spent most of their 239 warp
-// instructions a step on finding the node, on two-node sums and on shared
-// atomics; a step that belongs to one node needs about 70.  
+// Bound by instruction issue (62% at out-degree 33..64) and the L1 (60%).
+// Chunks of whole nodes in a CTA-wide set, where a step of 32 edges could meet
+// two nodes, spent most of their 239 warp instructions a step on finding the
+// node, on two-node sums and on shared atomics; a step that belongs to one node
+// takes 95 to 145.  Out-degree 17..32 ran one thread per node with 32 keys in
+// registers, whose uncoalesced loads kept the L1 at 77%: 155 -> 145 us a round
+// for 18M edges, and 635 -> 567 us for a refinement of 1M edges.  
 constexpr int kNodeWarps = 8;  // per CTA
 
 // Distinct elements of a node that only counts, with its duplicates marked: the
@@ -3253,9 +3205,8 @@ Status run_hubs(Store& s, const SigArgs& a) {
 template <typename LabelT, typename K>
 Status run_signatures(Store& s, const SigArgs& a, bool defer) {
   Status st;
-  // thread-per-node classes: 0..4 (out-degree <= 8) in one launch, 5 and 6
-  // (9..16, 17..32) in one launch each, so that each kernel carries only its
-  // own unrolled code; class 7 (33..64) runs as 128-thread chunks
+  // thread-per-node classes: 0..4 (out-degree <= 8) in one launch, 5 (9..16)
+  // in another; then a warp per node up to 256 and a CTA per node up to 4096
   auto small_launch = [&](int first, int last) {
     SmallLaunch L;
     uint32_t b = 0;
@@ -3268,8 +3219,8 @@ Status run_signatures(Store& s, const SigArgs& a, bool defer) {
     L.bstart[kSmallClasses] = b;
     return L;
   };
-  const SmallLaunch L04 = small_launch(0, 4), L5 = small_launch(5, 5), L6 = small_launch(6, 6);
-  const uint32_t n04 = L04.bstart[5], n5 = L5.bstart[6] - L5.bstart[5], n6 = L6.bstart[7] - L6.bstart[6];
+  const SmallLaunch L04 = small_launch(0, 4), L5 = small_launch(5, 5);
+  const uint32_t n04 = L04.bstart[5], n5 = L5.bstart[6] - L5.bstart[5];
   // the first kernel starts when all earlier work has ended, clear_round's
   // launch (which starts then and writes nothing these kernels read) excepted
   bool overlapped = defer;
@@ -3284,11 +3235,16 @@ Status run_signatures(Store& s, const SigArgs& a, bool defer) {
     run(kernel, grid_for(count, kNodeWarps * per), kNodeWarps * 32, 0, a, first, count, per);
   };
   {
+    const uint64_t n32 = s.class_start[kSmallClasses - 1] - s.class_start[kSmallClasses - 2];
     const uint64_t n64 = s.class_start[kClassWarp] - s.class_start[kSmallClasses - 1];
-    TimedScope ts(s, KBISIM_KERNEL_SIG_SMALL, (n04 ? 1 : 0) + (n5 ? 1 : 0) + (n6 ? 1 : 0) + (n64 ? 1 : 0));
+    TimedScope ts(s, KBISIM_KERNEL_SIG_SMALL, (n04 ? 1 : 0) + (n5 ? 1 : 0) + (n32 ? 1 : 0) + (n64 ? 1 : 0));
     if (n04 && !a.mark) run(k_sig_small<0, 4, LabelT, K>, n04, kSmallThreads, 0, a, L04);
     if (n5 && !a.mark) run(k_sig_small<5, 5, LabelT, K>, n5, kSmallThreads, 0, a, L5);
-    if (n6 && !a.mark) run(k_sig_small<6, 6, LabelT, K>, n6, kSmallThreads, 0, a, L6);
+    if (n32)
+      warp_nodes(a.mark  ? k_sig_warp<1, kMarking, LabelT, K>
+                 : a.dup ? k_sig_warp<1, kWithDup, LabelT, K>
+                         : k_sig_warp<1, kPlain, LabelT, K>,
+                 s.class_start[kSmallClasses - 2], n32);
     if (n64)
       warp_nodes(a.mark  ? k_sig_warp<2, kMarking, LabelT, K>
                  : a.dup ? k_sig_warp<2, kWithDup, LabelT, K>
