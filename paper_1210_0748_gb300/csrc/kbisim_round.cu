@@ -1823,7 +1823,7 @@ __device__ __forceinline__ void mark_unresolved(const VerifyArgs& v, uint32_t* r
 // ids and table slots; representatives; their fields; the short key lists).
 constexpr int kVerNodeThreads = 256, kVerItems = 2, kVerTile = kVerNodeThreads * kVerItems;
 
-__global__ void __launch_bounds__(kVerNodeThreads, 5) k_group_verify(GroupArgs g, VerifyArgs v, const uint32_t* list,
+__global__ void __launch_bounds__(kVerNodeThreads, 6) k_group_verify(GroupArgs g, VerifyArgs v, const uint32_t* list,
                                                                    uint64_t count) {
   overlap_next();
   overlap_wait();
