@@ -560,8 +560,8 @@ def main():
     # measured DRAM bytes of the class per round (ncu), per launch like the algorithmic bytes
     traffic_round = recorded_traffic(dom, units[dom]) if args.workload == "single" else None
     traffic = traffic_round / d["launches_per_call"] if traffic_round is not None else None
-    names = {"sig_small": "k_sig_small (out-degree <= 64, one thread per node)",
-             "sig_medium": "k_sig_chunk (out-degree 65..4096, CTA chunks)",
+    names = {"sig_small": "k_sig_small (out-degree <= 16, one thread per node) and k_sig_warp (17..64, a warp per node)",
+             "sig_medium": "k_sig_warp (out-degree 65..256, a warp per node) and k_sig_cta (257..4096, a CTA per node)",
              "sig_hub": "k_hub_sample, k_hub_chunk or k_hub_scatter per hub, k_hub_bucket, k_hub_finish (out-degree > 4096)",
              "group": "k_group_insert", "verify": "k_group_verify", "renumber": "renumbering kernels"}
     roofline = {"bound": "hbm", "kernel": names.get(dom, dom), "achieved": d["achieved"], "peak": peak,

@@ -220,7 +220,7 @@ def test_batch_finds_the_one_edge_between_graphs(degree, bad):
             assert np.array_equal(kb.many_pids(j, k), ref.pids[k])
 
 
-@pytest.mark.parametrize("edge_labels", [3, 5000])
+@pytest.mark.parametrize("edge_labels", [3, 5000, 1 << 20])
 def test_refining_again_with_duplicates_marked(edge_labels):
     """From 8M edges on, the second refinement of an edge table marks the edges that repeat an earlier (label, target)
     of their node and later rounds skip set inserts for targets alone in their block: levels and round statistics stay
