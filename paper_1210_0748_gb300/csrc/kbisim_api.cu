@@ -657,6 +657,16 @@ Status refine_levels(Store& s, uint32_t k) {
   return Status::Ok();
 }
 
+// Under a budget set after the marks were made, the rounds need the bytes that
+// the marks hold: nothing can release them while a call refines.
+void drop_marks_under_budget(Store& s) {
+  if (!s.budget || !(s.dup.p || s.alone_bits.p)) return;
+  cudaStreamSynchronize(s.stream);
+  release(s, s.dup);
+  release(s, s.alone_bits);
+  s.dup_valid = false;
+}
+
 // Levels 0..k of the loaded graph.  The new levels are computed into spare
 // buffers; the current result (level buffers, alone flags, counts) is set
 // aside and put back if the call fails, so a failed refinement leaves the
@@ -664,6 +674,7 @@ Status refine_levels(Store& s, uint32_t k) {
 Status refine(Store& s, uint32_t k, kbisim_result* out) {
   if (!s.has_graph) return Status::Err(KBISIM_ERR_STATE, "no graph loaded");
   if (k > KBISIM_MAX_K) return Status::Err(KBISIM_ERR_INVALID_ARG, "k too large");
+  drop_marks_under_budget(s);
   InUse use(s, kCacheSpare);
   LevelSnapshot snap = take_snapshot(s);
   std::swap(s.level, s.spare_level);
@@ -698,6 +709,7 @@ Status refine(Store& s, uint32_t k, kbisim_result* out) {
 Status extend(Store& s, uint32_t k_new, kbisim_result* out) {
   if (!s.has_levels) return Status::Err(KBISIM_ERR_STATE, "no computed levels");
   if (k_new > KBISIM_MAX_K) return Status::Err(KBISIM_ERR_INVALID_ARG, "k too large");
+  drop_marks_under_budget(s);
   InUse use(s, kCacheSpare);
   Status st;
   const bool need = k_new > s.computed && !(s.early_stop && s.stable);

@@ -257,3 +257,30 @@ def test_refining_again_with_duplicates_marked(edge_labels):
         kb.update(4, dels=ins)
         for _ in range(2):
             same(result(kb, kb.refine(4)), first)
+
+
+def test_marks_are_given_back_under_a_budget():
+    """A budget set after the duplicate marks were made: later refinements run without them and hold what they hold on
+    a handle that had the budget all along."""
+    n, deg = 210_000, 41
+    rng = np.random.default_rng(37)
+    g = synth.Graph(n, (np.arange(n + 1) * deg).astype(np.uint64), (n * rng.random(n * deg) ** 2).astype(np.uint32),
+                    rng.integers(0, 3, n * deg).astype(np.uint8), rng.integers(0, 4, n).astype(np.uint32))
+
+    def run(marks):
+        with KBisim(early_stop=False) as kb:
+            if not marks:
+                kb.set_hbm_budget(1 << 40)
+            kb.build(g, 2)
+            plain = kb.device_bytes
+            kb.refine(2)
+            grown = kb.device_bytes - plain
+            kb.set_hbm_budget(1 << 40)
+            kb.refine(3)
+            res = kb.extend(5)
+            return grown, kb.device_bytes, res.counts, kb.all_pids(5)
+
+    marked, unmarked = run(True), run(False)
+    assert marked[0] >= unmarked[0] + n * deg // 8  # the marks were made
+    assert marked[1:3] == unmarked[1:3]
+    assert np.array_equal(marked[3], unmarked[3])
