@@ -2157,6 +2157,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(uint64_t* bsum, uin
 // the compiler keeps that order).  The grid is one resident wave and a CTA adds
 // its counts with one atomic per statistic: with one per warp the same-address
 // atomics took most of the time at 1M nodes (39 us a call).
+// When a hub's buckets overflowed, the groups come from incomplete signatures
+// and the round is grouped again: nothing is written then but the scalars,
+// since alone and alone_bits still hold the level before, which that grouping
+// and the repeated hubs read (the flags are final: every earlier kernel ended).
 constexpr int kFillThreads = 256, kFillItems = 4;
 
 __global__ void __launch_bounds__(kFillThreads, 4) k_pid_fill(RankArgs r) {
@@ -2173,8 +2177,9 @@ __global__ void __launch_bounds__(kFillThreads, 4) k_pid_fill(RankArgs r) {
   unsigned long long keys = 0;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const uint32_t lane = threadIdx.x & 31;
+  const uint64_t n_fill = *r.err & (kErrHubOverflow | kErrHubSet) ? 0 : r.n;
   // (the whole warp goes through the loop together)
-  for (uint64_t p0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p0 - lane < r.n; p0 += stride * kFillItems) {
+  for (uint64_t p0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p0 - lane < n_fill; p0 += stride * kFillItems) {
     uint32_t h[kFillItems], o[kFillItems], u[kFillItems];
     uint8_t mem[kFillItems];
     uint2 hr[kFillItems];
