@@ -773,6 +773,7 @@ __device__ __forceinline__ void sig_warp_block(const SigArgs& a, uint64_t first,
   K* set = sets[w];
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(set);
   while (todo) {
+    __syncwarp();  // the set is cleared for this node after every insert of the one before (votes order no memory)
     const uint32_t j = (uint32_t)__ffs(todo) - 1u;
     todo &= todo - 1;
     const uint64_t e0 = base + __shfl_sync(kFull, r_l, j);

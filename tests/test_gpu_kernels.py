@@ -284,3 +284,37 @@ def test_marks_are_given_back_under_a_budget():
     assert marked[0] >= unmarked[0] + n * deg // 8  # the marks were made
     assert marked[1:3] == unmarked[1:3]
     assert np.array_equal(marked[3], unmarked[3])
+
+
+@pytest.mark.parametrize("wide", [False, True])
+def test_one_set_for_the_nodes_of_a_warp(wide):
+    """A warp signs several consecutive nodes in the same shared-memory set, which is cleared in between: neighbours
+    share most of their elements, in pairs of equal sets and alone in their block, over targets of which half are
+    alone in theirs.  50,000 nodes of each class that a warp takes; 8.7M edges, so refining again marks duplicates."""
+    rng = np.random.default_rng(41)
+    nt, per = 1 << 11, 50_000
+    adj = []
+    for d in (24, 48, 102):
+        base = np.arange(per)[:, None] // 6 % (nt - 256)  # neighbours draw from nearly the same window
+        el = np.sort((base + rng.integers(0, 2 * d, (per, d))), axis=1)
+        el[1::4] = el[0::4, ::-1]  # pairs of equal sets, in another order
+        adj.append(el)
+    dst = np.concatenate([a.reshape(-1) for a in adj]).astype(np.uint32)
+    deg = np.concatenate([np.zeros(nt, np.int64)] + [np.full(per, a.shape[1]) for a in adj])
+    lab = (dst % 3).astype(np.uint32)
+    if wide:
+        lab[0] = 0xFFFFFFFF
+    nlab = np.concatenate([np.where(np.arange(nt) % 2, np.arange(nt), np.arange(nt) // 4 * 4),
+                           10_000 + np.arange(3 * per) // 4])
+    g = synth.Graph(nt + 3 * per, np.concatenate([[0], np.cumsum(deg)]).astype(np.uint64), dst,
+                    lab if wide else lab.astype(np.uint8), nlab.astype(np.uint32))
+    assert g.num_edges >= 8 << 20
+    ref = oracle_levels(g, 3, early_stop=False)
+    edge = g.src().astype(np.int64) * 4 + np.minimum(lab, 3)
+    sets = [np.bincount(np.unique(edge << 32 | p[dst]) >> 34) for p in ref.pids[:3]]
+    with KBisim(early_stop=False) as kb:
+        for run in (lambda: kb.build(g, 3), lambda: kb.refine(3), lambda: kb.refine(3)):
+            assert_same(run(), kb.all_pids(3), ref)
+            for r in (1, 2, 3):
+                got = [kb.round_stats(r)[f] for f in ("unique_keys", "max_signature")]
+                assert got == [int(sets[r - 1].sum()), int(sets[r - 1].max())]
