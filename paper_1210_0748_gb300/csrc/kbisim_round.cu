@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "kbisim_internal.cuh"
+#include "per_device.h"
 
 namespace kb {
 
@@ -123,24 +124,20 @@ inline unsigned grid_for(uint64_t work, unsigned per_block) {
 Status launch_check(const char* what) { return cuda_check(cudaGetLastError(), what); }
 
 int sm_count(int device) {
-  static int cached[64] = {0};
-  if (device < 0 || device >= 64) return 148;
-  if (!cached[device]) {
+  static PerDevice known;
+  return known.get(device, [&] {
     int v = 0;
     cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device);
-    cached[device] = v > 0 ? v : 148;
-  }
-  return cached[device];
+    return v > 0 ? v : 148;
+  });
 }
 
 // resident_blocks of one kernel, asked of the runtime once per device (the
 // answer depends on the compiled kernel and the device only).
 template <typename F>
-unsigned resident_grid(F kernel, int threads, size_t dyn_smem, int device, int* cached) {
-  const int sms = sm_count(device);
-  if (device < 0 || device >= 64) return resident_blocks(kernel, threads, dyn_smem, sms);
-  if (!cached[device]) cached[device] = (int)resident_blocks(kernel, threads, dyn_smem, 1);
-  return (unsigned)cached[device] * (unsigned)sms;
+unsigned resident_grid(F kernel, int threads, size_t dyn_smem, int device, PerDevice& known) {
+  const int per_sm = known.get(device, [&] { return (int)resident_blocks(kernel, threads, dyn_smem, 1); });
+  return (unsigned)per_sm * (unsigned)sm_count(device);
 }
 
 // Launch overlap within a round (programmatic dependent launch).  Every
@@ -2709,11 +2706,13 @@ Status set_smem_attrs_for() {
 }
 
 Status set_smem_attrs(int device) {
-  static bool done[64] = {false};
-  if (device >= 0 && device < 64 && done[device]) return Status::Ok();
-  Status st = set_smem_attrs_for<uint32_t>();
-  if (st.ok()) st = set_smem_attrs_for<uint64_t>();
-  if (st.ok() && device >= 0 && device < 64) done[device] = true;
+  static PerDevice done;
+  Status st;
+  done.get(device, [&] {
+    st = set_smem_attrs_for<uint32_t>();
+    if (st.ok()) st = set_smem_attrs_for<uint64_t>();
+    return st.ok() ? 1 : 0;
+  });
   return st;
 }
 
@@ -2756,16 +2755,16 @@ Status check_below(Store& s, const uint32_t* a, uint64_t n, uint64_t bound, cons
 uint64_t table_capacity(uint64_t n) { return table_slots(n); }
 
 void launch_insert(Store& s, const GroupArgs& g, const uint32_t* list, uint64_t count) {
-  static int cached[64];
-  const unsigned res = resident_grid(k_group_insert, kInsThreads, 0, s.device, cached);
+  static PerDevice known;
+  const unsigned res = resident_grid(k_group_insert, kInsThreads, 0, s.device, known);
   launch_chained(s, k_group_insert, (unsigned)std::min<uint64_t>((count + kInsChunk - 1) / kInsChunk, res),
                     kInsThreads, 0, g, list, count);
 }
 
 template <typename K>
 void launch_verify_long(Store& s, const GroupArgs& g, const VerifyArgs& v, uint64_t count) {
-  static int cached[64];
-  const unsigned res = resident_grid(k_verify_long<K>, kVerThreads, verify_ws_bytes<K>(), s.device, cached);
+  static PerDevice known;
+  const unsigned res = resident_grid(k_verify_long<K>, kVerThreads, verify_ws_bytes<K>(), s.device, known);
   launch_chained(s, k_verify_long<K>, (unsigned)std::min<uint64_t>((count + 31) / 32, res), kVerThreads,
                     verify_ws_bytes<K>(), g, v);
 }
@@ -2781,8 +2780,8 @@ Status launch_pairs(Store& s, const GroupArgs& g, const VerifyArgs& v, uint64_t 
 // hash: the short signatures, then (with_pairs) the others.
 Status launch_verify(Store& s, const GroupArgs& g, const VerifyArgs& v, const uint32_t* list, uint64_t count,
                      bool with_pairs) {
-  static int cached[64];
-  const unsigned res = resident_grid(k_group_verify, kVerNodeThreads, 0, s.device, cached);
+  static PerDevice known;
+  const unsigned res = resident_grid(k_group_verify, kVerNodeThreads, 0, s.device, known);
   launch_chained(s, k_group_verify, (unsigned)std::min<uint64_t>(grid_for(count, kVerTile), res), kVerNodeThreads,
                     0, g, v, list, count);
   Status st = launch_check("k_group_verify");
@@ -2957,14 +2956,14 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
   r.host = ptr<unsigned long long>(s.h_scalars);
   r.stats = sc;
   auto renumber = [&]() -> Status {
-    static int cached[64];
+    static PerDevice known;
     TimedScope ts(s, KBISIM_KERNEL_RENUMBER, n ? 2 : 0);
     if (!n) return Status::Ok();
     launch_chained(s, k_head_ranks, (unsigned)((words + kRankTile - 1) / kRankTile), kRankThreads, 0,
                       ptr<uint32_t>(s.hbits), words, ptr<uint2>(s.hword), ptr<uint32_t>(s.bsum), sc + 9, sc + 15);
     launch_chained(s, k_pid_fill,
                       (unsigned)std::min<uint64_t>(grid_for(n, kFillThreads * kFillItems),
-                                                   resident_grid(k_pid_fill, kFillThreads, 0, s.device, cached)),
+                                                   resident_grid(k_pid_fill, kFillThreads, 0, s.device, known)),
                       kFillThreads, 0, r);
     return launch_check("renumber");
   };
@@ -2975,15 +2974,15 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
       TimedScope ts(s, KBISIM_KERNEL_GROUP, bits ? 4 : 1);
       if (bits) {
         uint32_t* cand = ptr<uint32_t>(s.ulist[1]);
-        static int cf[64], cs[64];
+        static PerDevice known_filter, known_select;
         g.seen = ptr<uint2>(s.long_pairs);
         g.seen_mask = bits - 1;
         const uint64_t tiles = grid_for(na, kFilTile);
         launch_chained(s, k_group_filter,
-                       (unsigned)std::min<uint64_t>(tiles, resident_grid(k_group_filter, kFilThreads, 0, s.device, cf)),
+                       (unsigned)std::min<uint64_t>(tiles, resident_grid(k_group_filter, kFilThreads, 0, s.device, known_filter)),
                        kFilThreads, 0, g, na);
         launch_chained(s, k_group_select,
-                       (unsigned)std::min<uint64_t>(tiles, resident_grid(k_group_select, kFilThreads, 0, s.device, cs)),
+                       (unsigned)std::min<uint64_t>(tiles, resident_grid(k_group_select, kFilThreads, 0, s.device, known_select)),
                        kFilThreads, 0, g, v, na, cand, sc + 11);
         list = cand;
         g.alone = nullptr;  // none of the listed nodes is
@@ -3084,9 +3083,9 @@ Status hub_layout(Store& s) {
 // The bucket pass with buckets of at most U key words: one resident wave of CTAs.
 template <typename K, int U>
 void launch_hub_bucket(Store& s, const SigArgs& a, const HubArgs& h) {
-  static int cached[64];
+  static PerDevice known;
   const unsigned g = (unsigned)std::min<uint64_t>(
-      s.n_hub_buckets, resident_grid(k_hub_bucket<K, U>, kBucketThreads, sizeof(BucketSmem<K, U>), s.device, cached));
+      s.n_hub_buckets, resident_grid(k_hub_bucket<K, U>, kBucketThreads, sizeof(BucketSmem<K, U>), s.device, known));
   launch_chained(s, k_hub_bucket<K, U>, g, kBucketThreads, sizeof(BucketSmem<K, U>), a, h, s.n_hub_buckets);
 }
 
