@@ -125,19 +125,22 @@ Status launch_check(const char* what) { return cuda_check(cudaGetLastError(), wh
 
 int sm_count(int device) {
   static PerDevice known;
-  return known.get(device, [&] {
-    int v = 0;
-    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device);
-    return v > 0 ? v : 148;
+  const int v = known.get(device, [&] {
+    int sms = 0;
+    return cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) == cudaSuccess ? sms : 0;
   });
+  return v > 0 ? v : 148;
 }
 
 // resident_blocks of one kernel, asked of the runtime once per device (the
 // answer depends on the compiled kernel and the device only).
 template <typename F>
 unsigned resident_grid(F kernel, int threads, size_t dyn_smem, int device, PerDevice& known) {
-  const int per_sm = known.get(device, [&] { return (int)resident_blocks(kernel, threads, dyn_smem, 1); });
-  return (unsigned)per_sm * (unsigned)sm_count(device);
+  const int per_sm = known.get(device, [&] {
+    int v = 0;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kernel, threads, dyn_smem) == cudaSuccess ? v : 0;
+  });
+  return (unsigned)std::max(per_sm, 1) * (unsigned)sm_count(device);
 }
 
 // Launch overlap within a round (programmatic dependent launch).  Every

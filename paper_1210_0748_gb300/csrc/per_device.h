@@ -10,7 +10,8 @@ struct PerDevice {
   static constexpr int kDevices = 64;
   std::atomic<int> known[kDevices] = {};  // 0 = not asked yet
 
-  // The answer for `device` (an int > 0), from query() the first time.
+  // The answer for `device`, from query() the first time.  A query that fails
+  // returns 0, which is handed on but not kept: the next call asks again.
   // Threads that ask at the same time each query and store the same answer.
   template <typename Query>
   int get(int device, Query query) {
@@ -18,7 +19,7 @@ struct PerDevice {
     int v = known[device].load(std::memory_order_acquire);
     if (!v) {
       v = query();
-      known[device].store(v, std::memory_order_release);
+      if (v > 0) known[device].store(v, std::memory_order_release);
     }
     return v;
   }

@@ -40,3 +40,19 @@ int main() {
     if "unexpected memory mapping" in checked.stderr:
         pytest.skip("the sanitizer cannot map its memory here")
     assert checked.returncode == 0 and "data race" not in checked.stderr, checked.stderr[-2000:]
+
+
+def test_a_failed_query_is_asked_again(tmp_path):
+    """A query fails by returning 0; neither that nor a negative answer is kept."""
+    body = """
+int main() {
+  static kb::PerDevice known;
+  int asked = 0;
+  const int answers[] = {0, -1, 5, 7};
+  auto query = [&] { return answers[asked++]; };
+  const bool ok = known.get(3, query) == 0 && known.get(3, query) == -1 && known.get(3, query) == 5 &&
+                  known.get(3, query) == 5 && asked == 3 && known.get(2, query) == 7;
+  return ok ? 0 : 1;
+}
+"""
+    assert _run(tmp_path, body).returncode == 0
