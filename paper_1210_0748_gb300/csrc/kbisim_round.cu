@@ -152,12 +152,19 @@ unsigned resident_grid(F kernel, int threads, size_t dyn_smem, int device, PerDe
 // At 1M edges a signature kernel has too few blocks to fill the device and its
 // 5 to 10 us are latency; at 256M edges only the tails overlap.
 //
-// The kernels that wait first (launch_chained) overlap only up to kChainEdges:
-// it hides launch latency (1M edges: 0.67 against 0.80 ms a refinement of five
-// rounds, 16M: 1.46 against 1.59), but blocks that already hold their place,
-// and their shared memory, slow the kernel before (200M edges: 20.2 against
-// 16.9 ms, 64M: 4.98 against 4.65; equal at 32M).
-constexpr uint64_t kChainEdges = 32ull << 20;
+// The kernels that wait first (launch_chained) overlap only on small graphs
+// (chained): it hides launch latency (100K nodes, 1M edges: 0.38 against 0.49
+// ms a refinement of four rounds), but blocks that already hold their place,
+// and their shared memory, slow the kernel before.  Whether that costs more is
+// decided by the nodes, whose grouping and numbering these kernels do: at 4
+// edges a node 1.58 against 1.72 ms with 1.5M nodes but 2.75 against 2.65 with
+// 3M and 12.0 against 7.2 with 8.3M; at 8 edges a node 0.91 against 0.96 with
+// 1.5M, 1.48 against 1.41 with 2.5M, 2.87 against 2.49 with 4.1M; at 16 edges
+// 0.94 against 0.96 with 1.5M, 1.27 against 1.20 with 2.1M.  With few nodes and
+// many edges the two are equal from about 32M edges on (1M nodes: 1.11 against
+// 1.12 ms).
+constexpr uint64_t kChainNodes = 3ull << 19, kChainEdges = 32ull << 20;
+inline bool chained(const Store& s) { return s.n <= kChainNodes && s.m <= kChainEdges; }
 __device__ __forceinline__ void overlap_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void overlap_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -179,7 +186,7 @@ void launch_if_overlapped(bool on, Store& s, void (*kernel)(P...), unsigned bloc
 
 template <typename... P, typename... A>
 void launch_chained(Store& s, void (*kernel)(P...), unsigned blocks, int threads, size_t smem, A&&... args) {
-  launch_if_overlapped(s.m <= kChainEdges, s, kernel, blocks, threads, smem, args...);
+  launch_if_overlapped(chained(s), s, kernel, blocks, threads, smem, args...);
 }
 
 // --------------------------------------------------------------------------
@@ -3109,7 +3116,7 @@ Status launch_hubs(Store& s, const SigArgs& a, bool cleared) {
   h.cursor = ptr<uint32_t>(s.hub_cursor);
   h.hub_cur = ptr<unsigned long long>(s.hub_acc);
   h.hub_term = reinterpret_cast<uint32_t*>(h.hub_cur + s.n_hub);
-  const bool small = s.m <= kChainEdges;
+  const bool small = chained(s);
   h.done = small ? reinterpret_cast<uint32_t*>(h.hub_cur + 2 * s.n_hub) : nullptr;
   h.tmp = s.hub_tmp.p;
   h.mode = ptr<uint8_t>(s.hub_mode);

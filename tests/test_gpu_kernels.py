@@ -318,3 +318,21 @@ def test_one_set_for_the_nodes_of_a_warp(wide):
             for r in (1, 2, 3):
                 got = [kb.round_stats(r)[f] for f in ("unique_keys", "max_signature")]
                 assert got == [int(sets[r - 1].sum()), int(sets[r - 1].max())]
+
+
+@pytest.mark.parametrize("nodes,chained", [(3 << 19, True), ((3 << 19) + 1, False)])
+def test_launches_chain_up_to_a_number_of_nodes(nodes, chained):
+    """Above 3 * 2^19 nodes the kernels of a round do not overlap (chained they made graphs of some millions of nodes
+    slower than one launch after the other); the hub chunks' two kernels are then launched apart."""
+    rng = np.random.default_rng(43)
+    hub, m = 60_000, 5_000_000
+    src = np.concatenate([np.zeros(hub, np.uint32), rng.integers(1, nodes, m).astype(np.uint32)])
+    dst = rng.integers(0, nodes, src.size).astype(np.uint32)
+    g = synth.from_coo(nodes, src, dst, rng.integers(0, 4, src.size).astype(np.uint32),
+                       (np.arange(nodes) % 6).astype(np.uint32))
+    with KBisim(hub_bucket_keys=4096) as kb:
+        kb.build(g, 2)  # (the hub's buckets have their size)
+        kb.reset_times()
+        res = kb.refine(2)
+        assert kb.kernel_times()["sig_hub"][1] == res.rounds_run * (3 if chained else 5)
+        assert_same(res, kb.all_pids(2), oracle_levels(g, 2))
