@@ -1719,7 +1719,15 @@ __device__ __forceinline__ void mark_member(const VerifyArgs& v, uint32_t r) {
 // of the 16M-node powerlaw graph's four rounds: 1.95 -> 1.55 ms; 25.6M nodes of
 // the alpha = 2.0 one, five rounds: 5.2 -> 4.7 ms.  Up to 4M nodes the table
 // is as cheap (64 MB) and the two passes only cost.
+// They also only cost in round 1 where most nodes share their hash: level 0 has
+// few blocks, so a signature of no element or one repeats unless (label, block)
+// takes many values (kFilterValues), and where more than a node in 20 has such
+// a signature, the others are short too.  Refinement to level 1 with the filter
+// against without: 10M nodes of which 55% have two out-edges or more 1,454
+// against 1,254 us, 86% 1,710 and 1,622, 98% 1,837 and 1,900, 100% 1,475 to
+// 1,962 against 1,497 to 2,054; 10M with 5,000 edge labels 1,494 against 1,696.
 constexpr uint64_t kFilterNodes = 4u << 20;  // table above 64 MB
+constexpr uint64_t kFilterValues = 1u << 14;
 constexpr int kFilThreads = 256, kFilItems = 4, kFilTile = kFilThreads * kFilItems;
 
 __device__ __forceinline__ uint64_t filter_bit(const GroupArgs& g, uint64_t h) { return (mix64(h) >> 32) & g.seen_mask; }
@@ -2881,21 +2889,28 @@ VerifyArgs verify_args(Store& s, int mode, const uint32_t* prev, bool key64) {
 
 // Bits of the filter before the grouping of `ins` nodes (0 = none): 8 to 16 per
 // node, two bitmaps, so at most 4 of the 8 bytes per node of the pair lists,
-// which nothing uses before the comparison.
-uint64_t filter_bits(uint64_t ins) { return ins > kFilterNodes ? 4 * table_slots(ins) : 0; }
+// which nothing uses before the comparison.  `first`: the grouping of round 1.
+uint64_t filter_bits(const Store& s, uint64_t ins, bool first) {
+  if (ins <= kFilterNodes) return 0;
+  if (first) {
+    const bool many_values = s.counts[0] << s.label_bits >= kFilterValues;
+    if (s.class_start[many_values ? 1 : 2] > s.n_alive / 20) return 0;  // nodes of out-degree 0, or 0 and 1
+  }
+  return 4 * table_slots(ins);
+}
 
 // Clear what a level's signatures and grouping start from: error flags,
 // scalars, the marks of the canonical numbering, the hash table for `ins`
-// inserted nodes or the filter before it, and, with hubs, their buckets'
-// cursors and totals.
+// inserted nodes or the filter of `bits` before it (0 = none), and, with hubs,
+// their buckets' cursors and totals.
 // `keep`: the head marks of the level before stay.
-Status clear_round(Store& s, uint64_t ins, bool filter, bool hubs, bool keep) {
+Status clear_round(Store& s, uint64_t ins, uint64_t bits, bool hubs, bool keep) {
   ClearArgs c;
   c.add(s.d_err.p, 16, 0u);
   c.add(s.d_scalars.p, 16 * 8, 0u);
   if (!keep) c.add(s.hbits.p, (s.n + 31) / 32 * 4, 0u);
   c.add(s.member.p, s.n, 0u);
-  if (filter && filter_bits(ins)) c.add(s.long_pairs.p, filter_bits(ins) / 4, 0u);
+  if (bits) c.add(s.long_pairs.p, bits / 4, 0u);
   else c.add(s.table.p, group_slots(s, ins) * 8, ~0u);
   if (hubs) {
     c.add(s.hub_cursor.p, s.n_hub_buckets * 4, 0u);
@@ -2977,7 +2992,7 @@ Status group_and_rank(Store& s, int mode, const uint32_t* prev, bool key64, uint
                       kFillThreads, 0, r);
     return launch_check("renumber");
   };
-  const uint64_t bits = mode ? filter_bits(insert_count(s, use_alone)) : 0;
+  const uint64_t bits = mode ? filter_bits(s, insert_count(s, use_alone), first) : 0;
   if (na) {
     const uint32_t* list = nullptr;
     {
@@ -3809,7 +3824,7 @@ Status compute_level0(Store& s) {
   if (done) return Status::Ok();
   const int sms = sm_count(s.device);
   const unsigned blocks = (unsigned)std::min<uint64_t>(grid_for(s.n_alive, 256), (uint64_t)sms * 16);
-  if (!(st = clear_round(s, s.n_alive, false, false, false)).ok()) return st;
+  if (!(st = clear_round(s, s.n_alive, 0, false, false)).ok()) return st;
   {
     TimedScope ts(s, KBISIM_KERNEL_LABEL_GROUP, s.n_alive ? 1 : 0);
     if (s.n_alive)
@@ -3864,7 +3879,8 @@ Status compute_round(Store& s, uint32_t i) {
   if (!st.ok()) return st;
   bool keep = s.heads_level == (int64_t)i - 1;
   s.heads_level = -1;
-  if (!(st = clear_round(s, insert_count(s, true), true, s.n_hub != 0, keep)).ok()) return st;
+  const uint64_t ins = insert_count(s, true), filter = filter_bits(s, ins, i <= 1);
+  if (!(st = clear_round(s, ins, filter, s.n_hub != 0, keep)).ok()) return st;
   if (s.checked && !(st = check_round_inputs(s, i)).ok()) return st;
   SigArgs a;
   a.off = ptr<uint64_t>(s.offsets);
@@ -3924,7 +3940,7 @@ Status compute_round(Store& s, uint32_t i) {
     if (attempt >= kHubAttempts) return Status::Err(KBISIM_ERR_TIMEOUT, "hub bucket overflow persists");
     if (!(st = grow_hubs(s, &a)).ok()) return st;
     keep = false;  // heads were marked with incomplete signatures
-    if (!(st = clear_round(s, insert_count(s, true), true, true, false)).ok()) return st;
+    if (!(st = clear_round(s, ins, filter, true, false)).ok()) return st;
     if (!(st = typed(hubs_again)).ok()) return st;
   }
   s.heads_level = i;

@@ -336,3 +336,26 @@ def test_launches_chain_up_to_a_number_of_nodes(nodes, chained):
         res = kb.refine(2)
         assert kb.kernel_times()["sig_hub"][1] == res.rounds_run * (3 if chained else 5)
         assert_same(res, kb.all_pids(2), oracle_levels(g, 2))
+
+
+@pytest.mark.parametrize("hash_bits", [64, 22])
+@pytest.mark.parametrize("degree", [2, 13])
+def test_rounds_that_take_the_filter(degree, hash_bits):
+    """Above 4M nodes to group, the filter runs in round 1 where nearly all nodes have two out-edges or more (not with
+    a tenth of leaves) and in later rounds always: blocks of one, of two, of hundreds and of 100,000s."""
+    n, leaves, k = 4_700_000, 500_000 if degree == 2 else 0, 2 if degree == 2 else 1
+    rng = np.random.default_rng(47)
+    dst = rng.integers(0, n, (n - leaves, degree), dtype=np.uint32)
+    dst[1:400_000:2] = dst[0:400_000:2, ::-1]  # pairs of equal sets
+    off = np.concatenate([np.zeros(leaves, np.uint64), np.arange(n - leaves + 1, dtype=np.uint64) * degree])
+    label = (np.arange(n) // 2 * 2 % 16 if degree == 2 else np.arange(n) // 2 % 5).astype(np.uint32)
+    g = synth.Graph(n, off, dst.reshape(-1), (dst.reshape(-1) % 3).astype(np.uint8), label)
+    ref = oracle_levels(g, k)
+    alone = np.bincount(ref.pids[k - 1])
+    assert n - int((alone == 1).sum()) > 4 << 20 and 100_000 < int(ref.counts[k]) < n
+    with KBisim(hash_bits=hash_bits) as kb:
+        kb.reset_times()
+        res = kb.build(g, k)
+        assert_same(res, kb.all_pids(k), ref)
+        # launches of a grouping (level 0 has its own): 1 without and 4 with the filter
+        assert kb.kernel_times()["group"][1] == (1 + 4 if degree == 2 else 4)
