@@ -223,9 +223,12 @@ int kbisim_load(kbisim_handle *h, const kbisim_graph *g);
 /* Compute levels 0..k of the loaded graph (Algorithm 1, Build_Bisim).
  * Refining a graph of 8M edges or more again, in a handle without an HBM
  * budget and not in checked mode, first marks the edges that repeat an earlier
- * (label, target) of their source: one pass over the edges, once per edge
- * table, and one bit per edge and per node of device memory, which make that
- * and later refinements of the same edges faster.
+ * (label, target) of their source, those of sources of out-degree above 4096
+ * one refinement later: about one pass over the edges in all, once per edge
+ * table, and one bit per edge and per node of device memory, which make these
+ * and later refinements of the same edges faster.  It does so when at least
+ * two rounds (three above 32M edges) are to be expected: k, or with early stop
+ * those that made the result at hand stable.
  * Errors: STATE (no graph), INVALID_ARG (k > KBISIM_MAX_K or out == NULL),
  * OUT_OF_MEMORY, BUDGET, TIMEOUT, CHECKED, CUDA. */
 int kbisim_refine(kbisim_handle *h, uint32_t k, kbisim_result *out);

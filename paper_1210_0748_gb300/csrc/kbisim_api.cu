@@ -677,6 +677,8 @@ Status refine(Store& s, uint32_t k, kbisim_result* out) {
   drop_marks_under_budget(s);
   InUse use(s, kCacheSpare);
   LevelSnapshot snap = take_snapshot(s);
+  // the rounds to expect: with early stop, not more than made the result at hand stable
+  const uint32_t rounds = s.has_levels && s.stable && s.early_stop ? std::min(k, s.rounds_run) : k;
   std::swap(s.level, s.spare_level);
   std::swap(s.alone, s.spare_alone);
   s.has_levels = false;
@@ -686,9 +688,9 @@ Status refine(Store& s, uint32_t k, kbisim_result* out) {
   s.heads_level = -1;
   s.stats.clear();
   s.counts.assign(std::max<size_t>(snap.counts.size(), 1), 0);
-  // the second refinement of an edge table marks its duplicate edges for this
-  // and later ones
-  Status st = s.refined && !s.dup_valid && k >= 2 ? mark_duplicates(s) : Status::Ok();
+  // refining an edge table again marks its duplicate edges for this and later
+  // refinements
+  Status st = s.refined ? mark_duplicates(s, rounds) : Status::Ok();
   if (st.ok()) st = refine_levels(s, k);
   if (!st.ok()) {
     std::swap(s.level, s.spare_level);

@@ -397,8 +397,9 @@ Status relabel_graph(Store& s, const uint64_t* off0, const uint32_t* dst0, const
 Status apply_batch(Store& s, const kbisim_batch* b, uint64_t* missing);
 Status compute_level0(Store& s);                  // pId_0 into level[0]
 // Mark the edges that repeat an earlier (label, target) of their node, for the
-// rounds of this edge table (once per table, when it is refined again).
-Status mark_duplicates(Store& s);
+// rounds of this edge table (when it is refined again, the hubs' one refinement
+// later), unless the rounds expected of the refinement don't repay it.
+Status mark_duplicates(Store& s, uint32_t rounds);
 // Work lists of the degree classes from s.offsets (after a relabel, or after
 // a batch applied in place); `fresh` drops what hub buckets learned.
 Status build_chunk_lists(Store& s, bool fresh);

@@ -3207,12 +3207,15 @@ Status grow_hubs(Store& s, SigArgs* a) {
 
 constexpr int kHubAttempts = 40;
 constexpr uint64_t kHubCalmNodes = 4u << 20;
-// Edges from which a graph's duplicates are marked: refining the 16M-edge
-// powerlaw graph again takes 1.21 against 1.30 ms, the uniform one 1.50 against
-// 1.54, 256M edges 8.51 against 9.58; below, a round is latency and the extra
-// words only cost.  Marking takes about one pass over the signatures, so a
-// graph refined once is not marked.
-constexpr uint64_t kMarkEdges = 8u << 20;
+// Edges from which a graph's duplicates are marked: below, a round is latency
+// and the extra words only cost.  The rounds from level 2 on use the marks
+// (256M-edge powerlaw graph, five rounds 9.70 against 11.08 ms, three 6.89
+// against 7.30, two 5.47 against 5.40; 16M edges, three rounds 0.64 against
+// 0.71, two 0.51 against 0.53).  Marking takes about one pass over the edges, so
+// a graph refined once is not marked, nor one of more than kMarkEdgesTwoRounds
+// edges whose refinement ends after two rounds; and the hubs, the larger half of
+// the work (1.4 of 2.4 ms at 256M edges), are marked one refinement later.
+constexpr uint64_t kMarkEdges = 8u << 20, kMarkEdgesTwoRounds = 32ull << 20;
 
 // Hub passes until no bucket overflows, the host waiting for each.
 template <typename LabelT, typename K>
@@ -3308,16 +3311,7 @@ Status run_signatures(Store& s, const SigArgs& a, bool defer) {
           s.class_start[kClassBlock]);
   }
   if (!(st = launch_check("k_sig_warp")).ok()) return st;
-  if (s.n_hub && a.mark) {
-    if (!a.dup_hubs) return Status::Ok();
-    TimedScope ts(s, KBISIM_KERNEL_OTHER, 1);
-    const uint64_t first = s.class_start[kClassHub];
-    cudaMemsetAsync(s.hub_err.p, 0, s.n_hub * 4, s.stream);
-    k_mark_hubs<LabelT><<<(unsigned)s.n_hub_chunks, kChunkThreads, 0, s.stream>>>(a, first, ptr<uint4>(s.hub_chunks),
-                                                                                  ptr<uint32_t>(s.hub_err));
-    return launch_check("k_mark_hubs");
-  }
-  if (s.n_hub) {
+  if (s.n_hub && !a.mark) {
     if (!s.tune_now) return defer ? launch_hubs<LabelT, K>(s, a, true) : run_hubs<LabelT, K>(s, a);
     // tuning (once per handle, on a full round from level 2 on): each bucket
     // size runs the hub pass twice, the sizes alternating, each pass timed
@@ -3957,18 +3951,29 @@ Status compute_round(Store& s, uint32_t i) {
   return Status::Ok();
 }
 
-Status mark_duplicates(Store& s) {
-  s.dup_valid = false;
+// The edges of hubs into the marks: their set in the key buffer has 32-bit slots.
+template <typename LabelT>
+Status mark_hub_edges(Store& s, const SigArgs& a) {
+  cudaMemsetAsync(static_cast<char*>(s.sigkey.p) + s.hub_edge0 * 8, 0xFF, s.hub_edges * 8, s.stream);
+  cudaMemsetAsync(s.hub_err.p, 0, s.n_hub * 4, s.stream);
+  k_mark_hubs<LabelT><<<(unsigned)s.n_hub_chunks, kChunkThreads, 0, s.stream>>>(
+      a, s.class_start[kClassHub], ptr<uint4>(s.hub_chunks), ptr<uint32_t>(s.hub_err));
+  return launch_check("k_mark_hubs");
+}
+
+Status mark_duplicates(Store& s, uint32_t rounds) {
   if (!s.n || s.m < kMarkEdges || s.budget || s.checked || s.fault_alloc >= 0) return Status::Ok();
+  if (rounds < (s.m > kMarkEdgesTwoRounds ? 3u : 2u)) return Status::Ok();
+  const uint32_t pbits = bits_for(s.n - 1);
+  const bool key64 = pbits + s.label_bits > 32, hubs = s.dup_valid;  // (the hubs' turn)
+  if (hubs && (s.dup_hubs || !s.n_hub || key64)) return Status::Ok();
   Status st = ensure_round_scratch(s);
   if (!st.ok()) return st;
   const uint64_t words = s.m / 32 + 1;
-  if (!ensure(s, s.dup, words * 4 + 16).ok() || !ensure(s, s.alone_bits, s.n / 32 * 4 + 16).ok()) {
+  if (!hubs && (!ensure(s, s.dup, words * 4 + 16).ok() || !ensure(s, s.alone_bits, s.n / 32 * 4 + 16).ok())) {
     release(s, s.dup);
     return Status::Ok();  // no room: every round runs without the marks
   }
-  const uint32_t pbits = bits_for(s.n - 1);
-  const bool key64 = pbits + s.label_bits > 32;
   SigArgs a = {};
   a.off = ptr<uint64_t>(s.offsets);
   a.dst = ptr<uint32_t>(s.dst);
@@ -3981,21 +3986,23 @@ Status mark_duplicates(Store& s) {
   a.pbits = (int)pbits;
   a.err = ptr<uint32_t>(s.d_err);
   a.mark = ptr<uint32_t>(s.dup);
-  a.dup_hubs = !key64;  // (a hub's set has 32-bit slots)
   TimedScope ts(s, KBISIM_KERNEL_OTHER, 1);
-  cudaMemsetAsync(s.dup.p, 0, words * 4, s.stream);
-  cudaMemsetAsync(s.member.p, 1, s.n, s.stream);
-  if (s.n_hub && a.dup_hubs)
-    cudaMemsetAsync(static_cast<char*>(s.sigkey.p) + s.hub_edge0 * 8, 0xFF, s.hub_edges * 8, s.stream);
   k_iota<<<(unsigned)std::min<uint64_t>(grid_for(s.n, 256), (uint64_t)sm_count(s.device) * 16), 256, 0, s.stream>>>(
       s.n, ptr<uint32_t>(s.slot));
   if (!(st = launch_check("mark duplicates")).ok()) return st;
-  if (s.label8)
-    st = key64 ? run_signatures<uint8_t, uint64_t>(s, a, false) : run_signatures<uint8_t, uint32_t>(s, a, false);
-  else
-    st = key64 ? run_signatures<uint32_t, uint64_t>(s, a, false) : run_signatures<uint32_t, uint32_t>(s, a, false);
+  s.dup_valid = false;  // (until the marks are whole)
+  if (hubs) {
+    st = s.label8 ? mark_hub_edges<uint8_t>(s, a) : mark_hub_edges<uint32_t>(s, a);
+  } else {
+    cudaMemsetAsync(s.dup.p, 0, words * 4, s.stream);
+    cudaMemsetAsync(s.member.p, 1, s.n, s.stream);
+    if (s.label8)
+      st = key64 ? run_signatures<uint8_t, uint64_t>(s, a, false) : run_signatures<uint8_t, uint32_t>(s, a, false);
+    else
+      st = key64 ? run_signatures<uint32_t, uint64_t>(s, a, false) : run_signatures<uint32_t, uint32_t>(s, a, false);
+  }
   if (!st.ok()) return st;
-  s.dup_hubs = a.dup_hubs;
+  s.dup_hubs = hubs;
   s.dup_valid = true;
   return Status::Ok();
 }

@@ -359,3 +359,52 @@ def test_rounds_that_take_the_filter(degree, hash_bits):
         assert_same(res, kb.all_pids(k), ref)
         # launches of a grouping (level 0 has its own): 1 without and 4 with the filter
         assert kb.kernel_times()["group"][1] == (1 + 4 if degree == 2 else 4)
+
+
+def _regular(n, deg, node_label, hub=0, seed=53):
+    """n nodes of out-degree deg, the first of out-degree deg + hub."""
+    rng = np.random.default_rng(seed)
+    off = np.concatenate([[0], np.arange(1, n + 1) * deg + hub]).astype(np.uint64)
+    dst = rng.integers(0, n, n * deg + hub, dtype=np.uint32)
+    return synth.Graph(n, off, dst, (dst % 3).astype(np.uint8), node_label.astype(np.uint32))
+
+
+@pytest.mark.parametrize("stable", [False, True])
+def test_marks_wait_for_a_refinement_that_repays_them(stable):
+    """Duplicate edges are marked when a table is refined again, but not by a refinement of two rounds above 32M edges
+    nor by one of a graph that was stable after one round: their calls would only get slower."""
+    n, deg = (210_000, 41) if stable else (820_000, 41)
+    g = _regular(n, deg, np.arange(n) if stable else np.arange(n) % 4)
+    assert g.num_edges > (8 << 20 if stable else 32 << 20)
+    ks = (10, 10, 10) if stable else (2, 2, 2, 3)
+
+    def run(budget):
+        with KBisim(early_stop=stable) as kb:
+            kb.load(g)
+            kb.set_hbm_budget(budget)
+            held = []
+            for k in ks:
+                res = kb.refine(k)
+                held.append(kb.device_bytes)
+            assert not stable or res.rounds_run == 1
+            return held, res.counts, kb.all_pids(min(ks[-1], 3))
+
+    free, bound = run(0), run(1 << 40)  # under a budget nothing is marked
+    marks = [a - b for a, b in zip(free[0], bound[0])]
+    assert marks[:3] == marks[:1] * 3
+    assert stable or marks[3] >= marks[0] + g.num_edges // 8
+    assert free[1] == bound[1] and np.array_equal(free[2], bound[2])
+
+
+def test_hubs_are_marked_one_refinement_later():
+    n, deg = 210_000, 41
+    g = _regular(n, deg, np.arange(n) % 4, hub=70_000)
+    with KBisim(early_stop=False, hub_bucket_keys=4096) as kb:
+        kb.build(g, 3)
+        first, launches = kb.all_pids(3), []
+        for _ in range(4):
+            kb.reset_times()
+            kb.refine(3)
+            launches.append(kb.kernel_times()["other"][1])
+            assert np.array_equal(kb.all_pids(3), first)
+    assert launches[0] > launches[2] == launches[3] and launches[1] > launches[2]
