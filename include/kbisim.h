@@ -192,7 +192,7 @@ enum {
   KBISIM_KERNEL_GROUP,           /* hash-table grouping of equal signatures */
   KBISIM_KERNEL_VERIFY,          /* exact signature comparison, marking block heads */
   KBISIM_KERNEL_RENUMBER,        /* canonical renumbering (scan of head counts + ranks) */
-  KBISIM_KERNEL_OTHER,           /* clears, collision repair, copies */
+  KBISIM_KERNEL_OTHER,           /* clears, marks of duplicate edges, collision repair, copies */
   KBISIM_KERNEL_COUNT
 };
 

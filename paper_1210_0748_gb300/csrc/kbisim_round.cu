@@ -3257,7 +3257,7 @@ Status run_signatures(Store& s, const SigArgs& a, bool defer) {
     return L;
   };
   const SmallLaunch L04 = small_launch(0, 4), L5 = small_launch(5, 5);
-  const uint32_t n04 = L04.bstart[5], n5 = L5.bstart[6] - L5.bstart[5];
+  const uint32_t n04 = a.mark ? 0 : L04.bstart[5], n5 = a.mark ? 0 : L5.bstart[6] - L5.bstart[5];
   // the first kernel starts when all earlier work has ended, clear_round's
   // launch (which starts then and writes nothing these kernels read) excepted
   bool overlapped = defer;
@@ -3274,9 +3274,10 @@ Status run_signatures(Store& s, const SigArgs& a, bool defer) {
   {
     const uint64_t n32 = s.class_start[kSmallClasses - 1] - s.class_start[kSmallClasses - 2];
     const uint64_t n64 = s.class_start[kClassWarp] - s.class_start[kSmallClasses - 1];
-    TimedScope ts(s, KBISIM_KERNEL_SIG_SMALL, (n04 ? 1 : 0) + (n5 ? 1 : 0) + (n32 ? 1 : 0) + (n64 ? 1 : 0));
-    if (n04 && !a.mark) run(k_sig_small<0, 4, LabelT, K>, n04, kSmallThreads, 0, a, L04);
-    if (n5 && !a.mark) run(k_sig_small<5, 5, LabelT, K>, n5, kSmallThreads, 0, a, L5);
+    TimedScope ts(s, a.mark ? KBISIM_KERNEL_OTHER : KBISIM_KERNEL_SIG_SMALL,
+                  (n04 ? 1 : 0) + (n5 ? 1 : 0) + (n32 ? 1 : 0) + (n64 ? 1 : 0));
+    if (n04) run(k_sig_small<0, 4, LabelT, K>, n04, kSmallThreads, 0, a, L04);
+    if (n5) run(k_sig_small<5, 5, LabelT, K>, n5, kSmallThreads, 0, a, L5);
     if (n32)
       warp_nodes(a.mark  ? k_sig_warp<1, kMarking, LabelT, K>
                  : a.dup ? k_sig_warp<1, kWithDup, LabelT, K>
@@ -3293,7 +3294,8 @@ Status run_signatures(Store& s, const SigArgs& a, bool defer) {
   const uint64_t n1k = s.class_start[kClassBlock] - s.class_start[kClassWarp2];
   const uint64_t n4k = s.class_start[kClassHub] - s.class_start[kClassBlock];
   if (n256 + n1k + n4k) {
-    TimedScope ts(s, KBISIM_KERNEL_SIG_MEDIUM, (n256 ? 1 : 0) + (n1k ? 1 : 0) + (n4k ? 1 : 0));
+    TimedScope ts(s, a.mark ? KBISIM_KERNEL_OTHER : KBISIM_KERNEL_SIG_MEDIUM,
+                  (n256 ? 1 : 0) + (n1k ? 1 : 0) + (n4k ? 1 : 0));
     if (n256)
       warp_nodes(a.mark  ? k_sig_warp<8, kMarking, LabelT, K>
                  : a.dup ? k_sig_warp<8, kWithDup, LabelT, K>
@@ -3954,6 +3956,7 @@ Status compute_round(Store& s, uint32_t i) {
 // The edges of hubs into the marks: their set in the key buffer has 32-bit slots.
 template <typename LabelT>
 Status mark_hub_edges(Store& s, const SigArgs& a) {
+  TimedScope ts(s, KBISIM_KERNEL_OTHER, 1);
   cudaMemsetAsync(static_cast<char*>(s.sigkey.p) + s.hub_edge0 * 8, 0xFF, s.hub_edges * 8, s.stream);
   cudaMemsetAsync(s.hub_err.p, 0, s.n_hub * 4, s.stream);
   k_mark_hubs<LabelT><<<(unsigned)s.n_hub_chunks, kChunkThreads, 0, s.stream>>>(
@@ -3986,9 +3989,11 @@ Status mark_duplicates(Store& s, uint32_t rounds) {
   a.pbits = (int)pbits;
   a.err = ptr<uint32_t>(s.d_err);
   a.mark = ptr<uint32_t>(s.dup);
-  TimedScope ts(s, KBISIM_KERNEL_OTHER, 1);
-  k_iota<<<(unsigned)std::min<uint64_t>(grid_for(s.n, 256), (uint64_t)sm_count(s.device) * 16), 256, 0, s.stream>>>(
-      s.n, ptr<uint32_t>(s.slot));
+  {
+    TimedScope ts(s, KBISIM_KERNEL_OTHER, 1);
+    k_iota<<<(unsigned)std::min<uint64_t>(grid_for(s.n, 256), (uint64_t)sm_count(s.device) * 16), 256, 0, s.stream>>>(
+        s.n, ptr<uint32_t>(s.slot));
+  }
   if (!(st = launch_check("mark duplicates")).ok()) return st;
   s.dup_valid = false;  // (until the marks are whole)
   if (hubs) {

@@ -408,3 +408,20 @@ def test_hubs_are_marked_one_refinement_later():
             launches.append(kb.kernel_times()["other"][1])
             assert np.array_equal(kb.all_pids(3), first)
     assert launches[0] > launches[2] == launches[3] and launches[1] > launches[2]
+
+
+def test_marking_is_timed_once_and_not_as_signatures():
+    """The launches that make the marks count as "other": a refinement's signature classes show its rounds alone."""
+    n, deg = 210_000, 41
+    g = _regular(n, deg, np.arange(n) % 4, hub=70_000)
+    with KBisim(early_stop=False, hub_bucket_keys=4096, collect_timing=True) as kb:
+        kb.build(g, 3)
+        seen = []
+        for _ in range(3):
+            kb.reset_times()
+            kb.refine(3)
+            seen.append(kb.kernel_times())
+        for cls in ("sig_small", "sig_medium", "sig_hub"):
+            assert len({t[cls][1] for t in seen}) == 1, cls
+        # identifiers and the one class of the graph; identifiers and the hub
+        assert [t["other"][1] - seen[2]["other"][1] for t in seen] == [2, 2, 0]
