@@ -3965,7 +3965,7 @@ Status mark_hub_edges(Store& s, const SigArgs& a) {
 }
 
 Status mark_duplicates(Store& s, uint32_t rounds) {
-  if (!s.n || s.m < kMarkEdges || s.budget || s.checked || s.fault_alloc >= 0) return Status::Ok();
+  if (!s.n || s.m < kMarkEdges || s.budget || s.checked) return Status::Ok();
   if (rounds < (s.m > kMarkEdgesTwoRounds ? 3u : 2u)) return Status::Ok();
   const uint32_t pbits = bits_for(s.n - 1);
   const bool key64 = pbits + s.label_bits > 32, hubs = s.dup_valid;  // (the hubs' turn)

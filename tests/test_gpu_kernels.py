@@ -425,3 +425,24 @@ def test_marking_is_timed_once_and_not_as_signatures():
             assert len({t[cls][1] for t in seen}) == 1, cls
         # identifiers and the one class of the graph; identifiers and the hub
         assert [t["other"][1] - seen[2]["other"][1] for t in seen] == [2, 2, 0]
+
+
+def test_no_room_for_the_marks(monkeypatch):
+    """When the bit per edge (first allocation of the call) or the bit per node (second) of the duplicate marks cannot
+    be allocated, the refinement runs without them and keeps nothing of them; one that finds room makes them."""
+    n, deg = 210_000, 41
+    g = _regular(n, deg, np.arange(n) % 4)
+    with KBisim(early_stop=False) as kb:
+        kb.build(g, 2)
+        first = [kb.pids(j) for j in range(3)]
+        kb.refine(1)  # (makes the spare buffers, and no marks)
+        kb.extend(2)
+        kb.pids(2)
+        held = kb.device_bytes
+        for fails_after in ("0", "1", "2"):  # the third allocation is never asked for
+            monkeypatch.setenv("KBISIM_FAULT_ALLOC", fails_after)
+            kb.refine(2)
+            monkeypatch.delenv("KBISIM_FAULT_ALLOC")
+            grown = kb.device_bytes - held
+            assert grown >= g.num_edges // 8 if fails_after == "2" else grown == 0, (fails_after, grown)
+            assert all(np.array_equal(kb.pids(j), first[j]) for j in range(3))
