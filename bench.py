@@ -562,8 +562,10 @@ def main():
     traffic = traffic_round / d["launches_per_call"] if traffic_round is not None else None
     names = {"sig_small": "k_sig_small (out-degree <= 16, one thread per node) and k_sig_warp (17..64, a warp per node)",
              "sig_medium": "k_sig_warp (out-degree 65..256, a warp per node) and k_sig_cta (257..4096, a CTA per node)",
-             "sig_hub": "k_hub_sample, k_hub_chunk or k_hub_scatter per hub, k_hub_bucket, k_hub_finish (out-degree > 4096)",
-             "group": "k_group_insert", "verify": "k_group_verify", "renumber": "renumbering kernels"}
+             "sig_hub": "k_hub_sample, k_hub_chunk or k_hub_scatter per hub (small graphs: k_hub_pieces), k_hub_bucket, "
+                        "k_hub_finish (out-degree > 4096)",
+             "group": "k_group_filter, k_group_select and k_table_clear (large graphs), k_group_insert",
+             "verify": "k_group_verify, k_verify_long", "renumber": "k_head_ranks, k_pid_fill"}
     roofline = {"bound": "hbm", "kernel": names.get(dom, dom), "achieved": d["achieved"], "peak": peak,
                 "unit": "GB/s", "frac": d["frac"], "peak_kind": peak_kind, "traffic": traffic,
                 "traffic_per_round": traffic_round, "algorithmic_bytes_per_round": d["algorithmic_bytes_per_call"],

@@ -32,12 +32,12 @@ CSRC = os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_1210_0748
 # kernel name -> class of the library's timing (kbisim_kernel_times)
 CLASS_OF = [
     (r"k_label_hash|k_l0_collect|k_l0_rank", "label_group"),
-    (r"k_sig_small|k_sig_warp<[12],|k_sig_chunk<128, 33,", "sig_small"),  # the library times out-degree 33..64 with <= 32
-    (r"k_sig_warp|k_sig_cta|k_sig_chunk", "sig_medium"),
-    (r"k_hub_sample|k_hub_chunk|k_hub_scatter|k_hub_bucket|k_hub_finish", "sig_hub"),
+    (r"k_sig_small|k_sig_warp<[12],", "sig_small"),  # <1, and <2,: out-degree 17..32 and 33..64
+    (r"k_sig_warp|k_sig_cta", "sig_medium"),
+    (r"k_hub_sample|k_hub_pieces|k_hub_chunk|k_hub_scatter|k_hub_bucket|k_hub_finish", "sig_hub"),
     (r"k_group_insert|k_group_filter|k_group_select|k_table_clear", "group"),
     (r"k_group_verify|k_verify_long", "verify"),
-    (r"k_head_ranks|k_word_counts|k_tile_sum64|k_scan_tiles|k_tile_scan64|k_pid_fill|k_l0_fill", "renumber"),
+    (r"k_head_ranks|k_pid_fill|k_l0_fill", "renumber"),
 ]
 
 UNITS = {"ns": 1e-9, "nsecond": 1e-9, "us": 1e-6, "usecond": 1e-6, "ms": 1e-3, "msecond": 1e-3,

@@ -112,3 +112,19 @@ def test_traffic_record_units(tmp_path, monkeypatch):
     # every edge and node is in exactly one signature class
     assert sum(r["class_units"][c]["edges"] for c in ("sig_small", "sig_medium", "sig_hub")) == g.num_edges
     assert sum(r["class_units"][c]["nodes"] for c in ("sig_small", "sig_medium", "sig_hub")) == g.num_nodes
+
+
+def test_classes_name_the_kernels_that_exist():
+    """Every pattern names kernels of the sources, and every kernel that a round's timing classes run has its class."""
+    import os
+    import re
+    src = "".join(open(os.path.join(ncu_summary.CSRC, f)).read() for f in ncu_summary.ROUND_SOURCES)
+    kernels = set(re.findall(r"__global__[^;{(]*?(?:__launch_bounds__\((?:[^()]|\([^()]*\))*\)\s*)?(k_\w+)\(", src))
+    assert {"k_hub_pieces", "k_sig_warp", "k_pid_fill", "k_group_select"} <= kernels
+    named = {n for pat, _ in ncu_summary.CLASS_OF for n in re.findall(r"k_\w+", pat)}
+    assert named <= kernels, named - kernels
+    rounds = {k for k in kernels if re.match(r"k_(sig|hub|group|verify|l0|table)_", k)}
+    assert rounds <= named, rounds - named
+    assert ncu_summary.class_of("k_hub_pieces<0, unsigned char, unsigned int>") == "sig_hub"
+    assert [ncu_summary.class_of("k_sig_warp<%d, 1, unsigned char, unsigned int>" % s) for s in (1, 2, 8)] == [
+        "sig_small", "sig_small", "sig_medium"]
