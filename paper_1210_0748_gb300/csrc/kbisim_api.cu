@@ -2,8 +2,6 @@
 // (CSR build on the device), refinement, extension, copy-out.
 #include <cuda_runtime.h>
 #include <stdint.h>
-#include <sys/mman.h>
-#include <unistd.h>
 
 #include <algorithm>
 #include <chrono>
@@ -13,6 +11,7 @@
 #include <string>
 #include <vector>
 
+#include "host_pages.h"
 #include "kbisim_internal.cuh"
 
 struct kbisim_handle {
@@ -565,22 +564,6 @@ Status materialize_level(Store& s, uint32_t l) {
   if (!(st = unpermute_level(s, l, ptr<uint32_t>(s.out_level[l]))).ok()) return st;
   s.out_valid[l] = true;
   return Status::Ok();
-}
-
-// Have the kernel map the pages of a large host destination in one call, while
-// the device still prepares the copy.  An array just allocated (the usual
-// destination) has none, and the copy would fault them in one by one: 12.8 MB
-// take 455 us with the pages mapped first, 580 without, 80 once mapped.
-// Contents stay; where the call is not known or does not apply (pinned memory)
-// it fails and the copy does as before.
-void map_host_pages(void* dst, size_t bytes) {
-#ifndef MADV_POPULATE_WRITE
-#define MADV_POPULATE_WRITE 23
-#endif
-  if (bytes < (1u << 20)) return;
-  const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE), a = reinterpret_cast<uintptr_t>(dst);
-  const uintptr_t lo = (a + page - 1) / page * page, hi = (a + bytes) / page * page;
-  if (hi > lo) madvise(reinterpret_cast<void*>(lo), hi - lo, MADV_POPULATE_WRITE);
 }
 
 void fill_result(Store& s, uint32_t k, kbisim_result* out) {
