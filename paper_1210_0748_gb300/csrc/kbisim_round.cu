@@ -675,7 +675,7 @@ __device__ __forceinline__ int pow2_insert(uint32_t base, uint32_t hmask, K k) {
 // node, on two-node sums and on shared atomics; a step that belongs to one node
 // takes 95 to 145.  Out-degree 17..32 ran one thread per node with 32 keys in
 // registers, whose uncoalesced loads kept the L1 at 77%: 155 -> 145 us a round
-// for 18M edges, and 635 -> 567 us for a refinement of 1M edges.  
+// for 18M edges, and 625 -> 582 us for a refinement of 1M edges.
 constexpr int kNodeWarps = 8;  // per CTA
 
 // Distinct elements of a node that only counts, with its duplicates marked: the
@@ -1252,9 +1252,10 @@ __global__ void __launch_bounds__(kChunkThreads, sizeof(K) == 4 ? 4 : 3) k_hub_s
 }
 
 // Both kinds of chunk in one launch, for graphs whose rounds are launches and
-// latency more than work (up to kChainEdges): one launch less per round.  Its
-// shared memory is the chunk set's, which above that size would take the L1
-// from the scatter's gathers.
+// latency more than work (chained): one launch less per round (1M nodes, 8
+// edges a node, 767 -> 736 us a refinement of four rounds; equal from 2M nodes
+// on).  Its shared memory is the chunk set's, which on larger graphs would take
+// the L1 from the scatter's gathers.
 template <int MODE, typename LabelT, typename K>
 __global__ void __launch_bounds__(kChunkThreads, sizeof(K) == 4 ? 4 : 3) k_hub_pieces(SigArgs a, HubArgs h) {
   overlap_next();
