@@ -2,11 +2,11 @@
 (``python ncu_summary.py CSV ...``).
 
 The CSV comes from ``ncu --metrics gpu__time_duration.sum,dram__bytes_read.sum,
-dram__bytes_write.sum --csv`` over ``bench.py --steps 1 --warmup 2``: every
-launch of the graph load and of three refinements (level 0 and each round).
-Only the last refinement is summarised (from its level-0 kernel on):
-the warm-up refinements have already grown any hub bucket that overflows, as
-in the timed steps.  Two outputs:
+dram__bytes_write.sum --csv`` over ``bench.py --steps 1 --warmup 3``: every
+launch of the graph load and of four refinements (level 0 and each round).
+Only the last refinement is summarised (from its level-0 kernel on): the
+warm-up refinements have already grown any hub bucket that overflows and
+marked the duplicate edges, as in the timed steps.  Two outputs:
 
 * a Markdown table per kernel (launches, total time, share, DRAM bytes);
 * a JSON record of DRAM bytes per call of each kernel class (per round for the

@@ -455,8 +455,10 @@ __device__ __forceinline__ uint32_t edge_rest(const SigArgs& a, uint64_t base, u
 // and the warp stores the whole range coalesced (slots past a node's distinct
 // count keep leftovers that nothing reads).  A node alone in its block only
 // counts.  Lanes past the class end take part without a node.
-// Bound by the L1's data pipe (81% at out-degree <= 8: about 0.75 of 1.4
-// wavefronts per edge are the identifier gather).
+// Bound by the L1's data pipe (81% at out-degree <= 8 where every node writes
+// its keys: about 0.75 of 1.4 wavefronts per edge are the identifier gather; 67%
+// and 1.05 wavefronts in round 2 of the 64M-edge powerlaw graph, where most
+// nodes only count).
 template <int S, typename LabelT, typename K>
 __device__ __forceinline__ void sig_warp_staged(const SigArgs& a, uint64_t p_first, uint32_t nvalid, K* wsm,
                                                 const Policies& pol) {
@@ -669,13 +671,14 @@ __device__ __forceinline__ int pow2_insert(uint32_t base, uint32_t hmask, K k) {
 // insert was the first writes the key out behind those found before.  Count and
 // term sums stay in registers, and the hashes of the warp's nodes are made
 // together at the end, a lane per node.
-// Bound by instruction issue (62% at out-degree 33..64) and the L1 (60%).
+// Bound by instruction issue (57% at out-degree 17..64) and the L1 (47 to 61%).
 // Chunks of whole nodes in a CTA-wide set, where a step of 32 edges could meet
 // two nodes, spent most of their 239 warp instructions a step on finding the
 // node, on two-node sums and on shared atomics; a step that belongs to one node
-// takes 95 to 145.  Out-degree 17..32 ran one thread per node with 32 keys in
-// registers, whose uncoalesced loads kept the L1 at 77%: 155 -> 145 us a round
-// for 18M edges, and 625 -> 582 us for a refinement of 1M edges.
+// takes 130 (out-degree 65..256) to 187 (17..32), with marks 85 to 155.
+// Out-degree 17..32 ran one thread per node with 32 keys in registers, whose
+// uncoalesced loads kept the L1 at 77%: 155 -> 145 us a round for 18M edges, and
+// 625 -> 582 us for a refinement of 1M edges.
 constexpr int kNodeWarps = 8;  // per CTA
 
 // Distinct elements of a node that only counts, with its duplicates marked: the
